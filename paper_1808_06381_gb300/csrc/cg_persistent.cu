@@ -25,6 +25,7 @@
 #include <mutex>
 
 #include "internal.cuh"
+#include "pcg64.cuh"
 
 namespace ss {
 
@@ -1699,40 +1700,33 @@ __global__ void __launch_bounds__(BS, 1) k32_cg_resident(KParams P, DevBuffers B
 }
 
 // ------------------------------------------------------ FP64 persistent solve
-// The FP64 solve in one cooperative launch, every scalar decided by thread 0
+// The FP64 solve in one cooperative launch, every scalar decided by one thread
 // of every block from identical totals; the recurrence residual arms an FP64
 // true-residual check that accepts or restarts.
-// Large systems (TPR = 1): the FP64 solver's iteration as the two-kernel form
-// of cg.cu (Jacobi-PCG with the direction update fused into the SpMV: q = A z
-// + beta q, p = z + beta p; x += alpha p, r -= alpha q, z = D^-1 r), two grid
-// reductions per iteration (the barrier of the second one also publishes z
-// for the next SpMV); a block owns whole windows of 256 rows, one thread per
-// row, warps take the windows' chunks in zig-zag order (as the mixed
-// streaming solve).
-// Small systems (TPR = 4, fewer than two windows per SM): pipelined CG, one
-// grid reduction per iteration (below), where the barriers are a large share
-// of an iteration; a block owns a run of chunks of 32 rows and four
-// neighbouring lanes share a row, each summing every fourth of its entries,
-// so a row's gathers are in flight together; GB300 issues FP64 at ~2 FMA per
-// clock per SM, so a small system is also spread over as many SMs as it has
-// chunk pairs.  Gathered vectors go through plain (coherent) loads: other
-// blocks wrote them before the last barrier.
+// Large systems (k64_cg_persistent): the FP64 solver's iteration as the
+// two-kernel form of cg.cu (Jacobi-PCG with the direction update fused into
+// the SpMV: q = A z + beta q, p = z + beta p; x += alpha p, r -= alpha q, z =
+// D^-1 r), two grid reductions per iteration (the barrier of the second one
+// also publishes z for the next SpMV); a block owns whole windows of 256 rows,
+// one thread per row, warps take the windows' chunks in zig-zag order (as the
+// mixed streaming solve).  Gathered vectors go through plain (coherent)
+// loads: other blocks wrote them before the last barrier.
+// Small systems (k64_cg_pipelined, below): pipelined CG on chip.
 constexpr int kBatch64 = 6;
 
-// s_a = sum over the row's entries k = sub, sub + TPR, ... of w_k v_a[col_k]
-template <int TPR>
+// s_a = sum over the row's entries of w_k v_a[col_k]
 __device__ __forceinline__ void p_row_sum64(const int* __restrict__ col, const double* __restrict__ val,
-                                            const double* v, int np, int e0, int e1, int sub, bool active,
-                                            double& s0, double& s1, double& s2)
+                                            const double* v, int np, int e0, int e1, bool active, double& s0,
+                                            double& s1, double& s2)
 {
     s0 = s1 = s2 = 0.0;
     if (active) {
-        for (int eb = e0 + 32 * sub; eb < e1; eb += 32 * TPR * kBatch64) {
+        for (int eb = e0; eb < e1; eb += 32 * kBatch64) {
             int j[kBatch64];
             double w[kBatch64];
 #pragma unroll
             for (int u = 0; u < kBatch64; ++u) {
-                const int e = eb + 32 * TPR * u;
+                const int e = eb + 32 * u;
                 j[u] = 0;
                 w[u] = 0.0;
                 if (e < e1) {
@@ -1758,37 +1752,18 @@ __device__ __forceinline__ void p_row_sum64(const int* __restrict__ col, const d
             }
         }
     }
-#pragma unroll
-    for (int o = 1; o < TPR; o <<= 1) {   // the row's lanes are neighbours in the warp
-        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-    }
 }
 
-// The block's rows in slot order: calls f(slot, sub, active) the same number
-// of times in every thread of the block (the shuffles of p_row_sum64 need
-// whole warps).
-template <int TPR, class F>
+// The block's rows in slot order.
+template <class F>
 __device__ __forceinline__ void for_each_slot64(const KParams& P, int bid, int nb, F f)
 {
-    if (TPR == 1) {
-        const int nwin = P.nslots / 256;
-        const int wb = (int)((long long)bid * nwin / nb), we = (int)((long long)(bid + 1) * nwin / nb);
-        const int G = blockDim.x >> 8, t = threadIdx.x & 255;
-        for (int w = wb + (int)(threadIdx.x >> 8), k = 0; w < we; w += G, ++k) f(w * 256 + chunk_lane(k, t), 0, true);
-    } else {
-        const int s0 = 32 * (int)((long long)bid * P.nchunks / nb);
-        const int s1 = 32 * (int)((long long)(bid + 1) * P.nchunks / nb);
-        const int per = blockDim.x / TPR;
-        for (int base = s0; base < s1; base += per) {
-            const int slot = base + (int)threadIdx.x / TPR;
-            f(slot, (int)threadIdx.x % TPR, slot < s1);
-        }
-    }
+    const int nwin = P.nslots / 256;
+    const int wb = (int)((long long)bid * nwin / nb), we = (int)((long long)(bid + 1) * nwin / nb);
+    const int G = blockDim.x >> 8, t = threadIdx.x & 255;
+    for (int w = wb + (int)(threadIdx.x >> 8), k = 0; w < we; w += G, ++k) f(w * 256 + chunk_lane(k, t));
 }
 
-template <int TPR>
 __device__ __forceinline__ void persistent_solve64(const KParams& P, const DevBuffers& B, int bid, int nb,
                                                    PShared& sh, int from_x)
 {
@@ -1803,7 +1778,7 @@ __device__ __forceinline__ void persistent_solve64(const KParams& P, const DevBu
     double* z = B.z;
     double* p = B.p;
     double* q = B.q;
-    auto row_of = [&](int slot, bool active) { return active ? B.slot_row[slot] : -1; };
+    auto row_of = [&](int slot) { return B.slot_row[slot]; };
     auto ends = [&](int slot, int& e0, int& e1) {
         e0 = B.chunk_off[slot >> 5] + (slot & 31);
         e1 = B.chunk_off[(slot >> 5) + 1];
@@ -1812,13 +1787,13 @@ __device__ __forceinline__ void persistent_solve64(const KParams& P, const DevBu
     // r = b - A x0 (or b, x = 0); z = D^-1 r; p = q = 0; ||b||^2, r.r, r.z
     {
         double bb = 0.0, rr = 0.0, rz = 0.0;
-        for_each_slot64<TPR>(P, bid, nb, [&](int slot, int sub, bool active) {
-            const int row = row_of(slot, active);
+        for_each_slot64(P, bid, nb, [&](int slot) {
+            const int row = row_of(slot);
             int e0 = 0, e1 = 0;
             if (row >= 0) ends(slot, e0, e1);
             double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-            if (from_x) p_row_sum64<TPR>(B.col, B.val, x, np, e0, e1, sub, row >= 0, s0, s1, s2);
-            if (row < 0 || sub != 0) return;
+            if (from_x) p_row_sum64(B.col, B.val, x, np, e0, e1, row >= 0, s0, s1, s2);
+            if (row < 0) return;
             const double sv[3] = {s0, s1, s2};
             const double d = B.diag[row], di = B.dinv[row];
             double rs = 0.0;
@@ -1872,13 +1847,13 @@ __device__ __forceinline__ void persistent_solve64(const KParams& P, const DevBu
         // ---- q = A z + beta q; p = z + beta p; p.q
         const double beta = sh.bcast[3];
         double pq = 0.0;
-        for_each_slot64<TPR>(P, bid, nb, [&](int slot, int sub, bool active) {
-            const int row = row_of(slot, active);
+        for_each_slot64(P, bid, nb, [&](int slot) {
+            const int row = row_of(slot);
             int e0 = 0, e1 = 0;
             if (row >= 0) ends(slot, e0, e1);
             double s0, s1, s2;
-            p_row_sum64<TPR>(B.col, B.val, z, np, e0, e1, sub, row >= 0, s0, s1, s2);
-            if (row < 0 || sub != 0) return;
+            p_row_sum64(B.col, B.val, z, np, e0, e1, row >= 0, s0, s1, s2);
+            if (row < 0) return;
             const double sv[3] = {s0, s1, s2};
             const double d = B.diag[row];
 #pragma unroll
@@ -1912,9 +1887,9 @@ __device__ __forceinline__ void persistent_solve64(const KParams& P, const DevBu
         // ---- x += alpha p; r -= alpha q; z = D^-1 r (own rows); r.r, r.z
         const double a = sh.bcast[2];
         double rr = 0.0, rz = 0.0;
-        for_each_slot64<TPR>(P, bid, nb, [&](int slot, int sub, bool active) {
-            const int i = row_of(slot, active);
-            if (i < 0 || sub != 0) return;
+        for_each_slot64(P, bid, nb, [&](int slot) {
+            const int i = row_of(slot);
+            if (i < 0) return;
             const double di = B.dinv[i];
             double rs = 0.0;
 #pragma unroll
@@ -1952,13 +1927,13 @@ __device__ __forceinline__ void persistent_solve64(const KParams& P, const DevBu
         // ---- the FP64 true residual r = b - A x (z = D^-1 r): accept, restart or give up
         {
             double trr = 0.0, trz = 0.0;
-            for_each_slot64<TPR>(P, bid, nb, [&](int slot, int sub, bool active) {
-                const int row = row_of(slot, active);
+            for_each_slot64(P, bid, nb, [&](int slot) {
+                const int row = row_of(slot);
                 int e0 = 0, e1 = 0;
                 if (row >= 0) ends(slot, e0, e1);
                 double s0, s1, s2;
-                p_row_sum64<TPR>(B.col, B.val, x, np, e0, e1, sub, row >= 0, s0, s1, s2);
-                if (row < 0 || sub != 0) return;
+                p_row_sum64(B.col, B.val, x, np, e0, e1, row >= 0, s0, s1, s2);
+                if (row < 0) return;
                 const double sv[3] = {s0, s1, s2};
                 const double d = B.diag[row], di = B.dinv[row];
                 double rs = 0.0;
@@ -2015,284 +1990,228 @@ done:
     }
 }
 
-// s_a = sum over the row's entries k = sub, sub + TPR, ... of w_k D^-1_col v_a[col_k]
-template <int TPR>
-__device__ __forceinline__ void p_row_sum64_scaled(const int* __restrict__ col, const double* __restrict__ val,
-                                                   const double* __restrict__ dinv, const double* v, int np, int e0,
-                                                   int e1, int sub, bool active, double& s0, double& s1, double& s2)
-{
-    s0 = s1 = s2 = 0.0;
-    if (active) {
-        for (int eb = e0 + 32 * sub; eb < e1; eb += 32 * TPR * kBatch64) {
-            int j[kBatch64];
-            double w[kBatch64];
-#pragma unroll
-            for (int u = 0; u < kBatch64; ++u) {
-                const int e = eb + 32 * TPR * u;
-                j[u] = 0;
-                w[u] = 0.0;
-                if (e < e1) {
-                    j[u] = ld_stream(col + e);
-                    w[u] = __ldg(val + e);
-                }
-            }
-            double g0[kBatch64], g1[kBatch64], g2[kBatch64], dj[kBatch64];
-#pragma unroll
-            for (int u = 0; u < kBatch64; ++u) {
-                g0[u] = g1[u] = g2[u] = dj[u] = 0.0;
-                if (w[u] != 0.0) {
-                    dj[u] = __ldg(dinv + j[u]);
-                    g0[u] = v[j[u]];
-                    g1[u] = v[np + j[u]];
-                    g2[u] = v[2 * np + j[u]];
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < kBatch64; ++u) {
-                const double ww = w[u] * dj[u];
-                s0 += ww * g0[u];
-                s1 += ww * g1[u];
-                s2 += ww * g2[u];
-            }
-        }
-    }
-#pragma unroll
-    for (int o = 1; o < TPR; o <<= 1) {
-        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-    }
-}
-
 // Small systems: pipelined CG (Ghysels & Vanroose, Parallel Computing 40, 2014)
-// with the Jacobi preconditioner, FP64, one grid reduction per iteration.  With
-// u = D^-1 r and m = D^-1 w formed where they are used, per iteration:
+// with the Jacobi preconditioner, FP64, on chip (pcg64.cuh), one grid
+// reduction per iteration.  With u = D^-1 r and m = D^-1 w, per iteration:
 //   gamma = (r, u), delta = (w, u), ||r||^2           (the barrier's reduction)
-//   beta = gamma / gamma_old, alpha = gamma / (delta - beta gamma / alpha_old)
+//   beta = gamma / gamma_old, alpha = gamma / den, den = delta - beta^2 den_old
 //   n = A m;  z = n + beta z;  s = w + beta s;  p = u + beta p;
 //   x += alpha p;  r -= alpha s;  w -= alpha z
-// so the reduction of the next iteration's scalars and the publication of w
-// for its SpMV share one barrier (w double-buffered: the SpMV reads the
-// iteration's w while the update writes the next one).  The recurrence
-// residual arms an FP64 true residual b - A x, which ends the solve or
-// restarts the recurrences from it.
-__device__ __forceinline__ void pipelined_solve64(const KParams& P, const DevBuffers& B, int bid, int nb, PShared& sh,
-                                                  int from_x)
-{
-    constexpr int TPR = 4;
-    DevState* st = B.st;
-    if (threadIdx.x == 0) sh.flag = 0;
-    __syncthreads();
-    if (st->error | st->overflow) return;   // uniform: set before the launch
-    unsigned int gen = 0u;
-    const int np = P.npad;
-    double* x = B.x;
-    double* r = B.r;
-    double* z = B.z;
-    double* p = B.p;
-    double* sv = B.s64;
-    double* wbuf[2] = {B.q, B.s64 + 3 * (size_t)np};
-    int cur = 0;        // the w buffer of the current iteration
-    int pset = 0;       // partial-sum set of the next reduction (consecutive ones differ)
-    auto row_of = [&](int slot, bool active) { return active ? B.slot_row[slot] : -1; };
-    auto ends = [&](int slot, int& e0, int& e1) {
-        e0 = B.chunk_off[slot >> 5] + (slot & 31);
-        e1 = B.chunk_off[(slot >> 5) + 1];
-    };
-    auto partials = [&]() {   // two sets of up to three sums each
-        double* q = B.partials + (size_t)pset * 4 * kMaxPartials;
-        pset ^= 1;
-        return q;
-    };
-    // w = A D^-1 r into wbuf[cur]; z = s = p = 0; gamma, delta, ||r||^2 (after a barrier that published r)
-    auto restart_w = [&](double (&tot)[3]) -> bool {
-        double g = 0.0, d = 0.0, rr = 0.0;
-        double* w = wbuf[cur];
-        for_each_slot64<TPR>(P, bid, nb, [&](int slot, int sub, bool active) {
-            const int row = row_of(slot, active);
-            int e0 = 0, e1 = 0;
-            if (row >= 0) ends(slot, e0, e1);
-            double s0, s1, s2;
-            p_row_sum64_scaled<TPR>(B.col, B.val, B.dinv, r, np, e0, e1, sub, row >= 0, s0, s1, s2);
-            if (row < 0 || sub >= 3) return;   // lane c: component c
-            const double sm = sub == 0 ? s0 : (sub == 1 ? s1 : s2);
-            const double dg = B.diag[row], di = B.dinv[row];
-            {
-                const int k2 = sub * np + row;
-                const double rk = r[k2], uk = di * rk;
-                const double wk = dg * uk - P.alpha * sm;
-                w[k2] = wk;
-                z[k2] = 0.0;
-                sv[k2] = 0.0;
-                p[k2] = 0.0;
-                g += rk * uk;
-                d += wk * uk;
-                rr += rk * rk;
+// (den is delta - beta gamma / alpha_old with alpha_old = gamma_old / den_old:
+// one division less on the path).  The reduction of the next iteration's
+// scalars and the publication of m for its product share one barrier, and the
+// product A m, which needs no scalar, runs while three warps per block sum
+// the partials and form alpha and beta.  m is double-buffered: a product reads
+// one buffer while the updates write the other.  The recurrence residual arms
+// an FP64 true residual b - A x, which ends the solve or restarts the
+// recurrences from it.
+// Measured per iteration (whole solve / iterations, clustered systems), the
+// form with four lanes per row and vectors in memory -> this one: n = 500, 8
+// -> 16 blocks: 14.1 -> 5.9 us; n = 4,096, 64 -> 128 blocks: 15.2 -> 6.7 us; n
+// = 60,013: 44 -> 24 us (there the gathers' L1 wavefronts and the FP64 issue).
+struct SellSystem64 {   // the sliced layout as pcg64's system
+    const KParams& P;
+    const DevBuffers& B;
+    int bid, nb;
+    struct Entries {
+        const int* col;
+        const double* val;
+        int cnt;
+        __device__ bool valid() const { return true; }
+        __device__ void get(int k, int& j, double& w) const
+        {
+            if (k < cnt) {
+                j = __ldg(col + 32 * k);
+                w = __ldg(val + 32 * k);
             }
-        });
-        const double v[3] = {g, d, rr};
-        return grid_allreduce<3>(st, gen, sh, v, partials(), tot, bid, nb);
-    };
-    // the true residual r = b - A x (after a barrier that published x); ||r||^2
-    auto true_residual = [&](double (&tot)[1], bool first) -> bool {
-        double rr = 0.0, bb = 0.0;
-        for_each_slot64<TPR>(P, bid, nb, [&](int slot, int sub, bool active) {
-            const int row = row_of(slot, active);
-            int e0 = 0, e1 = 0;
-            if (row >= 0) ends(slot, e0, e1);
-            double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-            if (!first || from_x) p_row_sum64<TPR>(B.col, B.val, x, np, e0, e1, sub, row >= 0, s0, s1, s2);
-            if (row < 0 || sub >= 3) return;   // lane c: component c
-            const double sm = sub == 0 ? s0 : (sub == 1 ? s1 : s2);
-            const double dg = B.diag[row];
-            {
-                const int k2 = sub * np + row;
-                const double bk = B.b[k2];
-                double rk = bk;
-                if (!first || from_x)
-                    rk = bk - (dg * x[k2] - P.alpha * sm);
-                else
-                    x[k2] = 0.0;
-                r[k2] = rk;
-                rr += rk * rk;
-                bb += bk * bk;
-            }
-        });
-        if (first) {
-            const double v[2] = {rr, bb};
-            double t2[2];
-            if (!grid_allreduce<2>(st, gen, sh, v, partials(), t2, bid, nb)) return false;
-            if (threadIdx.x == 0) sh.bnorm2 = t2[1];
-            tot[0] = t2[0];
-            return true;
         }
-        const double v[1] = {rr};
-        return grid_allreduce<1>(st, gen, sh, v, partials(), tot, bid, nb);
     };
+    __device__ double alpha() const { return P.alpha; }
+    __device__ bool in_range(int) const { return true; }
+    __device__ int chunk(int i) const { return bid + nb * i; }
+    __device__ int row(int i, int lane) const { return B.slot_row[32 * chunk(i) + lane]; }
+    __device__ int chunk_len(int i, int) const { return (B.chunk_off[chunk(i) + 1] - B.chunk_off[chunk(i)]) >> 5; }
+    __device__ Entries entries(int i, int lane, int row) const
+    {
+        const int e = B.chunk_off[chunk(i)];
+        return Entries{B.col + e + lane, B.val + e + lane, row < 0 ? 0 : (B.chunk_off[chunk(i) + 1] - e) >> 5};
+    }
+};
 
-    double t3[3], t1[1];
-    bool first = true;   // beta = 0: the first iteration of the solve or of a restart
-    if (!true_residual(t1, true)) goto done;
+struct Cg64Scalars {
+    double rho, den, bnorm2, last_res;
+    int iter, restarts, status, started, first;
+};
+
+template <int U, int KB>
+__device__ __forceinline__ void pipelined_solve64(const KParams& P, const DevBuffers& B, const p64::Grid& G,
+                                                  p64::Shared& sh, Cg64Scalars& cg, unsigned char* dyn,
+                                                  int smem_bytes, int from_x)
+{
+    DevState* st = B.st;
+    const SellSystem64 S{P, B, G.bid, G.nb};
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, np = P.npad;
+    const int ncw = (blockDim.x >> 5) - p64::kScalarWarps, groups = ncw / 3;
+    const int grp = warp / 3, comp = warp - 3 * grp;
+    const int nc = (P.nchunks - G.bid + G.nb - 1) / G.nb;   // chunks bid, bid + nb, ...
+    const int cap = smem_bytes / p64::kEntryBytes;
     if (threadIdx.x == 0) {
-        sh.iter = 0;
-        sh.restarts = 0;
-        sh.status = SP_OK;
-        sh.last_res = sh.bnorm2 > 0.0 ? sqrt(t1[0] / sh.bnorm2) : 0.0;
+        sh.flag = 0;
         sh.action = 0;
-        if (!isfinite(sh.bnorm2) || !isfinite(t1[0])) {
-            sh.status = SP_ERR_NONFINITE;
-            sh.action = 2;
-        } else if (sh.bnorm2 == 0.0 || t1[0] <= P.tol2 * sh.bnorm2) {
-            sh.action = 2;   // b = 0 (x = 0 then) or the start meets the tolerance
-        }
-        if (bid == 0) {
-            st->bnorm2 = sh.bnorm2;
-            st->zero_b = sh.bnorm2 == 0.0 ? 1 : 0;
-        }
+        cg.started = 0;
+        cg.status = SP_OK;
+        cg.iter = cg.restarts = 0;
+        cg.last_res = 0.0;
     }
-    __syncthreads();
-    if (sh.action == 2) goto done;
-    if (!restart_w(t3)) goto done;
-    for (;;) {
-        // ---- the scalars of this iteration (thread 0, identical totals in every block)
-        if (threadIdx.x == 0) {
-            const double g = t3[0], d = t3[1], rr = t3[2];
-            sh.action = 0;
-            if (!isfinite(g) || !isfinite(d) || !isfinite(rr)) {
-                sh.status = SP_ERR_NONFINITE;
-                sh.action = 2;
-            } else if (rr <= P.tol2 * sh.bnorm2 || sh.iter >= P.max_iter) {
-                sh.action = 1;   // the true residual decides
+    p64::stage(S, sh, dyn, smem_bytes, nc);
+    unsigned int gen = 0u;
+    double* rec[2] = {B.s64, B.s64 + 4 * (size_t)np};
+    int cur = 0;   // the buffer of the next product
+    int row[U];
+    double x[U], r[U], w[U], z[U], s[U], p[U], di[U], sm[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int i = grp + groups * u;
+        row[u] = warp < ncw && i < nc ? S.row(i, lane) : -1;
+        x[u] = row[u] >= 0 && from_x ? B.x[comp * np + row[u]] : 0.0;
+        di[u] = row[u] >= 0 ? B.dinv[row[u]] : 0.0;
+        r[u] = w[u] = z[u] = s[u] = p[u] = sm[u] = 0.0;
+        if (row[u] >= 0) rec[0][4 * (size_t)row[u] + comp] = x[u];
+    }
+    enum { kX, kResidual, kIterate };   // the values the next reduction carries (kX: none, x was published)
+    int phase = kX;
+    double v0 = 0.0, v1 = 0.0, v2 = 0.0;
+    auto product = [&] {   // sum_j alpha w_ij of the published vector
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int i = grp + groups * u;
+            if (i < nc) sm[u] = p64::row_product<KB>(S, sh, dyn, cap, i, row[u], rec[cur], comp);
+        }
+    };
+    auto scalars = [&] {   // one thread per block, the same totals in every block
+        sh.action = 0;
+        if (phase == kResidual) {
+            const double rr = sh.tot[0];
+            if (!cg.started) {
+                cg.started = 1;
+                cg.bnorm2 = sh.tot[1];
+                cg.last_res = cg.bnorm2 > 0.0 ? sqrt(rr / cg.bnorm2) : 0.0;
+                if (!isfinite(cg.bnorm2) || !isfinite(rr)) {
+                    cg.status = SP_ERR_NONFINITE;
+                    sh.action = 2;
+                } else if (cg.bnorm2 == 0.0 || rr <= P.tol2 * cg.bnorm2) {
+                    sh.action = 2;   // b = 0 (the finishing kernel zeroes x) or the start meets the tolerance
+                }
+                if (G.bid == 0) {
+                    st->bnorm2 = cg.bnorm2;
+                    st->zero_b = cg.bnorm2 == 0.0 ? 1 : 0;
+                }
             } else {
-                const double beta = first ? 0.0 : g / sh.rho;
-                const double den = first ? d : d - beta * g / sh.alpha_d;   // (p, A p) of the new direction
-                if (!(den > 0.0)) {
-                    sh.action = 1;   // lost to rounding near convergence: the true residual decides
-                } else {
-                    sh.beta_d = beta;
-                    sh.alpha_d = g / den;
-                    sh.rho = g;
-                }
-            }
-        }
-        __syncthreads();
-        first = false;
-        if (sh.action == 2) break;
-        if (sh.action == 1) {
-            if (!true_residual(t1, false)) break;
-            if (threadIdx.x == 0) {
-                sh.last_res = sqrt(t1[0] / sh.bnorm2);
-                if (bid == 0) st->true_checks += 1;
-                sh.action = 0;
-                if (!isfinite(t1[0])) {
-                    sh.status = SP_ERR_NONFINITE;
+                cg.last_res = sqrt(rr / cg.bnorm2);
+                if (G.bid == 0) st->true_checks += 1;
+                if (!isfinite(rr)) {
+                    cg.status = SP_ERR_NONFINITE;
                     sh.action = 2;
-                } else if (t1[0] <= P.tol2 * sh.bnorm2) {
+                } else if (rr <= P.tol2 * cg.bnorm2) {
                     sh.action = 2;   // converged
-                } else if (sh.iter >= P.max_iter || sh.restarts >= kMaxCgRestarts + 8) {
-                    sh.status = SP_ERR_NOT_CONVERGED;
+                } else if (cg.iter >= P.max_iter || cg.restarts >= kMaxCgRestarts + 8) {
+                    cg.status = SP_ERR_NOT_CONVERGED;
                     sh.action = 2;
                 } else {
-                    ++sh.restarts;
+                    ++cg.restarts;
                 }
             }
-            __syncthreads();
-            if (sh.action == 2) break;
-            if (!restart_w(t3)) break;
-            first = true;
-            continue;
+            cg.first = 1;
+            return;
         }
-        // ---- n = A D^-1 w; the recurrences (w into the other buffer); the next reduction
-        const double a = sh.alpha_d, beta = sh.beta_d;
-        const double* w = wbuf[cur];
-        double* wn = wbuf[cur ^ 1];
-        double g = 0.0, d = 0.0, rr = 0.0;
-        for_each_slot64<TPR>(P, bid, nb, [&](int slot, int sub, bool active) {
-            const int row = row_of(slot, active);
-            int e0 = 0, e1 = 0;
-            if (row >= 0) ends(slot, e0, e1);
-            double s0, s1, s2;
-            p_row_sum64_scaled<TPR>(B.col, B.val, B.dinv, w, np, e0, e1, sub, row >= 0, s0, s1, s2);
-            // every lane of the row holds the sums: lane c updates component c
-            // (a third of the FP64 instructions per warp of a lane doing all three)
-            if (row < 0 || sub >= 3) return;
-            const double sm = sub == 0 ? s0 : (sub == 1 ? s1 : s2);
-            const double dg = B.diag[row], di = B.dinv[row];
-            {
-                const int k2 = sub * np + row;
-                const double wk = w[k2];
-                const double nk = dg * (di * wk) - P.alpha * sm;   // (A m)_k, m = D^-1 w
-                const double zk = nk + beta * z[k2];
-                const double sk = wk + beta * sv[k2];
-                const double pk = di * r[k2] + beta * p[k2];
-                z[k2] = zk;
-                sv[k2] = sk;
-                p[k2] = pk;
-                x[k2] += a * pk;
-                const double rk = r[k2] - a * sk;
-                r[k2] = rk;
-                const double wnk = wk - a * zk;
-                wn[k2] = wnk;
-                const double uk = di * rk;
-                g += rk * uk;
-                d += wnk * uk;
-                rr += rk * rk;
+        const double g = sh.tot[0], d = sh.tot[1], rr = sh.tot[2];
+        if (!isfinite(g) || !isfinite(d) || !isfinite(rr)) {
+            cg.status = SP_ERR_NONFINITE;
+            sh.action = 2;
+        } else if (rr <= P.tol2 * cg.bnorm2 || cg.iter >= P.max_iter) {
+            sh.action = 1;   // the true residual decides
+        } else {
+            const double beta = cg.first ? 0.0 : g / cg.rho;
+            const double den = cg.first ? d : fma(-beta * beta, cg.den, d);   // (p, A p) of the new direction
+            if (!(den > 0.0)) {
+                sh.action = 1;   // lost to rounding near convergence: the true residual decides
+            } else {
+                sh.beta = beta;
+                sh.alpha = g / den;
+                cg.rho = g;
+                cg.den = den;
+                cg.first = 0;
+                ++cg.iter;
             }
-        });
+        }
+    };
+    auto publish = [&](int u, double v) { rec[cur ^ 1][4 * (size_t)row[u] + comp] = v; };
+    for (;;) {
+        const int K = phase == kX ? 0 : (phase == kResidual ? 2 : 3);
+        if (!p64::reduce_overlapped(G, sh, gen, K, v0, v1, v2, product, scalars)) break;
+        if (K > 0 && sh.action == 2) break;
+        v0 = v1 = v2 = 0.0;
+        if (phase == kX) {   // r = b - A x, ||r||^2 and ||b||^2; u published
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (row[u] < 0) continue;
+                const double b = B.b[comp * np + row[u]];
+                r[u] = b - (B.diag[row[u]] * x[u] - sm[u]);
+                v0 = fma(r[u], r[u], v0);
+                v1 = fma(b, b, v1);
+                publish(u, di[u] * r[u]);
+            }
+            phase = kResidual;
+        } else if (phase == kResidual) {   // w = A u (A_ii u = r); m published
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (row[u] < 0) continue;
+                const double uk = di[u] * r[u];
+                w[u] = r[u] - sm[u];
+                z[u] = s[u] = p[u] = 0.0;
+                v0 = fma(r[u], uk, v0);
+                v1 = fma(w[u], uk, v1);
+                v2 = fma(r[u], r[u], v2);
+                publish(u, di[u] * w[u]);
+            }
+            phase = kIterate;
+        } else if (sh.action == 1) {   // the true residual: x published
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (row[u] >= 0) publish(u, x[u]);
+            phase = kX;
+        } else {
+            const double a = sh.alpha, beta = sh.beta;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (row[u] < 0) continue;
+                const double n = w[u] - sm[u];   // (A m)_k with A_ii D^-1_ii = 1
+                z[u] = fma(beta, z[u], n);
+                s[u] = fma(beta, s[u], w[u]);
+                w[u] = fma(-a, z[u], w[u]);
+                publish(u, di[u] * w[u]);
+                p[u] = fma(beta, p[u], di[u] * r[u]);
+                x[u] = fma(a, p[u], x[u]);
+                r[u] = fma(-a, s[u], r[u]);
+                const double uk = di[u] * r[u];
+                v0 = fma(r[u], uk, v0);
+                v1 = fma(w[u], uk, v1);
+                v2 = fma(r[u], r[u], v2);
+            }
+        }
         cur ^= 1;
-        const double v[3] = {g, d, rr};
-        if (!grid_allreduce<3>(st, gen, sh, v, partials(), t3, bid, nb)) break;
-        if (threadIdx.x == 0) ++sh.iter;
     }
-done:
-    if (bid == 0 && threadIdx.x == 0) {
-        st->iter = sh.iter;
-        st->restarts = sh.restarts;
-        st->last_res = sh.last_res;
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+        if (row[u] >= 0) B.x[comp * np + row[u]] = x[u];
+    if (G.bid == 0 && threadIdx.x == 0) {
+        st->iter = cg.iter;
+        st->restarts = cg.restarts;
+        st->last_res = cg.last_res;
         st->done = 1;
-        if (st->error == 0 && sh.status != SP_OK) {
-            st->status = sh.status;
-            st->error = sh.status;
+        if (st->error == 0 && cg.status != SP_OK) {
+            st->status = cg.status;
+            st->error = cg.status;
         } else if (st->error != 0) {
             st->status = st->error;
         } else {
@@ -2301,14 +2220,25 @@ done:
     }
 }
 
-template <int TPR>
+template <int U, int KB>
+__global__ void __launch_bounds__(p64::max_threads(U), 1) k64_cg_pipelined(KParams P, DevBuffers B, int from_x,
+                                                                          int smem_bytes)
+{
+    extern __shared__ float4 res_dyn[];
+    __shared__ p64::Shared sh;
+    __shared__ Cg64Scalars cg;
+    DevState* st = B.st;
+    const p64::Grid G{&st->bar_count, &st->bar_exit, &st->error, st->bar_timeout_ns, B.partials, kMaxPartials,
+                      (int)blockIdx.x, (int)gridDim.x};
+    if (!(st->error | st->overflow))   // uniform: set before the launch
+        pipelined_solve64<U, KB>(P, B, G, sh, cg, reinterpret_cast<unsigned char*>(res_dyn), smem_bytes, from_x);
+    p64::leave(G);
+}
+
 __global__ void __launch_bounds__(512, 1) k64_cg_persistent(KParams P, DevBuffers B, int from_x)
 {
     __shared__ PShared sh;
-    if (TPR == 1)
-        persistent_solve64<1>(P, B, blockIdx.x, gridDim.x, sh, from_x);
-    else
-        pipelined_solve64(P, B, blockIdx.x, gridDim.x, sh, from_x);
+    persistent_solve64(P, B, blockIdx.x, gridDim.x, sh, from_x);
     barrier_leave(B.st, gridDim.x);
 }
 
@@ -2508,52 +2438,48 @@ int cg_persistent_grid(const KParams& P, const DevBuffers& B, Launch L)
     return (int)grid_of(cfg_of(P, B, L), P, L);
 }
 
-// FP64 persistent solve.  Systems of at least two windows of 256 rows per SM:
-// blocks of 512 threads (two windows at a time), one per SM, one thread per
-// row.  Smaller ones: blocks of two chunks of 32 rows with four threads per
-// row (256 threads), as many blocks as chunk pairs up to one per SM.
-void cg64_shape(const KParams& P, Launch L, int* grid, int* threads, int* tpr)
+// FP64 solve in one launch.  Systems of up to 16 chunks of 32 rows per SM
+// (77,824 rows on 152 SMs: the registers' limit) run on chip, spread over as
+// many SMs as they have chunks (solve at n = 60,013: 2.51 ms with vectors in
+// memory, 1.37 on chip); larger ones with their vectors in memory: blocks of
+// 512 threads (two windows at a time), one per SM, one thread per row.
+struct Shape64 {
+    int blocks, threads, smem;
+    const void* fn;
+};
+Shape64 cg64_shape(const KParams& P, Launch L)
 {
+    const p64::Shape s = p64::shape_of(std::max(P.nchunks, 1), L.num_sms, 4);
+    if (s.u > 0)
+        return Shape64{s.blocks, s.threads, s.smem,
+                       s.u == 1 ? (const void*)k64_cg_pipelined<1, 12>
+                                : (s.u == 2 ? (const void*)k64_cg_pipelined<2, 8> : (const void*)k64_cg_pipelined<4, 6>)};
     const int nwin = P.nslots / 256;
-    const int cap = std::min(L.num_sms, kMaxPartials);
-    if (nwin >= 2 * L.num_sms) {
-        *grid = std::min(cap, (nwin + 1) / 2);
-        *threads = 512;
-        *tpr = 1;
-    } else {
-        const int nch = std::max(P.nchunks, 1);
-        const int g = std::max(1, std::min(cap, (nch + 1) / 2));
-        *grid = g;
-        *threads = 4 * 32 * std::min(4, (nch + g - 1) / g);
-        *tpr = 4;
-    }
+    return Shape64{std::min(std::min(L.num_sms, kMaxPartials), (nwin + 1) / 2), 512, 0, (const void*)k64_cg_persistent};
 }
 
 cudaError_t launch_cg64_persistent(const KParams& P, DevBuffers& B, int from_x, Launch L)
 {
-    int g = 1, bs = 32, tpr = 1;
-    cg64_shape(P, L, &g, &bs, &tpr);
+    Shape64 s = cg64_shape(P, L);
+    if (s.smem > 32 * 1024) {   // with the static arrays, near the 48 KB a kernel has by default
+        const cudaError_t e = cudaFuncSetAttribute(s.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, s.smem);
+        if (e != cudaSuccess) return e;
+    }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)g);
-    cfg.blockDim = dim3((unsigned)bs);
-    cfg.dynamicSmemBytes = 0;
+    cfg.gridDim = dim3((unsigned)s.blocks);
+    cfg.blockDim = dim3((unsigned)s.threads);
+    cfg.dynamicSmemBytes = (size_t)s.smem;
     cfg.stream = L.stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    void* args[] = {const_cast<KParams*>(&P), &B, &from_x};
-    return cudaLaunchKernelExC(&cfg, tpr == 1 ? (const void*)k64_cg_persistent<1> : (const void*)k64_cg_persistent<4>,
-                               args);
+    void* args[] = {const_cast<KParams*>(&P), &B, &from_x, &s.smem};   // the last for the on-chip form only
+    return cudaLaunchKernelExC(&cfg, s.fn, args);
 }
 
-int cg64_persistent_grid(const KParams& P, Launch L)
-{
-    int g = 1, bs = 32, tpr = 1;
-    cg64_shape(P, L, &g, &bs, &tpr);
-    return g;
-}
+int cg64_persistent_grid(const KParams& P, Launch L) { return cg64_shape(P, L).blocks; }
 
 cudaError_t launch_cg32_persistent(const KParams& P, DevBuffers& B, Launch L)
 {

@@ -160,8 +160,8 @@ struct DevBuffers {
     double* p;       // [3][npad]
     double* q;       // [3][npad]
     double* z;       // [3][npad] D^-1 r (FP64 solver)
-    double* s64;     // [6][npad] FP64 pipelined solve of small systems: s, and the second buffer of w
-                     // (w in q and s64 + 3 npad in turn, z in z)
+    double* s64;     // [2][npad][4] FP64 on-chip solve of small systems: the two buffers of its published
+                     // records (x, y, z, 0 of a row)
     uint4* posfix;   // [npad] mixed: positions in 32-bit fixed point of the box edges (x, y, z, 0), built
                      // before each matrix-free solve
     float4* r4;      // [npad] mixed solver vectors, (x, y, z, 0) per row

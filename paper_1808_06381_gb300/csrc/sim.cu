@@ -752,7 +752,7 @@ int sp_sim_create(const sp_params* p, const double* pos_host, sp_sim** out)
     A(dev_alloc(s, &B.p, v3));
     A(dev_alloc(s, &B.q, v3));
     A(dev_alloc(s, &B.z, v3));
-    if (!mixed(s)) A(dev_alloc(s, &B.s64, 2 * v3));
+    if (!mixed(s)) A(dev_alloc(s, &B.s64, 8 * (size_t)npad));
     A(dev_alloc(s, &B.r4, (size_t)npad));
     if (mixed(s)) {   // double-float forms of the mixed solver's true residuals
         A(dev_alloc(s, &B.diag32lo, (size_t)npad));

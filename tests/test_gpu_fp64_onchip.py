@@ -1,0 +1,56 @@
+"""The FP64 solve on chip (k64_cg_pipelined) at the edges of its range: one row per thread
+against two and four, the largest system, one chunk beyond it, ragged chunks, and chunks
+whose rows are too long for shared memory."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+ss = pytest.importorskip("paper_1808_06381_gb300")
+
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-11
+# The oracle forms b - A v in FP64 with its own sums: rounding of order n_partners * 2^-53 of
+# the row's terms, below 1e-13 of ||b|| for these systems.
+BOUND = TOL + 1e-13
+
+
+def _check(n, pos, L, warm):
+    kappa = ss.kappa_from_kappa_tau(0.5)
+    delta = 0.3 * L
+    sim = ss.Simulation(n, (L,) * 3, kappa, seed=9, precision="fp64", warm_start=warm, cg_tol=TOL, cg_max_iter=5000,
+                        positions=pos)
+    p = oracle.Params(n=n, L=(L,) * 3, kappa=oracle.kappa_from_kappa_tau(0.5), seed=9)
+    sim.set_positions(pos, delta)
+    for step in range(2 if warm == "prev" else 1):   # the second solve starts from the first's velocities
+        sim.set_step(step)
+        sim.build_neighbors()
+        sim.assemble()
+        info = sim.solve_velocities()
+        assert info["status"] == 0 and info["residual"] <= TOL, info
+        v = sim.get_velocities()
+        sysr = oracle.assemble(p, pos, oracle.neighbors(p, pos, delta), oracle.noise(9, step, np.arange(n)),
+                               delta)
+        res = np.linalg.norm(sysr.b - sysr.matvec(v)) / np.linalg.norm(sysr.b)
+        assert res <= BOUND, (step, res)
+    sim.close()
+
+
+# chunks of 32 rows per SM on 152 SMs: 1 up to 4,864 rows, 5 up to 24,320 (one component a
+# thread), 10 up to 48,640 (two), 16 up to 77,824 (four); beyond, vectors in memory
+@pytest.mark.parametrize("n,warm", [(33, "none"), (257, "prev"), (4865, "none"), (24320, "none"), (24321, "prev"),
+                                    (48641, "none"), (77824, "none"), (77825, "none")])
+def test_on_chip_solve_meets_the_tolerance_on_the_oracles_system(n, warm):
+    L = max(synth.box_length(n), 2.01)
+    _check(n, synth.uniform_positions(n, (L,) * 3, 3), L, warm)
+
+
+@pytest.mark.parametrize("n,knot", [(900, 300), (20011, 400)])
+def test_rows_too_long_for_shared_memory(n, knot):
+    """A knot of particles within r_c of each other: rows of more entries than a chunk's share."""
+    L = synth.box_length(n)
+    pos = synth.uniform_positions(n, (L,) * 3, 4)
+    pos[:knot] = 0.5 * L + 0.4 * (pos[:knot] / L - 0.5)
+    _check(n, pos, L, "none")
