@@ -520,7 +520,7 @@ const char* sp_batch_last_error(const sp_batch* b);
  *   the real length of col_dev and w_dev).
  *
  * It allocates nothing: its working vectors live in one fixed device array
- * (about 3.2 MB) that every device context loading this library holds until
+ * (about 2.1 MB) that every device context loading this library holds until
  * the process exits.  Hence:
  *   - n must be <= 32768, else SP_ERR_INVALID_ARG (sp_last_error(NULL) says why);
  *   - every call on a device shares that array, so calls that may overlap on

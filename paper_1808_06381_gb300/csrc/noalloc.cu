@@ -5,13 +5,22 @@
 // framework that owns every device allocation (a fixed memory pool, a
 // real-time or embedded loop that forbids allocation after start-up, or a
 // library that must not touch the caller's allocator).  This entry point takes
-// the system and the output from the caller and keeps its own working vectors
-// (r, z, p, q, the Jacobi diagonal, the partial sums and the solver scalars)
-// in one file-scope device array of fixed size, so it never allocates.
+// the system and the output from the caller and keeps what its blocks exchange
+// (the two buffers of published records, the partial sums and the solver's
+// state) in one file-scope device array of fixed size, so it never allocates.
+//
+// The solve is one cooperative launch of the on-chip CG of pcg64.cuh: the
+// entries in shared memory, the vectors in registers.  Jacobi-PCG with the
+// direction update fused into the product (q = A z + beta q, p = z + beta p),
+// two grid reductions per iteration: a caller's matrix may be worse
+// conditioned than Eq. algebra's, and pipelined CG (one reduction) drifts
+// further from the true residual.  Measured (n = 12,289 clustered rows in
+// random order, 62 iterations): one thread per row, four kernels an iteration
+// and the host polling every eighth, 3.48 ms; this form 0.96 ms.
 //
 // Limits and sharing:
 //   - at most kNoallocMaxRows rows; larger systems are rejected;
-//   - the array (about 3.2 MB) lives in every device context that loads the
+//   - the array (about 2.1 MB) lives in every device context that loads the
 //     library, until the process exits;
 //   - every call on a device uses the same array: calls that may overlap on
 //     the GPU (other streams, other host threads) race and must be serialised
@@ -29,270 +38,266 @@
 #include <string>
 
 #include "internal.cuh"
+#include "pcg64.cuh"
 
 namespace ss {
 namespace {
 
 constexpr long long kNoallocMaxRows = 32768;
-constexpr int kNaThreads = 256;
-constexpr int kNaBlocks = 128;   // kNaBlocks * kNaThreads = the rows handled per grid sweep
+constexpr int kNaMaxBlocks = 512;
 
 struct NaState {
-    double bnorm2, rho, alpha, beta, rr, last_res;
-    int iter, done, status, check_true, restarts;
-    unsigned int ticket;
+    double bnorm2, last_res;
+    int iter, status, done, error;
+    alignas(128) unsigned int count;   // the launch's grid barriers (pcg64.cuh)
+    alignas(128) unsigned int exits;
 };
 
-constexpr size_t kPlane = (size_t)kNoallocMaxRows;
-constexpr size_t kVecDoubles = 3 * kPlane;               // one [3][n] vector
-constexpr size_t kScratchDoubles = 4 * kVecDoubles       // r, z, p, q
-                                   + kPlane              // dinv
-                                   + 2 * kNaBlocks;      // partial sums
-constexpr size_t kScratchBytes = kScratchDoubles * sizeof(double) + 256;
+constexpr size_t kRecordDoubles = 2 * 4 * (size_t)kNoallocMaxRows;       // two buffers of (x, y, z, 0) per row
+constexpr size_t kPartialDoubles = 2 * p64::kScalarWarps * kNaMaxBlocks;
+constexpr size_t kScratchBytes = (kRecordDoubles + kPartialDoubles) * sizeof(double) + sizeof(NaState);
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
-struct NaPtrs {
-    double *r, *z, *p, *q, *dinv, *partials;
-    NaState* st;
-};
-
-NaPtrs carve(unsigned char* base)
-{
-    double* d = reinterpret_cast<double*>(base);
-    NaPtrs s;
-    s.r = d;
-    s.z = d + kVecDoubles;
-    s.p = d + 2 * kVecDoubles;
-    s.q = d + 3 * kVecDoubles;
-    s.dinv = d + 4 * kVecDoubles;
-    s.partials = s.dinv + kPlane;
-    s.st = reinterpret_cast<NaState*>(base + kScratchDoubles * sizeof(double));
-    return s;
-}
-
-struct NaSystem {
+struct NaSystem {   // the caller's arrays, and pcg64's system
     long long n;
     const int* row_ptr;
     const int* col;
     const double* w;
     const double* diag;
-    double alpha;
+    double alpha_e;
     const double* b;
     double* x;
     double tol2;
     int max_iter;
+    const int* rows;   // the block's rows by length, in its shared memory (-1: none)
+    struct Entries {
+        const int* col;
+        const double* w;
+        int cnt;
+        bool ok;
+        __device__ bool valid() const { return ok; }
+        __device__ void get(int k, int& j, double& v) const
+        {
+            if (k < cnt) {
+                j = __ldg(col + k);
+                v = __ldg(w + k);
+            }
+        }
+    };
+    __device__ double alpha() const { return alpha_e; }
+    __device__ bool in_range(int j) const { return j >= 0 && j < n; }
+    __device__ int row(int i, int lane) const { return rows[32 * i + lane]; }
+    // row_ptr must start at 0 and never decrease; a row that breaks this is
+    // not read (and fails the call)
+    __device__ Entries entries(int, int, int row) const
+    {
+        if (row < 0) return Entries{col, w, 0, true};
+        const int e0 = row_ptr[row], e1 = row_ptr[row + 1];
+        const bool ok = e0 >= 0 && e1 >= e0 && (row != 0 || e0 == 0);
+        return Entries{col + (ok ? e0 : 0), w + (ok ? e0 : 0), ok ? e1 - e0 : 0, ok};
+    }
+    __device__ int chunk_len(int i, int lane) const
+    {
+        return __reduce_max_sync(0xffffffffu, entries(i, lane, row(i, lane)).cnt);
+    }
 };
 
-// Sum over the block, then the last block to finish reduces the per-block sums.
-template <int K>
-__device__ bool na_publish(double (&v)[K], double* partials, unsigned int* ticket)
+struct NaScalars {
+    double rho, bnorm2, last_res;
+    int iter, restarts, status;
+};
+
+// Every block validates the rows it reads (row_ptr, and every column inside [0,
+// n)) while it places them, before anything gathers through a column; the
+// first grid reduction carries the verdict, so a malformed system is refused
+// by all blocks together and x stays as it was.
+template <int U, int KB>
+__global__ void __launch_bounds__(p64::max_threads(U), 1) k_na_solve(NaSystem S, double* scratch, int smem_bytes,
+                                                                       unsigned long long limit_ns)
 {
-    __shared__ double sh[32];
-    __shared__ bool last;
-    for (int k = 0; k < K; ++k) {
-        const double t = block_sum(v[k], sh);
-        if (threadIdx.x == 0) partials[k * kNaBlocks + blockIdx.x] = t;
-    }
+    extern __shared__ double na_dyn[];
+    __shared__ p64::Shared sh;
+    __shared__ NaScalars cg;
+    __shared__ int rows[32 * p64::kMaxChunks];
+    unsigned char* dyn = reinterpret_cast<unsigned char*>(na_dyn);
+    NaState* st = reinterpret_cast<NaState*>(scratch + kRecordDoubles + kPartialDoubles);
+    const p64::Grid G{&st->count, &st->exits, &st->error, limit_ns, scratch + kRecordDoubles, kNaMaxBlocks,
+                      (int)blockIdx.x, (int)gridDim.x};
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int ncw = (blockDim.x >> 5) - p64::kScalarWarps, groups = ncw / 3;
+    const int grp = warp / 3, comp = warp - 3 * grp;
+    const int nch = (int)((S.n + 31) / 32), nc = (nch - G.bid + G.nb - 1) / G.nb;   // chunks bid, bid + nb, ...
+    const int cap = smem_bytes / p64::kEntryBytes;
     if (threadIdx.x == 0) {
-        __threadfence();
-        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        sh.flag = 0;
+        sh.action = 0;
+        cg.status = SP_OK;
+        cg.iter = cg.restarts = 0;
+        cg.bnorm2 = cg.last_res = 0.0;
     }
-    __syncthreads();
-    if (!last) return false;
-    __threadfence();
-    for (int k = 0; k < K; ++k) {
-        double s = 0.0;
-        for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) s += __ldcg(partials + k * kNaBlocks + i);
-        v[k] = block_sum(s, sh);
-    }
-    if (threadIdx.x == 0) *ticket = 0u;
-    return true;
-}
-
-// (A u)_i for the three planes of a scratch vector u (plane stride kPlane): A = diag - alpha W.
-__device__ __forceinline__ void na_row_apply(const NaSystem& S, const double* u, long long i, double* out3)
-{
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-    for (int k = S.row_ptr[i]; k < S.row_ptr[i + 1]; ++k) {
-        const long long j = S.col[k];
-        const double w = S.w[k];
-        s0 += w * u[j];
-        s1 += w * u[kPlane + j];
-        s2 += w * u[2 * kPlane + j];
-    }
-    const double d = S.diag[i];
-    out3[0] = d * u[i] - S.alpha * s0;
-    out3[1] = d * u[kPlane + i] - S.alpha * s1;
-    out3[2] = d * u[2 * kPlane + i] - S.alpha * s2;
-}
-
-// Rejects a malformed CSR before anything gathers through it: row_ptr must
-// start at 0 and never decrease, and every column must lie in [0, n) (a
-// column in [n, kPlane) would read another call's stale entries of the shared
-// array, one beyond it memory outside the array).
-__global__ void k_na_validate(NaSystem S, NaPtrs W)
-{
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < S.n; i += gridDim.x * blockDim.x) {
-        const int b = S.row_ptr[i], e = S.row_ptr[i + 1];
-        bool bad = (i == 0 && b != 0) || e < b;
-        for (int k = b; k < e && !bad; ++k) {
-            const int j = S.col[k];
-            bad = j < 0 || (long long)j >= S.n;
+    // the block's rows sorted by length, so that a chunk's rows are about
+    // equally long (the caller's order is arbitrary: chunks of 32 rows as they
+    // come carry ~1.9x the entries of their rows as padding); the keys are
+    // ordered in the dynamic space that the entries take afterwards
+    {
+        unsigned long long* key = reinterpret_cast<unsigned long long*>(na_dyn);
+        const int R = 32 * nc;
+        for (int k = threadIdx.x; k < R; k += blockDim.x) {
+            const long long i = 32ll * (G.bid + (long long)G.nb * (k >> 5)) + (k & 31);
+            const unsigned long long len = i < S.n ? 1ull + (unsigned)S.entries(0, 0, (int)i).cnt : 0ull;
+            key[k] = (len << 32) | (unsigned)k;
         }
-        if (bad) {
-            W.st->status = SP_ERR_INVALID_ARG;
-            W.st->done = 1;
+        __syncthreads();
+        for (int k = threadIdx.x; k < R; k += blockDim.x) {
+            const unsigned long long mine = key[k];
+            int before = 0;
+            for (int m = 0; m < R; ++m) before += key[m] > mine;
+            rows[before] = mine >> 32 ? 32 * (G.bid + G.nb * (k >> 5)) + (k & 31) : -1;
         }
+        __syncthreads();
     }
-}
-
-// x = 0, r = b, z = D^-1 r, p = z; b.b and r.z.
-__global__ void k_na_init(NaSystem S, NaPtrs W)
-{
-    if (W.st->done) return;   // rejected by k_na_validate (uniform over the grid)
-    double v[2] = {0.0, 0.0};
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < S.n; i += gridDim.x * blockDim.x) {
-        const double di = 1.0 / S.diag[i];
-        W.dinv[i] = di;
-        for (int c = 0; c < 3; ++c) {
-            const double bk = S.b[c * S.n + i];
-            S.x[c * S.n + i] = 0.0;
-            W.r[c * kPlane + i] = bk;
-            W.z[c * kPlane + i] = di * bk;
-            W.p[c * kPlane + i] = di * bk;
-            v[0] += bk * bk;
-            v[1] += di * bk * bk;
-        }
+    S.rows = rows;
+    p64::stage(S, sh, dyn, smem_bytes, nc);
+    unsigned int gen = 0u;
+    double* rec[2] = {scratch, scratch + 4 * (size_t)kNoallocMaxRows};
+    int cur = 0;   // the buffer of the next product
+    int row[U];
+    double x[U], r[U], p[U], q[U], di[U], sm[U];
+    double v0 = 0.0, v1 = 0.0, v2 = threadIdx.x == 0 && sh.bad ? 1.0 : 0.0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {   // x = 0, r = b; z = D^-1 r published; b.b, r.z
+        const int i = grp + groups * u;
+        row[u] = warp < ncw && i < nc ? S.row(i, lane) : -1;
+        x[u] = r[u] = p[u] = q[u] = di[u] = sm[u] = 0.0;
+        if (row[u] < 0) continue;
+        r[u] = S.b[comp * S.n + row[u]];
+        di[u] = 1.0 / S.diag[row[u]];
+        const double z = di[u] * r[u];
+        v0 = fma(r[u], r[u], v0);
+        v1 = fma(r[u], z, v1);
+        rec[0][4 * (size_t)row[u] + comp] = z;
     }
-    if (na_publish<2>(v, W.partials, &W.st->ticket) && threadIdx.x == 0) {
-        NaState* st = W.st;
-        st->bnorm2 = v[0];
-        st->rho = v[1];
-        st->rr = v[0];
-        st->iter = 0;
-        st->restarts = 0;
-        st->check_true = 0;
-        st->status = SP_OK;
-        st->last_res = 0.0;
-        st->done = (v[0] == 0.0) ? 1 : 0;
-        if (!std::isfinite(v[0])) {
-            st->status = SP_ERR_NONFINITE;
-            st->done = 1;
+    auto publish = [&](int u, double v) { rec[cur ^ 1][4 * (size_t)row[u] + comp] = v; };
+    enum { kStart, kDirection, kUpdate, kX, kTrue };   // the values the next reduction carries (kX: none)
+    int phase = kStart;
+    auto product = [&] {   // sum_j alpha w_ij of the published vector
+        if (phase == kDirection || sh.bad) return;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int i = grp + groups * u;
+            if (i < nc) sm[u] = p64::row_product<KB>(S, sh, dyn, cap, i, row[u], rec[cur], comp);
         }
-    }
-}
-
-// q = A p; p.q; alpha = rho / p.q.
-__global__ void k_na_spmv(NaSystem S, NaPtrs W)
-{
-    NaState* st = W.st;
-    if (st->done) return;
-    double v[1] = {0.0};
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < S.n; i += gridDim.x * blockDim.x) {
-        double q3[3];
-        na_row_apply(S, W.p, i, q3);
-        for (int c = 0; c < 3; ++c) {
-            W.q[c * kPlane + i] = q3[c];
-            v[0] += W.p[c * kPlane + i] * q3[c];
+    };
+    auto scalars = [&] {   // one thread per block, the same totals in every block
+        const double t0 = sh.tot[0], t1 = sh.tot[1];
+        sh.action = 0;
+        sh.beta = 0.0;
+        if (phase == kStart) {
+            cg.bnorm2 = t0;
+            cg.rho = t1;
+            if (sh.tot[2] != 0.0) {
+                cg.status = SP_ERR_INVALID_ARG;
+                sh.action = 2;
+            } else if (!isfinite(t0)) {
+                cg.status = SP_ERR_NONFINITE;
+                sh.action = 2;
+            } else if (t0 == 0.0) {
+                sh.action = 2;   // b = 0: x = 0
+            }
+        } else if (phase == kDirection) {   // p.q
+            if (!(t0 > 0.0) || !isfinite(t0)) {
+                cg.status = SP_ERR_NONFINITE;
+                sh.action = 2;
+            } else {
+                sh.alpha = cg.rho / t0;
+            }
+        } else if (phase == kUpdate) {      // r.r, r.z
+            ++cg.iter;
+            if (!isfinite(t0)) {
+                cg.status = SP_ERR_NONFINITE;
+                sh.action = 2;
+            } else if (t0 <= S.tol2 * cg.bnorm2 || cg.iter >= S.max_iter) {
+                sh.action = 1;   // the true residual decides
+            } else {
+                sh.beta = t1 / cg.rho;
+                cg.rho = t1;
+            }
+        } else {                            // the true residual's r.r, r.z
+            cg.last_res = sqrt(t0 / cg.bnorm2);
+            if (t0 <= S.tol2 * cg.bnorm2) {
+                sh.action = 2;
+            } else if (cg.iter >= S.max_iter || cg.restarts >= kMaxCgRestarts) {
+                cg.status = SP_ERR_NOT_CONVERGED;
+                sh.action = 2;
+            } else {
+                ++cg.restarts;
+                cg.rho = t1;
+            }
         }
-    }
-    if (na_publish<1>(v, W.partials, &st->ticket) && threadIdx.x == 0) {
-        if (!(v[0] > 0.0) || !std::isfinite(v[0])) {
-            st->status = SP_ERR_NONFINITE;
-            st->done = 1;
-        } else {
-            st->alpha = st->rho / v[0];
-        }
-    }
-}
-
-// x += alpha p; r -= alpha q; z = D^-1 r; r.r, r.z; beta; the recurrence test.
-__global__ void k_na_update(NaSystem S, NaPtrs W)
-{
-    NaState* st = W.st;
-    if (st->done) return;
-    const double a = st->alpha;
-    double v[2] = {0.0, 0.0};
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < S.n; i += gridDim.x * blockDim.x) {
-        const double di = W.dinv[i];
-        for (int c = 0; c < 3; ++c) {
-            S.x[c * S.n + i] += a * W.p[c * kPlane + i];
-            const double rk = W.r[c * kPlane + i] - a * W.q[c * kPlane + i];
-            W.r[c * kPlane + i] = rk;
-            W.z[c * kPlane + i] = di * rk;
-            v[0] += rk * rk;
-            v[1] += di * rk * rk;
-        }
-    }
-    if (na_publish<2>(v, W.partials, &st->ticket) && threadIdx.x == 0) {
-        st->iter += 1;
-        st->rr = v[0];
-        st->beta = v[1] / st->rho;
-        st->rho = v[1];
-        if (!std::isfinite(v[0])) {
-            st->status = SP_ERR_NONFINITE;
-            st->done = 1;
-        } else if (v[0] <= S.tol2 * st->bnorm2 || st->iter >= S.max_iter) {
-            st->check_true = 1;
-        }
-    }
-}
-
-// When armed: r = b - A x exactly, accept or restart (beta = 0); then p = z + beta p.
-__global__ void k_na_check(NaSystem S, NaPtrs W)
-{
-    NaState* st = W.st;
-    if (st->done || !st->check_true) return;
-    double v[2] = {0.0, 0.0};
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < S.n; i += gridDim.x * blockDim.x) {
-        // A x with x in the caller's planes (plane stride n)
-        double ax[3];
-        const double x3[3] = {S.x[i], S.x[S.n + i], S.x[2 * S.n + i]};
-        double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-        for (int k = S.row_ptr[i]; k < S.row_ptr[i + 1]; ++k) {
-            const long long j = S.col[k];
-            const double w = S.w[k];
-            s0 += w * S.x[j];
-            s1 += w * S.x[S.n + j];
-            s2 += w * S.x[2 * S.n + j];
-        }
-        const double d = S.diag[i];
-        ax[0] = d * x3[0] - S.alpha * s0;
-        ax[1] = d * x3[1] - S.alpha * s1;
-        ax[2] = d * x3[2] - S.alpha * s2;
-        const double di = W.dinv[i];
-        for (int c = 0; c < 3; ++c) {
-            const double rk = S.b[c * S.n + i] - ax[c];
-            W.r[c * kPlane + i] = rk;
-            W.z[c * kPlane + i] = di * rk;
-            v[0] += rk * rk;
-            v[1] += di * rk * rk;
+    };
+    for (;;) {
+        const int K = phase == kX ? 0 : (phase == kStart ? 3 : (phase == kDirection ? 1 : 2));
+        if (!p64::reduce_overlapped(G, sh, gen, K, v0, v1, v2, product, scalars)) break;
+        if (K > 0 && sh.action == 2) break;
+        v0 = v1 = v2 = 0.0;
+        if (phase == kX) {   // r = b - A x
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (row[u] < 0) continue;
+                r[u] = S.b[comp * S.n + row[u]] - (S.diag[row[u]] * x[u] - sm[u]);
+                const double z = di[u] * r[u];
+                v0 = fma(r[u], r[u], v0);
+                v1 = fma(r[u], z, v1);
+                publish(u, z);
+            }
+            cur ^= 1;
+            phase = kTrue;
+        } else if (phase == kDirection) {   // x += alpha p; r -= alpha q; z published
+            const double a = sh.alpha;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (row[u] < 0) continue;
+                r[u] = fma(-a, q[u], r[u]);
+                const double z = di[u] * r[u];
+                publish(u, z);
+                x[u] = fma(a, p[u], x[u]);
+                v0 = fma(r[u], r[u], v0);
+                v1 = fma(r[u], z, v1);
+            }
+            cur ^= 1;
+            phase = kUpdate;
+        } else if (sh.action == 1) {        // the true residual: x published
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (row[u] >= 0) publish(u, x[u]);
+            cur ^= 1;
+            phase = kX;
+        } else {                            // q = A z + beta q (A_ii z = r); p = z + beta p
+            const double beta = sh.beta;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (row[u] < 0) continue;
+                q[u] = fma(beta, q[u], r[u] - sm[u]);
+                p[u] = fma(beta, p[u], di[u] * r[u]);
+                v0 = fma(p[u], q[u], v0);
+            }
+            phase = kDirection;
         }
     }
-    if (na_publish<2>(v, W.partials, &st->ticket) && threadIdx.x == 0) {
-        st->check_true = 0;
-        st->last_res = st->bnorm2 > 0.0 ? sqrt(v[0] / st->bnorm2) : 0.0;
-        if (v[0] <= S.tol2 * st->bnorm2) {
-            st->done = 1;
-        } else if (st->iter >= S.max_iter || st->restarts >= kMaxCgRestarts) {
-            st->status = SP_ERR_NOT_CONVERGED;
-            st->done = 1;
-        } else {
-            st->restarts += 1;
-            st->rho = v[1];
-            st->beta = 0.0;
-        }
+    if (cg.status != SP_ERR_INVALID_ARG) {
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (row[u] >= 0) S.x[comp * S.n + row[u]] = x[u];
     }
-}
-
-__global__ void k_na_direction(NaSystem S, NaPtrs W)
-{
-    const NaState* st = W.st;
-    if (st->done) return;
-    const double beta = st->beta;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < S.n; i += gridDim.x * blockDim.x)
-        for (int c = 0; c < 3; ++c) W.p[c * kPlane + i] = W.z[c * kPlane + i] + beta * W.p[c * kPlane + i];
+    if (G.bid == 0 && threadIdx.x == 0) {
+        st->bnorm2 = cg.bnorm2;
+        st->last_res = cg.last_res;
+        st->iter = cg.iter;
+        st->status = cg.status;
+        st->done = 1;
+    }
+    p64::leave(G);
 }
 
 std::mutex g_na_mutex;
@@ -351,28 +356,45 @@ extern "C" int sp_solve_csr_noalloc(int32_t device, void* stream, int64_t n, con
         }
         base = g_na_base[device];
     }
-    NaPtrs Wp = carve(static_cast<unsigned char*>(base));
-    NaSystem S{n, row_ptr_dev, col_dev, w_dev, diag_dev, alpha, b_dev, x_dev, tol * tol, max_iter};
+    double* scratch = static_cast<double*>(base);
+    NaSystem S{n, row_ptr_dev, col_dev, w_dev, diag_dev, alpha, b_dev, x_dev, tol * tol, max_iter, nullptr};
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // the state (and the reduction ticket) must start at zero on every call
-    if (cudaMemsetAsync(Wp.st, 0, sizeof(NaState), s) != cudaSuccess) return finish(SP_ERR_CUDA, "cudaMemsetAsync");
-    const int grid = (int)std::min<long long>(kNaBlocks, (n + kNaThreads - 1) / kNaThreads);
-    k_na_validate<<<grid, kNaThreads, 0, s>>>(S, Wp);
-    k_na_init<<<grid, kNaThreads, 0, s>>>(S, Wp);
+    NaState* st = reinterpret_cast<NaState*>(scratch + kRecordDoubles + kPartialDoubles);
+    int num_sms = 1;
+    if (cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
+        return finish(SP_ERR_CUDA, "cudaDeviceGetAttribute");
+    p64::Shape sp = p64::shape_of((int)((n + 31) / 32), std::min(num_sms, kNaMaxBlocks), 16);
+    const void* fn = sp.u == 1 ? (const void*)k_na_solve<1, 12>
+                               : (sp.u == 2 ? (const void*)k_na_solve<2, 8>
+                                            : (sp.u == 4 ? (const void*)k_na_solve<4, 6> : (const void*)k_na_solve<16, 4>));
+    if (sp.u == 0) {
+        err = "sp_solve_csr_noalloc: too few SMs for this system";
+        return finish(SP_ERR_CUDA, nullptr);
+    }
+    // the state (and the grid barriers' counters) must start at zero on every call
+    if (cudaMemsetAsync(st, 0, sizeof(NaState), s) != cudaSuccess) return finish(SP_ERR_CUDA, "cudaMemsetAsync");
+    if (sp.smem > 32 * 1024 &&   // with the static arrays, near the 48 KB a kernel has by default
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, sp.smem) != cudaSuccess)
+        return finish(SP_ERR_CUDA, "cudaFuncSetAttribute");
+    unsigned long long limit_ns = kDefaultWaitLimitNs;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)sp.blocks);
+    cfg.blockDim = dim3((unsigned)sp.threads);
+    cfg.dynamicSmemBytes = (size_t)sp.smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    void* args[] = {&S, &scratch, &sp.smem, &limit_ns};
+    if (cudaLaunchKernelExC(&cfg, fn, args) != cudaSuccess) return finish(SP_ERR_CUDA, "launching the solve");
     NaState h;
     std::memset(&h, 0, sizeof(h));
-    for (int it = 0; it < max_iter + kMaxCgRestarts + 8; it += 8) {
-        for (int k = 0; k < 8; ++k) {
-            k_na_spmv<<<grid, kNaThreads, 0, s>>>(S, Wp);
-            k_na_update<<<grid, kNaThreads, 0, s>>>(S, Wp);
-            k_na_check<<<grid, kNaThreads, 0, s>>>(S, Wp);
-            k_na_direction<<<grid, kNaThreads, 0, s>>>(S, Wp);
-        }
-        if (cudaMemcpyAsync(&h, Wp.st, sizeof(NaState), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaStreamSynchronize(s) != cudaSuccess)
-            return finish(SP_ERR_CUDA, "reading the solver state");
-        if (h.done) break;
-    }
+    if (cudaMemcpyAsync(&h, st, sizeof(NaState), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess)
+        return finish(SP_ERR_CUDA, "reading the solver state");
+    if (h.error != 0) h.status = h.error;
     int status = h.done ? h.status : SP_ERR_NOT_CONVERGED;
     if (info) {
         info->status = status;
@@ -386,6 +408,8 @@ extern "C" int sp_solve_csr_noalloc(int32_t device, void* stream, int64_t n, con
     else if (status == SP_ERR_NOT_CONVERGED)
         err = "sp_solve_csr_noalloc: not converged (max_iter reached, or the true residual stayed above tol "
               "after the restart limit)";
+    else if (status == SP_ERR_TIMEOUT)
+        err = "sp_solve_csr_noalloc: a grid-barrier wait ran past its limit";
     else if (status != SP_OK)
         err = "sp_solve_csr_noalloc: solve failed";
     return finish(status, nullptr);
