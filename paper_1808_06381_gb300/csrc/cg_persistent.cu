@@ -2009,16 +2009,24 @@ done:
 // form with four lanes per row and vectors in memory -> this one: n = 500, 8
 // -> 16 blocks: 14.1 -> 5.9 us; n = 4,096, 64 -> 128 blocks: 15.2 -> 6.7 us; n
 // = 60,013: 44 -> 24 us (there the gathers' L1 wavefronts and the FP64 issue).
-struct SellSystem64 {   // the sliced layout as pcg64's system
+template <class V>
+struct SellSystem {   // the sliced layout as pcg64's system, with the FP64 or the FP32 weights
+    using Value = V;
     const KParams& P;
     const DevBuffers& B;
     int bid, nb;
+    bool run;
+    __device__ int chunks() const
+    {
+        if (run) return (int)((long long)(bid + 1) * P.nchunks / nb) - (int)((long long)bid * P.nchunks / nb);
+        return (P.nchunks - bid + nb - 1) / nb;
+    }
     struct Entries {
         const int* col;
-        const double* val;
+        const V* val;
         int cnt;
         __device__ bool valid() const { return true; }
-        __device__ void get(int k, int& j, double& w) const
+        __device__ void get(int k, int& j, V& w) const
         {
             if (k < cnt) {
                 j = __ldg(col + 32 * k);
@@ -2026,15 +2034,33 @@ struct SellSystem64 {   // the sliced layout as pcg64's system
             }
         }
     };
-    __device__ double alpha() const { return P.alpha; }
+    __device__ V alpha() const { return (V)P.alpha; }
     __device__ bool in_range(int) const { return true; }
-    __device__ int chunk(int i) const { return bid + nb * i; }
+    // chunk i of the block: a run of neighbouring chunks (run), or chunk bid +
+    // nb i of the windows' chunks with their order rotated from window to window
+    // (a window's chunks hold rows of decreasing length; unrotated, 8 | nb would
+    // give a block the same rank in every window).  The strided form shares a
+    // dense region's long rows out among the blocks; a run of at least a window
+    // holds every rank anyway, and its rows' partners are largely the same rows,
+    // so an FP32 product, bound by its gathers, finds more of them in L1 (mixed
+    // solve, strided against runs: n = 33,000 0.39 / 0.47 ms, n = 48,000 0.455 /
+    // 0.426, n = 100,000 0.84 / 0.74; FP64, n = 60,013: 1.42 / 1.54).
+    __device__ int chunk(int i) const
+    {
+        if (run) return (int)((long long)bid * P.nchunks / nb) + i;
+        const int q = bid + nb * i, w = q >> 3;
+        return (q & ~7) | ((q + 3 * w + (w >> 4)) & 7);
+    }
     __device__ int row(int i, int lane) const { return B.slot_row[32 * chunk(i) + lane]; }
     __device__ int chunk_len(int i, int) const { return (B.chunk_off[chunk(i) + 1] - B.chunk_off[chunk(i)]) >> 5; }
     __device__ Entries entries(int i, int lane, int row) const
     {
         const int e = B.chunk_off[chunk(i)];
-        return Entries{B.col + e + lane, B.val + e + lane, row < 0 ? 0 : (B.chunk_off[chunk(i) + 1] - e) >> 5};
+        const int cnt = row < 0 ? 0 : (B.chunk_off[chunk(i) + 1] - e) >> 5;
+        if constexpr (sizeof(V) == sizeof(double))
+            return Entries{B.col + e + lane, B.val + e + lane, cnt};
+        else
+            return Entries{B.col + e + lane, B.val32 + e + lane, cnt};
     }
 };
 
@@ -2049,12 +2075,12 @@ __device__ __forceinline__ void pipelined_solve64(const KParams& P, const DevBuf
                                                   int smem_bytes, int from_x)
 {
     DevState* st = B.st;
-    const SellSystem64 S{P, B, G.bid, G.nb};
+    const SellSystem<double> S{P, B, G.bid, G.nb, false};
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, np = P.npad;
     const int ncw = (blockDim.x >> 5) - p64::kScalarWarps, groups = ncw / 3;
     const int grp = warp / 3, comp = warp - 3 * grp;
-    const int nc = (P.nchunks - G.bid + G.nb - 1) / G.nb;   // chunks bid, bid + nb, ...
-    const int cap = smem_bytes / p64::kEntryBytes;
+    const int nc = S.chunks();
+    const int cap = smem_bytes / p64::kEntryBytes<double>;
     if (threadIdx.x == 0) {
         sh.flag = 0;
         sh.action = 0;
@@ -2235,6 +2261,309 @@ __global__ void __launch_bounds__(p64::max_threads(U), 1) k64_cg_pipelined(KPara
     p64::leave(G);
 }
 
+// The mixed solve of small systems: the same pipelined iteration on chip in
+// FP32, one row per thread (lane = row; FP32 issues at full rate, so a row's
+// three components stay in one thread and an entry costs one 16-byte gather),
+// inside the mixed solver's residual replacements: x += d in double-float, r =
+// b - A x in double-float from the sliced layout, after every reduction of the
+// recursive residual by 10^-4 (KParams::inner2) and at the end.  The sums
+// behind the scalars are FP64 from the row products on.  Bound by the barrier
+// (~2.3 us) and the gathers' latency.  Measured (whole solve of a clustered
+// system to 1e-8; streaming form / k32_cg_resident / this one): n = 500 0.52 /
+// 0.33 / 0.19 ms, n = 20,011 1.02 / 0.75 / 0.38, n = 48,000 1.03 / 0.69 / 0.43,
+// n = 72,960 1.12 / 0.80 / 0.54, n = 100,000 1.13 / 0.84 / 0.79, n = 145,000
+// 1.20 / 0.92 / 1.04 (there its gathers, which k32_cg_resident serves from
+// shared memory).
+template <int KB, class Sys>
+__device__ __forceinline__ void row_product32(const Sys& S, const p64::Shared& sh, const unsigned char* dyn, int cap,
+                                              int i, int row, const float4* m, float (&s)[3])
+{
+    const int lane = threadIdx.x & 31, len = sh.len[i], off = sh.off[i];
+    s[0] = s[1] = s[2] = 0.f;
+    if (off >= 0) {
+        const float* val = reinterpret_cast<const float*>(dyn) + off + lane;
+        const int* col = reinterpret_cast<const int*>(dyn + sizeof(float) * (size_t)cap) + off + lane;
+        for (int kb = 0; kb < len; kb += KB) {
+            float4 g[KB];
+#pragma unroll
+            for (int u = 0; u < KB; ++u)
+                g[u] = kb + u < len ? m[col[32 * (kb + u)]] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int u = 0; u < KB; ++u) {
+                const float w = kb + u < len ? val[32 * (kb + u)] : 0.f;
+                s[0] = fmaf(w, g[u].x, s[0]);
+                s[1] = fmaf(w, g[u].y, s[1]);
+                s[2] = fmaf(w, g[u].z, s[2]);
+            }
+        }
+        return;
+    }
+    if (row < 0) return;
+    const auto at = S.entries(i, lane, row);
+    for (int kb = 0; kb < len; kb += KB) {
+        int j[KB];
+        float w[KB];
+        float4 g[KB];
+#pragma unroll
+        for (int u = 0; u < KB; ++u) {
+            j[u] = 0;
+            w[u] = 0.f;
+            if (kb + u < len) at.get(kb + u, j[u], w[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < KB; ++u) g[u] = w[u] != 0.f ? m[j[u]] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < KB; ++u) {
+            const float wa = S.alpha() * w[u];
+            s[0] = fmaf(wa, g[u].x, s[0]);
+            s[1] = fmaf(wa, g[u].y, s[1]);
+            s[2] = fmaf(wa, g[u].z, s[2]);
+        }
+    }
+}
+
+struct Cg32Scalars {
+    double bnorm2, rr_restart, target, last_res;
+    float rho, den, alpha, beta;
+    int iter, restarts, status, first;
+};
+
+template <int U, int KB>
+__device__ __forceinline__ void pipelined_solve32(const KParams& P, const DevBuffers& B, const p64::Grid& G,
+                                                  p64::Shared& sh, Cg32Scalars& cg, unsigned char* dyn,
+                                                  int smem_bytes)
+{
+    DevState* st = B.st;
+    const SellSystem<float> S{P, B, G.bid, G.nb, P.nchunks >= 8 * G.nb};
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, np = P.npad;
+    const int ncw = (blockDim.x >> 5) - p64::kScalarWarps;
+    const int nc = S.chunks();
+    const int cap = smem_bytes / p64::kEntryBytes<float>;
+    const bool from_x = P.fused_init == 2;
+    if (threadIdx.x == 0) {
+        sh.flag = 0;
+        sh.action = 0;
+        cg.status = SP_OK;
+        cg.iter = cg.restarts = 0;
+        cg.last_res = 0.0;
+    }
+    p64::stage(S, sh, dyn, smem_bytes, nc);
+    unsigned int gen = 0u;
+    float4* rec[2] = {B.p4, B.q4};
+    int cur = 1;   // the buffer of the next product (the first publication goes to the other)
+    int row[U] = {};
+    float r[U][3], w[U][3], z[U][3], s[U][3], p[U][3], d[U][3], sm[U][3], di[U] = {};
+    double v0 = 0.0, v1 = 0.0, v2 = 0.0;
+    auto publish = [&](int u, const float (&v)[3]) {
+        rec[cur ^ 1][row[u]] = make_float4(di[u] * v[0], di[u] * v[1], di[u] * v[2], 0.f);
+    };
+    // r = b - A x of the own rows in double-float, u = D^-1 r published; ||r||^2 into v0
+    auto residual = [&](bool product) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (row[u] < 0) continue;
+            const int slot = 32 * S.chunk(warp + ncw * u) + lane;
+            dfloat sd[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}}, rd[3];
+            if (product)
+                row_sum_df<4>(B.col, B.val32, B.val32lo, B.xdf, B.chunk_off[slot >> 5] + lane,
+                              B.chunk_off[(slot >> 5) + 1], sd);
+            residual_df(P, B, row[u], sd, rd);
+            float rs = 0.f;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                r[u][c] = rd[c].hi;
+                d[u][c] = 0.f;
+                rs += r[u][c] * r[u][c];
+            }
+            v0 += (double)rs;
+            publish(u, r[u]);
+        }
+        cur ^= 1;
+    };
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int i = warp + ncw * u;
+        row[u] = warp < ncw && i < nc ? S.row(i, lane) : -1;
+        di[u] = row[u] >= 0 ? B.dinv32[row[u]] : 0.f;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) r[u][c] = w[u][c] = z[u][c] = s[u][c] = p[u][c] = d[u][c] = sm[u][c] = 0.f;
+        if (row[u] < 0) continue;
+        const float4 bh = B.bdf[2 * row[u]];
+        v1 += (double)(bh.x * bh.x + bh.y * bh.y + bh.z * bh.z);
+        if (!from_x) {
+            B.xdf[2 * row[u]] = B.xdf[2 * row[u] + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) B.x[c * np + row[u]] = 0.0;
+        }
+    }
+    if (threadIdx.x == 0)   // blocks that read a chunk's entries from memory
+        for (int i = 0; i < nc; ++i)
+            if (sh.off[i] < 0) v2 = 1.0;
+    residual(from_x);
+    enum { kStart, kIterate, kX, kTrue };   // the values the next reduction carries (kX: none, x was folded)
+    int phase = kStart;
+    auto product = [&] {   // sum_j alpha w_ij of the published vector
+        if (phase == kX) return;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int i = warp + ncw * u;
+            if (i < nc) row_product32<KB>(S, sh, dyn, cap, i, row[u], rec[cur], sm[u]);
+        }
+    };
+    auto scalars = [&] {   // one thread per block, the same totals in every block
+        sh.action = 0;
+        if (phase == kIterate) {
+            const double g = sh.tot[0], dl = sh.tot[1], rr = sh.tot[2];
+            if (!isfinite(g) || !isfinite(dl) || !isfinite(rr)) {
+                cg.status = SP_ERR_NONFINITE;
+                sh.action = 2;
+            } else if (rr <= cg.target || cg.iter >= P.max_iter) {
+                sh.action = 1;   // the true residual decides
+            } else {
+                const float gf = (float)g, df = (float)dl;
+                const float beta = cg.first ? 0.f : gf / cg.rho;
+                const float den = cg.first ? df : fmaf(-beta * beta, cg.den, df);   // (p, A p) of the new direction
+                if (!(den > 0.f)) {
+                    sh.action = 1;   // lost to rounding: the true residual decides
+                } else {
+                    cg.beta = beta;
+                    cg.alpha = gf / den;
+                    cg.rho = gf;
+                    cg.den = den;
+                    cg.first = 0;
+                    ++cg.iter;
+                }
+            }
+            return;
+        }
+        const double rr = sh.tot[0];
+        if (phase == kStart) {
+            cg.bnorm2 = sh.tot[1];
+            cg.last_res = 1.0;
+            if (!isfinite(cg.bnorm2) || !isfinite(rr)) {
+                cg.status = SP_ERR_NONFINITE;
+                sh.action = 2;
+            } else if (cg.bnorm2 == 0.0) {
+                sh.action = 2;   // b = 0: the solution is v = 0 (written by the finishing kernel)
+                cg.last_res = 0.0;
+            } else if (rr <= P.tol2 * cg.bnorm2) {
+                sh.action = 2;   // x0 already meets the tolerance
+                cg.last_res = sqrt(rr / cg.bnorm2);
+            }
+            if (G.bid == 0) {
+                st->bnorm2 = cg.bnorm2;
+                st->zero_b = (isfinite(cg.bnorm2) && cg.bnorm2 == 0.0) ? 1 : 0;
+                st->res_offchip = (int)sh.tot[2];
+            }
+        } else {
+            cg.last_res = sqrt(rr / cg.bnorm2);
+            if (G.bid == 0) st->true_checks += 1;
+            if (!isfinite(rr)) {
+                cg.status = SP_ERR_NONFINITE;
+                sh.action = 2;
+            } else if (rr <= P.tol2 * cg.bnorm2) {
+                sh.action = 2;   // converged
+            } else if (cg.iter >= P.max_iter || cg.restarts >= kMaxCgRestarts + 8) {
+                cg.status = SP_ERR_NOT_CONVERGED;
+                sh.action = 2;
+            } else {
+                ++cg.restarts;
+            }
+        }
+        cg.first = 1;
+        cg.target = fmax(P.inner2 * rr, kInnerFinal2 * P.tol2 * cg.bnorm2);
+    };
+    for (;;) {
+        const int K = phase == kX ? 0 : (phase == kTrue ? 1 : 3);
+        if (!p64::reduce_overlapped(G, sh, gen, K, v0, v1, v2, product, scalars)) break;
+        if (K > 0 && sh.action == 2) break;
+        v0 = v1 = v2 = 0.0;
+        if (phase == kX) {
+            residual(true);
+            phase = kTrue;
+            continue;
+        }
+        if (phase == kIterate && sh.action == 1) {   // x += d (own rows)
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (row[u] >= 0) fold_correction(B, row[u], make_float4(d[u][0], d[u][1], d[u][2], 0.f));
+            phase = kX;
+            continue;
+        }
+        const bool start = phase != kIterate;   // w = A u (A_ii u = r); else the recurrences
+        const float a = cg.alpha, beta = cg.beta;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (row[u] < 0) continue;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                if (start) {
+                    w[u][c] = r[u][c] - sm[u][c];
+                    z[u][c] = s[u][c] = p[u][c] = 0.f;
+                } else {   // n = A m = w - sum (A_ii D^-1_ii = 1)
+                    z[u][c] = fmaf(beta, z[u][c], w[u][c] - sm[u][c]);
+                    s[u][c] = fmaf(beta, s[u][c], w[u][c]);
+                    w[u][c] = fmaf(-a, z[u][c], w[u][c]);
+                }
+            }
+            publish(u, w[u]);
+            float g = 0.f, dl = 0.f, rr = 0.f;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                if (!start) {
+                    p[u][c] = fmaf(beta, p[u][c], di[u] * r[u][c]);
+                    d[u][c] = fmaf(a, p[u][c], d[u][c]);
+                    r[u][c] = fmaf(-a, s[u][c], r[u][c]);
+                }
+                const float uk = di[u] * r[u][c];
+                g = fmaf(r[u][c], uk, g);
+                dl = fmaf(w[u][c], uk, dl);
+                rr = fmaf(r[u][c], r[u][c], rr);
+            }
+            v0 += (double)g;
+            v1 += (double)dl;
+            v2 += (double)rr;
+        }
+        cur ^= 1;
+        phase = kIterate;
+    }
+    if (cg.iter > 0) {   // a solve that met the tolerance at x0 keeps x0 as it was
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (row[u] >= 0) store_x64(B, np, row[u]);
+    }
+    if (G.bid == 0 && threadIdx.x == 0) {
+        st->iter = cg.iter;
+        st->restarts = cg.restarts;
+        st->last_res = cg.last_res;
+        st->done = 1;
+        if (st->error == 0 && cg.status != SP_OK) {
+            st->status = cg.status;
+            st->error = cg.status;
+        } else if (st->error != 0) {
+            st->status = st->error;
+        } else {
+            st->status = SP_OK;
+        }
+    }
+}
+
+constexpr int kSmall32Warps = 15;   // chunks in flight of a block (one warp each)
+template <int U, int KB>
+__global__ void __launch_bounds__(32 * (kSmall32Warps + p64::kScalarWarps), 1)
+    k32_cg_pipelined(KParams P, DevBuffers B, int smem_bytes)
+{
+    extern __shared__ float4 res_dyn[];
+    __shared__ p64::Shared sh;
+    __shared__ Cg32Scalars cg;
+    DevState* st = B.st;
+    const p64::Grid G{&st->bar_count, &st->bar_exit, &st->error, st->bar_timeout_ns, B.partials, kMaxPartials,
+                      (int)blockIdx.x, (int)gridDim.x};
+    if (!(st->error | st->overflow))   // uniform: set before the launch
+        pipelined_solve32<U, KB>(P, B, G, sh, cg, reinterpret_cast<unsigned char*>(res_dyn), smem_bytes);
+    p64::leave(G);
+}
+
 __global__ void __launch_bounds__(512, 1) k64_cg_persistent(KParams P, DevBuffers B, int from_x)
 {
     __shared__ PShared sh;
@@ -2307,6 +2636,10 @@ PCfg g_pcfg[kPersistentConfigs] = {   // entry 0: the default without autotuning
     {4, 1, 0, 512, (const void*)k32_cg_persistent<4, 1, false, 512, true>, 0, 0, 1},
     {4, 3, 0, 256, (const void*)k32_cg_persistent<4, 3, false, 256, true>, 0, 0, 1},
 };
+constexpr int kResidentConfig = 9;    // the on-chip solve that a system without a chosen configuration takes
+constexpr int kSmall32ChunkSmem = 7 * 1024;   // shared memory planned per chunk (28 entries a row)
+constexpr int kSmall32SpareSmem = 48 * 1024;
+constexpr int kSmall32MaxChunks = 24; // chunks of 32 rows per SM up to which the on-chip configurations run pipelined
 struct BCfg {
     int kb, minb, bs;
     const void* fn;
@@ -2357,13 +2690,40 @@ bool resident_fits(const PCfg& c, const KParams& P, const DevBuffers& B, Launch 
     return g >= 1 && g <= L.num_sms && (P.nslots / 256 + g - 1) / g <= kResWindows;
 }
 
+// The on-chip form of small systems (k32_cg_pipelined): blocks, threads and
+// chunks a thread; u = 0 where the system is larger.
+p64::Shape small32_shape(const KParams& P, Launch L)
+{
+    const int nch = std::max(P.nchunks, 1), c = (nch + L.num_sms - 1) / L.num_sms;
+    p64::Shape s{};
+    if (c > kSmall32MaxChunks) return s;
+    s.u = c <= kSmall32Warps ? 1 : 2;
+    s.blocks = (nch + c - 1) / c;
+    s.threads = 32 * ((c + s.u - 1) / s.u + p64::kScalarWarps);
+    s.smem = std::min(c * kSmall32ChunkSmem + kSmall32SpareSmem, p64::kMaxSmem);
+    return s;
+}
+
 // The configuration a launch uses: the chosen one, or entry 0 where the
-// chosen one is the on-chip solve and the system does not fit it.
+// chosen one is the on-chip solve and the system does not fit it.  Without a
+// choice (pcfg < 0): on chip where the system fits and the entries of a
+// uniform configuration of this density, half as many again for clustering,
+// fit beside the rows' records (else many chunks would be gathered from
+// memory, where the streaming form is the faster one).  Solve, streaming entry
+// 0 against on chip: n = 145,000 1.20 / 0.92 ms, n = 262,144 1.58 / 1.23, n =
+// 311,000 1.62 / 1.45; smaller systems at k32_cg_pipelined.
 const PCfg& cfg_of(const KParams& P, const DevBuffers& B, Launch L)
 {
     pocc_init();
-    const int k = (P.pcfg >= 0 && P.pcfg < kPersistentConfigs) ? P.pcfg : 0;
-    if (g_pcfg[k].resident && !resident_fits(g_pcfg[k], P, B, L)) return g_pcfg[0];
+    if (P.pcfg < 0) {
+        const PCfg& r = g_pcfg[kResidentConfig];
+        if (small32_shape(P, L).u > 0) return r;
+        const double per_row = 4.18879 * P.rc2 * sqrt(P.rc2) * P.n / (P.L[0] * P.L[1] * P.L[2]);
+        const double rows = (double)P.n / (double)std::max<long long>(grid_of(r, P, L), 1);
+        return resident_fits(r, P, B, L) && rows * (16.0 + 4.0 * 1.5 * per_row) <= kResSmemBytes ? r : g_pcfg[0];
+    }
+    const int k = P.pcfg < kPersistentConfigs ? P.pcfg : 0;
+    if (g_pcfg[k].resident && small32_shape(P, L).u == 0 && !resident_fits(g_pcfg[k], P, B, L)) return g_pcfg[0];
     return g_pcfg[k];
 }
 }  // namespace
@@ -2425,7 +2785,7 @@ bool cg_persistent_usable(int k, const KParams& P, const DevBuffers& B, Launch L
 {
     pocc_init();
     if (k < 0 || k >= kPersistentConfigs || g_pcfg[k].occ < 1) return false;
-    return !g_pcfg[k].resident || resident_fits(g_pcfg[k], P, B, L);
+    return !g_pcfg[k].resident || small32_shape(P, L).u > 0 || resident_fits(g_pcfg[k], P, B, L);
 }
 
 bool cg_persistent_on_chip(const KParams& P, const DevBuffers& B, Launch L)
@@ -2435,7 +2795,12 @@ bool cg_persistent_on_chip(const KParams& P, const DevBuffers& B, Launch L)
 
 int cg_persistent_grid(const KParams& P, const DevBuffers& B, Launch L)
 {
-    return (int)grid_of(cfg_of(P, B, L), P, L);
+    const PCfg& c = cfg_of(P, B, L);
+    if (c.resident) {
+        const p64::Shape s = small32_shape(P, L);
+        if (s.u > 0) return s.blocks;
+    }
+    return (int)grid_of(c, P, L);
 }
 
 // FP64 solve in one launch.  Systems of up to 16 chunks of 32 rows per SM
@@ -2484,6 +2849,7 @@ int cg64_persistent_grid(const KParams& P, Launch L) { return cg64_shape(P, L).b
 cudaError_t launch_cg32_persistent(const KParams& P, DevBuffers& B, Launch L)
 {
     const PCfg& c = cfg_of(P, B, L);
+    const p64::Shape small = c.resident ? small32_shape(P, L) : p64::Shape{};
     const int g = (int)grid_of(c, P, L);
     if (g < 1) return cudaErrorCooperativeLaunchTooLarge;
     if (c.mf) {
@@ -2495,6 +2861,18 @@ cudaError_t launch_cg32_persistent(const KParams& P, DevBuffers& B, Launch L)
     cfg.blockDim = dim3((unsigned)c.bs);
     int smem = std::min(std::max(P.res_smem, 0), kResSmemBytes);
     cfg.dynamicSmemBytes = c.resident ? smem : 0;
+    const void* fn = c.fn;
+    if (small.u > 0) {
+        fn = small.u == 1 ? (const void*)k32_cg_pipelined<1, 10> : (const void*)k32_cg_pipelined<2, 6>;
+        smem = small.smem;
+        cfg.gridDim = dim3((unsigned)small.blocks);
+        cfg.blockDim = dim3((unsigned)small.threads);
+        cfg.dynamicSmemBytes = (size_t)smem;
+        if (smem > 32 * 1024) {
+            const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            if (e != cudaSuccess) return e;
+        }
+    }
     cfg.stream = L.stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
@@ -2502,7 +2880,7 @@ cudaError_t launch_cg32_persistent(const KParams& P, DevBuffers& B, Launch L)
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     void* args[] = {const_cast<KParams*>(&P), &B, &smem};
-    return cudaLaunchKernelExC(&cfg, c.fn, args);
+    return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
 }  // namespace ss

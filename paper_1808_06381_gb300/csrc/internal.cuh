@@ -56,7 +56,7 @@ struct KParams {
     float kap_hi, kap_lo;       // kappa
     float hly_hi, hly_lo;       // L_y / 2
     float akl_hi, akl_lo;       // alpha kappa L_y
-    int pcfg;           // tile configuration of the persistent solver (index, autotuned)
+    int pcfg;           // tile configuration of the persistent solver (index, autotuned; -1: chosen by the system)
     int res_smem;       // shared memory the on-chip solve uses (<= kResSmemBytes; less only to test its fallback)
     int fused_init;     // on-chip solve: 0 after the initial-residual kernel; 1 forms r = b itself (x0 = 0), 2 r = b - A x0
     long long hcopy;    // on-chip solve: where hcol / hval / hlo hold a second copy region (the lists of blocks

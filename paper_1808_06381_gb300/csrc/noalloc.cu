@@ -70,6 +70,7 @@ struct NaSystem {   // the caller's arrays, and pcg64's system
     double* x;
     double tol2;
     int max_iter;
+    using Value = double;
     const int* rows;   // the block's rows by length, in its shared memory (-1: none)
     struct Entries {
         const int* col;
@@ -128,7 +129,7 @@ __global__ void __launch_bounds__(p64::max_threads(U), 1) k_na_solve(NaSystem S,
     const int ncw = (blockDim.x >> 5) - p64::kScalarWarps, groups = ncw / 3;
     const int grp = warp / 3, comp = warp - 3 * grp;
     const int nch = (int)((S.n + 31) / 32), nc = (nch - G.bid + G.nb - 1) / G.nb;   // chunks bid, bid + nb, ...
-    const int cap = smem_bytes / p64::kEntryBytes;
+    const int cap = smem_bytes / p64::kEntryBytes<double>;
     if (threadIdx.x == 0) {
         sh.flag = 0;
         sh.action = 0;

@@ -1,6 +1,7 @@
-// FP64 conjugate gradients on chip: the building blocks shared by the solve
-// of small FP64 systems (cg_persistent.cu) and the allocation-free solve of a
-// caller's CSR system (noalloc.cu), both one cooperative launch.
+// Conjugate gradients on chip: the building blocks shared by the solves of
+// small FP64 and mixed systems (cg_persistent.cu) and the allocation-free solve
+// of a caller's CSR system (noalloc.cu), each one cooperative launch.  The
+// FP64 ones first:
 //
 // GB300 issues FP64 at 2 FMA per clock and SM, half an operation per clock on
 // each of its four schedulers, so one FP64 instruction of a warp holds its
@@ -35,8 +36,10 @@ constexpr int kMaxWarps = 3 * kMaxGroups;
 constexpr int kScalarWarps = 3;     // warps that sum the grid's partials, one value each
 // threads of a block whose threads hold u chunks (from u = 4 on four groups, so that 128 registers are left a thread)
 constexpr int max_threads(int u) { return 32 * ((u >= 4 ? 12 : kMaxWarps) + kScalarWarps); }
-constexpr int kEntryBytes = 12;     // alpha w (8) and column (4) of an entry in shared memory
-constexpr int kChunkSmem = 16 * 1024;        // shared memory planned per chunk (42 entries a row), one chunk spare
+// an entry in shared memory: alpha w (FP64, or FP32 in the mixed solve) and the column
+template <class V>
+constexpr int kEntryBytes = (int)sizeof(V) + 4;
+constexpr int kChunkSmem = 16 * 1024;        // shared memory planned per chunk (42 FP64 entries a row), one chunk spare
 constexpr int kMaxSmem = 200 * 1024;
 
 struct Grid {
@@ -124,7 +127,8 @@ __device__ __forceinline__ void stage(const Sys& S, Shared& sh, unsigned char* d
         if (lane == 0) sh.len[i] = len;
     }
     __syncthreads();
-    const int cap = smem_bytes / kEntryBytes;
+    using V = typename Sys::Value;
+    const int cap = smem_bytes / kEntryBytes<V>;
     if (threadIdx.x == 0) {
         int at = 0;
         for (int i = 0; i < nc; ++i) {
@@ -134,8 +138,8 @@ __device__ __forceinline__ void stage(const Sys& S, Shared& sh, unsigned char* d
         }
     }
     __syncthreads();
-    double* val = reinterpret_cast<double*>(dyn);
-    int* col = reinterpret_cast<int*>(dyn + 8 * (size_t)cap);
+    V* val = reinterpret_cast<V*>(dyn);
+    int* col = reinterpret_cast<int*>(dyn + sizeof(V) * (size_t)cap);
     constexpr int KS = 8;
     for (int i = warp; i < nc; i += nwarps) {
         const int row = S.row(i, lane), len = sh.len[i], off = sh.off[i];
@@ -144,11 +148,11 @@ __device__ __forceinline__ void stage(const Sys& S, Shared& sh, unsigned char* d
         bool bad = !at.valid();
         for (int kb = 0; kb < len; kb += KS) {
             int j[KS];
-            double w[KS];
+            V w[KS];
 #pragma unroll
             for (int u = 0; u < KS; ++u) {
                 j[u] = 0;
-                w[u] = 0.0;
+                w[u] = V(0);
                 if (kb + u < len) at.get(kb + u, j[u], w[u]);
             }
 #pragma unroll
@@ -156,11 +160,11 @@ __device__ __forceinline__ void stage(const Sys& S, Shared& sh, unsigned char* d
                 if (!S.in_range(j[u])) {
                     bad = true;
                     j[u] = 0;
-                    w[u] = 0.0;
+                    w[u] = V(0);
                 }
                 if (off >= 0 && kb + u < len) {
                     const int e = off + 32 * (kb + u) + lane;
-                    col[e] = w[u] != 0.0 ? j[u] : pad;
+                    col[e] = w[u] != V(0) ? j[u] : pad;
                     val[e] = S.alpha() * w[u];
                 }
             }

@@ -170,7 +170,7 @@ void derive(const sp_params& p, KParams& k, int npad)
     const double l2 = lambda2_of(p.rc);
     k.two_lambda2 = 2.0 * l2;
     k.w_scale = 256.0 / k.two_lambda2;
-    k.pcfg = 0;   // tile configuration of the persistent solver (sp_autotune)
+    k.pcfg = -1;   // no configuration chosen: by the system (sp_autotune, sp_set_solver_config choose one)
     k.res_smem = kResSmemBytes;
     k.alpha = p.alpha;
     k.mixed = p.precision == SP_PREC_MIXED ? 1 : 0;

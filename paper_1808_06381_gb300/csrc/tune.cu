@@ -82,7 +82,7 @@ extern "C" int sp_autotune(sp_sim* s, int32_t trials, sp_tune_info* info)
     auto finish = [&](int cfg) {
         s->kp.pcfg = cfg;
         free_graphs(s);   // captured graphs hold the previous configuration's kernel
-        out.config = cfg;
+        out.config = std::max(cfg, 0);   // no choice made (an FP64 simulation): entry 0
         cg_persistent_config(cfg, &out.gathers_in_flight, &out.blocks_per_sm, &out.pipelined, &out.block_threads,
                              &out.resident, &out.matrix_free);
         if (info) *info = out;
