@@ -95,11 +95,23 @@ __device__ __forceinline__ unsigned long long smem_desc(const void* base, int K)
            (1ull << 46);   // descriptor version 1; base offset 0, no swizzle
 }
 
-__host__ __device__ constexpr unsigned idesc_bf16(int M, int N)
+// The same with both strides given: K-major, lbo steps from one core matrix to
+// the next along K and sbo along the rows; MN-major (a transposed operand), lbo
+// steps along K (8 rows of the stored tile) and sbo along M or N.
+__device__ __forceinline__ unsigned long long smem_desc(const void* base, unsigned lbo, unsigned sbo)
+{
+    const unsigned long long addr = smem_addr(base);
+    return ((addr >> 4) & 0x3FFFull) | ((unsigned long long)(lbo >> 4) << 16) |
+           ((unsigned long long)(sbo >> 4) << 32) | (1ull << 46);
+}
+
+// mn_major: A and B are both stored transposed (MN-major) instead of K-major
+__host__ __device__ constexpr unsigned idesc_bf16(int M, int N, bool mn_major = false)
 {
     return (1u << 4)                  // D: FP32
            | (1u << 7) | (1u << 10)   // A, B: BF16
-           | ((unsigned)(N >> 3) << 17) | ((unsigned)(M >> 4) << 24);   // both K-major
+           | (mn_major ? (1u << 15) | (1u << 16) : 0u)
+           | ((unsigned)(N >> 3) << 17) | ((unsigned)(M >> 4) << 24);
 }
 
 __device__ __forceinline__ void mma(unsigned tmem_d, unsigned long long a, unsigned long long b, unsigned idesc,
@@ -295,47 +307,56 @@ __global__ void __launch_bounds__(128) k_mp_mlp_fwd_tc(int rows, MpBuffers M, De
 
 // ------------------------------------------ training backward on tcgen05
 //
-// One tile of 128 rows at a time, one thread per row, 128 threads; every
-// product is a tcgen05.mma with M = 128 (BF16 operands in the no-swizzle
-// K-major core-matrix layout above, FP32 accumulators in tensor memory):
+// One tile of 128 rows at a time, one thread per row, 128 threads, two blocks
+// per SM (one block's epilogues run under the other's products); every
+// product is a tcgen05.mma with M = 128 (BF16 operands in no-swizzle
+// core-matrix tiles as above, FP32 accumulators in tensor memory):
 //   h1 = tanh(X W1), h2 = tanh(h1 W2)             (forward recomputed; K 16, 64)
 //   dp2 = (dY W3^T) (1 - h2^2)                     (A = dY [128][16], B = W3 [64][16])
 //   dp1 = (dp2 W2^T) (1 - h1^2)                    (A = dp2 [128][64], B = W2 [64][64])
 // and the weight gradients as products over the tile's rows (K = 128), with
-// the tile's activations written transposed into the A and B operands:
-//   [h1^T; h2^T] (128 x 128) x dp2^T (64 x 128)^T -> rows 0-63: dW2 = h1^T dp2
-//   [h1^T; h2^T]             x dY^T  (16 x 128)^T -> rows 64-127: dW3 = h2^T dY
-//   [dp1^T; 0]               x X^T   (16 x 128)^T -> rows 0-63: dW1^T = dp1^T X
+// both operands read transposed (MN-major) from the tiles that the products
+// above use: H = [h1, h2] and Q = [dp2, dp1], 128 x 128 each,
+//   H^T dp2 -> rows 0-63: dW2 = h1^T dp2
+//   H^T dY  -> rows 64-127: dW3 = h2^T dY
+//   Q^T X   -> rows 64-127: dW1^T = dp1^T X
+// so nothing is written twice: a thread stores its row's activations 16 bytes
+// at a time (conflict-free) and keeps them packed for the derivatives.  The
+// earlier form wrote transposed copies of every operand two bytes at a time
+// (~512 four-way conflicting shared-memory accesses a thread and tile, 148 KB,
+// one block per SM): 233 us at 786,432 rows, this one 82.
+// dY of a row is formed here: d o[0:4] + (M^T d) o[4:8], o the readout (dout of
+// the row and its second message pass back, k_mp_loss and k_mp_pull).
 // The three gradient accumulators stay in tensor memory across all the
 // block's tiles and are read back once: one partial gradient per block,
-// summed over blocks in a fixed order (k_mp_grad_reduce).  Tensor memory:
-// columns 0-63 for the activations' products (reused), 64-127 dW2, 128-143
-// dW3, 144-159 dW1^T.  The derivative of tanh uses the BF16 activations the
+// summed over blocks in a fixed order (k_mp_update).  Tensor memory: columns
+// 0-63 for the activations' products (reused), 64-127 dW2, 128-143 dW3, 144-159
+// dW1^T, 160-223 dY W3^T.  The derivative of tanh uses the BF16 activations the
 // products use.  Every wait is bounded.
 namespace tcb {
 constexpr int kBRows = 128;
 constexpr int kBTmemCols = 256;
-constexpr int kColW2 = 64, kColW3 = 128, kColW1 = 144;
+constexpr int kColW2 = 64, kColW3 = 128, kColW1 = 144, kColH2 = 160;
 // dynamic shared memory layout (byte offsets, 128-byte aligned)
 constexpr int oW1T = 0;                      // [64][16]  W1^T          (B, layer 1)
 constexpr int oW2T = oW1T + 64 * 16 * 2;     // [64][64]  W2^T          (B, layer 2)
 constexpr int oW3P = oW2T + 64 * 64 * 2;     // [64][16]  W3 (k 4 -> 16) (B, dh2)
 constexpr int oW2N = oW3P + 64 * 16 * 2;     // [64][64]  W2            (B, dh1)
-constexpr int oX = oW2N + 64 * 64 * 2;       // [128][16] [x0, a0]      (A, layer 1)
-constexpr int oH1 = oX + kBRows * 16 * 2;     // [128][64] h1            (A, layer 2)
-constexpr int oDY = oH1 + kBRows * 64 * 2;    // [128][16] dY            (A, dh2)
-constexpr int oP2 = oDY + kBRows * 16 * 2;    // [128][64] dp2           (A, dh1)
-constexpr int oAT1 = oP2 + kBRows * 64 * 2;   // [128][128] [h1^T; h2^T] (A, dW2 and dW3)
-constexpr int oAT2 = oAT1 + 128 * 128 * 2;   // [128][128] [dp1^T; 0]   (A, dW1^T)
-constexpr int oBP2 = oAT2 + 128 * 128 * 2;   // [64][128] dp2^T         (B, dW2)
-constexpr int oBDY = oBP2 + 64 * 128 * 2;    // [16][128] dY^T          (B, dW3)
-constexpr int oBX = oBDY + 16 * 128 * 2;     // [16][128] X^T           (B, dW1^T)
-constexpr int kSmem = oBX + 16 * 128 * 2;
+constexpr int oX = oW2N + 64 * 64 * 2;       // [128][16] [x0, a0]      (A, layer 1; B, dW1^T)
+constexpr int oDY = oX + kBRows * 16 * 2;    // [128][16] dY            (A, dh2; B, dW3)
+constexpr int oH = oDY + kBRows * 16 * 2;    // [128][128] [h1, h2]     (A, layer 2, dW2 and dW3)
+constexpr int oQ = oH + kBRows * 128 * 2;    // [128][128] [dp2, dp1]   (A, dh1 and dW1^T; B, dW2)
+constexpr int kSmem = oQ + kBRows * 128 * 2;
+constexpr int kHalf = 8 * 128;               // bytes from column 0 to column 64 of a 128-column tile
+constexpr int kGroup = 16 * 128;             // bytes from one group of 8 rows of it to the next
 }  // namespace tcb
 
 int mp_bwd_tc_smem_bytes() { return tcb::kSmem + 128; }
 
-__global__ void __launch_bounds__(128, 1) k_mp_mlp_bwd_tc(int rows, MpBuffers M, DevState* st)
+__device__ __forceinline__ float bf16_lo(unsigned v) { return __uint_as_float(v << 16); }
+__device__ __forceinline__ float bf16_hi(unsigned v) { return __uint_as_float(v & 0xffff0000u); }
+
+__global__ void __launch_bounds__(128, 2) k_mp_mlp_bwd_tc(int rows, MpBuffers M, DevState* st)
 {
     using namespace tc;
     using namespace tcb;
@@ -346,13 +367,7 @@ __global__ void __launch_bounds__(128, 1) k_mp_mlp_bwd_tc(int rows, MpBuffers M,
     __shared__ unsigned tmem_base;
     __shared__ int failed;
     const int tid = threadIdx.x, warp = tid >> 5;
-    auto put = [&](int off, int r, int k, int K, float v) {
-        *reinterpret_cast<__nv_bfloat16*>(sm + off + core_off(r, k, K)) = __float2bfloat16_rn(v);
-    };
-    auto get = [&](int off, int r, int k, int K) {
-        return __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(sm + off + core_off(r, k, K)));
-    };
-    // weights (BF16 layouts of k_mp_adam) into core-matrix tiles
+    // weights (BF16 layouts of k_mp_update) into core-matrix tiles
     for (int e = tid; e < 64 * 16; e += blockDim.x) {
         *reinterpret_cast<__nv_bfloat16*>(sm + oW1T + core_off(e / 16, e % 16, 16)) = M.wb[kW1T + e];
         *reinterpret_cast<__nv_bfloat16*>(sm + oW3P + core_off(e / 16, e % 16, 16)) = M.wb[kW3P + e];
@@ -361,10 +376,6 @@ __global__ void __launch_bounds__(128, 1) k_mp_mlp_bwd_tc(int rows, MpBuffers M,
         *reinterpret_cast<__nv_bfloat16*>(sm + oW2T + core_off(e / 64, e % 64, 64)) = M.wb[kW2T + e];
         *reinterpret_cast<__nv_bfloat16*>(sm + oW2N + core_off(e / 64, e % 64, 64)) = M.wb[kW2N + e];
     }
-    // rows 64-127 of [dp1^T; 0], rows 4-15 of dY^T and 6-15 of X^T stay zero
-    for (int e = tid; e < 64 * 128; e += blockDim.x) put(oAT2, 64 + e / 128, e % 128, 128, 0.f);
-    for (int e = tid; e < 12 * 128; e += blockDim.x) put(oBDY, 4 + e / 128, e % 128, 128, 0.f);
-    for (int e = tid; e < 10 * 128; e += blockDim.x) put(oBX, 6 + e / 128, e % 128, 128, 0.f);
     if (tid == 0) {
         failed = 0;
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&mbar)) : "memory");
@@ -382,9 +393,13 @@ __global__ void __launch_bounds__(128, 1) k_mp_mlp_bwd_tc(int rows, MpBuffers M,
     fence_after();
     const unsigned tmem = tmem_base;
     const unsigned tlane = tmem + ((unsigned)(warp * 32) << 16);   // this warp's lane quarter
-    const unsigned id64 = idesc_bf16(kBRows, 64), id16 = idesc_bf16(kBRows, 16);
+    const unsigned id64 = idesc_bf16(kBRows, 64);
+    const unsigned idt64 = idesc_bf16(kBRows, 64, true), idt16 = idesc_bf16(kBRows, 16, true);
     unsigned phase = 0;
     int acc = 0;   // the gradient products accumulate after the block's first tile
+    float o[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) o[k] = M.master[kMpOffO + k];
     auto sync_mma = [&]() {   // operands written by all threads -> visible to the MMA issuer
         fence_async_smem();
         fence_before();
@@ -396,106 +411,118 @@ __global__ void __launch_bounds__(128, 1) k_mp_mlp_bwd_tc(int rows, MpBuffers M,
         phase ^= 1u;
         fence_after();
     };
+    auto put8 = [&](int off, const unsigned* w) {   // 8 columns of this thread's row of a 128-column tile
+        *reinterpret_cast<uint4*>(sm + off + (tid >> 3) * kGroup + (tid & 7) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+    };
+    // the row's inputs, requested a tile ahead
+    float4 x, a;
+    float d, md;
+    auto load = [&](int r) {
+        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        x = r < rows ? M.x0[r] : z;
+        a = r < rows ? M.a0[r] : z;
+        d = r < rows ? reinterpret_cast<const float*>(M.dout)[4 * (r / 3) + r % 3] : 0.f;
+        md = r < rows ? reinterpret_cast<const float*>(M.pull)[4 * (r / 3) + r % 3] : 0.f;
+    };
+    load(blockIdx.x * kBRows + tid);
 
     for (int base = blockIdx.x * kBRows; base < rows && !failed; base += gridDim.x * kBRows) {
-        const int r = base + tid;   // this thread's row (tile row tid)
-        {   // X = [x0, a0] (k 6..15 zero) and dY (k 4..15 zero): rows, and transposed
-            const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-            const float4 x = r < rows ? M.x0[r] : z, a = r < rows ? M.a0[r] : z, d = r < rows ? M.dy[r] : z;
-            const float xs[6] = {x.x, x.y, x.z, a.x, a.y, a.z}, ds[4] = {d.x, d.y, d.z, d.w};
+        {   // X = [x0, a0] (k 6..15 zero) and dY (k 4..15 zero)
+            const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+            float dy[4];
 #pragma unroll
-            for (int k = 0; k < 16; ++k) {
-                put(oX, tid, k, 16, k < 6 ? xs[k] : 0.f);
-                put(oDY, tid, k, 16, k < 4 ? ds[k] : 0.f);
-            }
-#pragma unroll
-            for (int k = 0; k < 6; ++k) put(oBX, k, tid, 128, xs[k]);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) put(oBDY, k, tid, 128, ds[k]);
+            for (int k = 0; k < 4; ++k) dy[k] = fmaf(d, o[k], md * o[4 + k]);
+            *reinterpret_cast<uint4*>(sm + oX + core_off(tid, 0, 16)) =
+                make_uint4(pack_bf16(x.x, x.y), pack_bf16(x.z, a.x), pack_bf16(a.y, a.z), 0u);
+            *reinterpret_cast<uint4*>(sm + oX + core_off(tid, 8, 16)) = zero;
+            *reinterpret_cast<uint4*>(sm + oDY + core_off(tid, 0, 16)) =
+                make_uint4(pack_bf16(dy[0], dy[1]), pack_bf16(dy[2], dy[3]), 0u, 0u);
+            *reinterpret_cast<uint4*>(sm + oDY + core_off(tid, 8, 16)) = zero;
         }
         sync_mma();
-        if (tid == 0) {
+        if (tid == 0) {   // layer 1, and dh2 = dY W3^T
             mma(tmem, smem_desc(sm + oX, 16), smem_desc(sm + oW1T, 16), id64, 0);
+            mma(tmem + kColH2, smem_desc(sm + oDY, 16), smem_desc(sm + oW3P, 16), id64, 0);
             commit(&mbar);
         }
         wait_mma();
-        // h1 = tanh(D): row operand and rows 0-63 of [h1^T; h2^T]
+        unsigned h1[32], h2[32];   // the row's activations, packed
 #pragma unroll
         for (int c = 0; c < 64; c += 16) {
             float v[16];
             ld16(tlane + c, v);
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                const float h = tanh_fast(v[q]);
-                put(oH1, tid, c + q, 64, h);
-                put(oAT1, c + q, tid, 128, h);
-            }
+            for (int q = 0; q < 16; q += 2) h1[(c + q) / 2] = pack_bf16(tanh_fast(v[q]), tanh_fast(v[q + 1]));
+            put8(oH + c / 8 * 128, h1 + c / 2);
+            put8(oH + (c / 8 + 1) * 128, h1 + c / 2 + 4);
         }
         sync_mma();
         if (tid == 0) {
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks)
-                mma(tmem, smem_desc(sm + oH1 + ks * 256, 64), smem_desc(sm + oW2T + ks * 256, 64), id64, ks > 0);
+                mma(tmem, smem_desc(sm + oH + ks * 256, 128u, (unsigned)kGroup), smem_desc(sm + oW2T + ks * 256, 64),
+                    id64, ks > 0);
             commit(&mbar);
         }
         wait_mma();
-        // h2 = tanh(D): rows 64-127 of [h1^T; h2^T]
+        // h2 = tanh(D) and dp2 = dh2 (1 - h2^2)
 #pragma unroll
         for (int c = 0; c < 64; c += 16) {
-            float v[16];
+            float v[16], g[16];
             ld16(tlane + c, v);
+            ld16(tlane + kColH2 + c, g);
+            unsigned w[8];
 #pragma unroll
-            for (int q = 0; q < 16; ++q) put(oAT1, 64 + c + q, tid, 128, tanh_fast(v[q]));
-        }
-        sync_mma();
-        if (tid == 0) {   // dh2 = dY W3^T
-            mma(tmem, smem_desc(sm + oDY, 16), smem_desc(sm + oW3P, 16), id64, 0);
-            commit(&mbar);
-        }
-        wait_mma();
-        // dp2 = dh2 (1 - h2^2): row operand and transposed
-#pragma unroll
-        for (int c = 0; c < 64; c += 16) {
-            float v[16];
-            ld16(tlane + c, v);
-#pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                const float h = get(oAT1, 64 + c + q, tid, 128);
-                const float g = v[q] * (1.f - h * h);
-                put(oP2, tid, c + q, 64, g);
-                put(oBP2, c + q, tid, 128, g);
+            for (int q = 0; q < 16; q += 2) {
+                const unsigned h = pack_bf16(tanh_fast(v[q]), tanh_fast(v[q + 1]));
+                const float lo = bf16_lo(h), hi = bf16_hi(h);
+                h2[(c + q) / 2] = h;
+                w[q / 2] = pack_bf16(g[q] * (1.f - lo * lo), g[q + 1] * (1.f - hi * hi));
             }
+            put8(oH + kHalf + c / 8 * 128, h2 + c / 2);
+            put8(oH + kHalf + (c / 8 + 1) * 128, h2 + c / 2 + 4);
+            put8(oQ + c / 8 * 128, w);
+            put8(oQ + (c / 8 + 1) * 128, w + 4);
         }
         sync_mma();
-        if (tid == 0) {   // dh1 = dp2 W2^T
+        if (tid == 0) {   // dh1 = dp2 W2^T, waited for; then dW2 and dW3 behind it (K = 128 rows, 16 a step)
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks)
-                mma(tmem, smem_desc(sm + oP2 + ks * 256, 64), smem_desc(sm + oW2N + ks * 256, 64), id64, ks > 0);
+                mma(tmem, smem_desc(sm + oQ + ks * 256, 128u, (unsigned)kGroup), smem_desc(sm + oW2N + ks * 256, 64),
+                    id64, ks > 0);
             commit(&mbar);
-        }
-        wait_mma();
-        // dp1 = dh1 (1 - h1^2), transposed into rows 0-63 of [dp1^T; 0]
-#pragma unroll
-        for (int c = 0; c < 64; c += 16) {
-            float v[16];
-            ld16(tlane + c, v);
-#pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                const float h = get(oH1, tid, c + q, 64);
-                put(oAT2, c + q, tid, 128, v[q] * (1.f - h * h));
-            }
-        }
-        sync_mma();
-        if (tid == 0) {   // the weight gradients, summed over the tile's rows (K = 128)
 #pragma unroll
             for (int ks = 0; ks < 8; ++ks) {
-                const int a = acc | (ks > 0);
-                mma(tmem + kColW2, smem_desc(sm + oAT1 + ks * 256, 128), smem_desc(sm + oBP2 + ks * 256, 128), id64, a);
-                mma(tmem + kColW3, smem_desc(sm + oAT1 + ks * 256, 128), smem_desc(sm + oBDY + ks * 256, 128), id16, a);
-                mma(tmem + kColW1, smem_desc(sm + oAT2 + ks * 256, 128), smem_desc(sm + oBX + ks * 256, 128), id16, a);
+                const int on = acc | (ks > 0);
+                const unsigned long long h = smem_desc(sm + oH + ks * 2 * kGroup, (unsigned)kGroup, 128u);
+                mma(tmem + kColW2, h, smem_desc(sm + oQ + ks * 2 * kGroup, (unsigned)kGroup, 128u), idt64, on);
+                mma(tmem + kColW3, h, smem_desc(sm + oDY + ks * 512, 256u, 128u), idt16, on);
             }
+        }
+        wait_mma();
+        // dp1 = dh1 (1 - h1^2)
+#pragma unroll
+        for (int c = 0; c < 64; c += 16) {
+            float v[16];
+            ld16(tlane + c, v);
+            unsigned w[8];
+#pragma unroll
+            for (int q = 0; q < 16; q += 2) {
+                const float lo = bf16_lo(h1[(c + q) / 2]), hi = bf16_hi(h1[(c + q) / 2]);
+                w[q / 2] = pack_bf16(v[q] * (1.f - lo * lo), v[q + 1] * (1.f - hi * hi));
+            }
+            put8(oQ + kHalf + c / 8 * 128, w);
+            put8(oQ + kHalf + (c / 8 + 1) * 128, w + 4);
+        }
+        sync_mma();
+        if (tid == 0) {
+#pragma unroll
+            for (int ks = 0; ks < 8; ++ks)
+                mma(tmem + kColW1, smem_desc(sm + oQ + ks * 2 * kGroup, (unsigned)kGroup, 128u),
+                    smem_desc(sm + oX + ks * 512, 256u, 128u), idt16, acc | (ks > 0));
             commit(&mbar);
         }
+        load(base + gridDim.x * kBRows + tid);
         wait_mma();   // the next tile overwrites the operands
         acc = 1;
         fence_before();
@@ -505,7 +532,7 @@ __global__ void __launch_bounds__(128, 1) k_mp_mlp_bwd_tc(int rows, MpBuffers M,
     // this block's partial gradient (zero if it had no tile)
     float* gp = M.gpart + (size_t)blockIdx.x * kMpParams;
     if (acc && !failed) {
-        if (warp < 2) {   // rows 0-63: dW2[i][h] (i = row) and dW1^T[i][f]
+        if (warp < 2) {   // rows 0-63: dW2[i][h] (i = row)
             const int i = tid;
 #pragma unroll
             for (int c = 0; c < 64; c += 16) {
@@ -514,16 +541,15 @@ __global__ void __launch_bounds__(128, 1) k_mp_mlp_bwd_tc(int rows, MpBuffers M,
 #pragma unroll
                 for (int q = 0; q < 16; ++q) gp[kMpOffW2 + i * 64 + c + q] = v[q];
             }
-            float v[16];
-            ld16(tlane + kColW1, v);
-#pragma unroll
-            for (int f = 0; f < 6; ++f) gp[kMpOffW1 + f * 64 + i] = v[f];
-        } else {          // rows 64-127: dW3[h][m] (h = row - 64)
+        } else {          // rows 64-127: dW3[h][m] (h = row - 64) and dW1^T[i][f] (i = row - 64)
             const int h = tid - 64;
             float v[16];
             ld16(tlane + kColW3, v);
 #pragma unroll
             for (int m = 0; m < 4; ++m) gp[kMpOffW3 + h * 4 + m] = v[m];
+            ld16(tlane + kColW1, v);
+#pragma unroll
+            for (int f = 0; f < 6; ++f) gp[kMpOffW1 + f * 64 + h] = v[f];
         }
     } else {
         for (int e = tid; e < kMpOffO; e += blockDim.x) gp[e] = 0.f;
@@ -534,9 +560,6 @@ __global__ void __launch_bounds__(128, 1) k_mp_mlp_bwd_tc(int rows, MpBuffers M,
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kBTmemCols) : "memory");
 }
-
-namespace {
-}  // namespace
 
 // -------------------------------------------------------------- kernels
 
@@ -587,24 +610,34 @@ __global__ void k_mp_input(KParams P, DevBuffers B, MpBuffers M)
     }
 }
 
-// out = M in (mode 0), out = M^T in (mode 1), out += M^T in (mode 2); three rows per node.
-__global__ void k_mp_aggregate(KParams P, DevBuffers B, const float4* __restrict__ in, float4* __restrict__ out,
-                               int mode)
+// This thread's node and its entries' range.  The message passes take the rows
+// in row order: neighbouring lanes gather largely the same rows (in slot order
+// the entry loads are coalesced, but a pass took 66 us instead of 61).
+struct MpNode {
+    int i, base, cnt;
+};
+__device__ __forceinline__ MpNode mp_node(const KParams& P, const DevBuffers& B)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= P.n) return;
+    if (i >= P.n) return MpNode{-1, 0, 0};
     const int slot = B.row_slot[i];
-    const int base = B.chunk_off[slot >> 5] + (slot & 31);
-    const int cnt = B.row_cnt[i];
+    return MpNode{i, B.chunk_off[slot >> 5] + (slot & 31), B.row_cnt[i]};
+}
+
+// a0 = M x0; three rows per node.
+__global__ void k_mp_aggregate(KParams P, DevBuffers B, const float4* __restrict__ in, float4* __restrict__ out)
+{
+    const MpNode nd = mp_node(P, B);
+    const int i = nd.i;
+    if (i < 0) return;
     const float ae = (float)P.alpha;
     float4 s[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) s[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int k = 0; k < cnt; ++k) {
-        const int e = base + 32 * k;
+    for (int k = 0; k < nd.cnt; ++k) {
+        const int e = nd.base + 32 * k;
         const int j = B.col[e];
-        float w = ae * B.val32[e];
-        if (mode != 0) w *= B.dinv32[j];
+        const float w = ae * B.val32[e];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const float4 u = in[3 * j + c];
@@ -614,16 +647,30 @@ __global__ void k_mp_aggregate(KParams P, DevBuffers B, const float4* __restrict
             s[c].w = fmaf(w, u.w, s[c].w);
         }
     }
-    const float di = mode == 0 ? B.dinv32[i] : 1.f;
+    const float di = B.dinv32[i];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        float4 r = make_float4(s[c].x * di, s[c].y * di, s[c].z * di, s[c].w * di);
-        if (mode == 2) {
-            const float4 o = out[3 * i + c];
-            r = make_float4(r.x + o.x, r.y + o.y, r.z + o.z, r.w + o.w);
-        }
-        out[3 * i + c] = r;
+    for (int c = 0; c < 3; ++c) out[3 * i + c] = make_float4(s[c].x * di, s[c].y * di, s[c].z * di, s[c].w * di);
+}
+
+// pull = M^T dout, one value per component: the gradient at the second message
+// pass is dout times the readout's four weights, a product of the row's scalar
+// with a constant vector, so M^T acts on the scalar (16 bytes per entry
+// instead of 48; scaled holds D^-1 dout).
+__global__ void k_mp_pull(KParams P, DevBuffers B, const float4* __restrict__ scaled, float4* __restrict__ pull)
+{
+    const MpNode nd = mp_node(P, B);
+    if (nd.i < 0) return;
+    const float ae = (float)P.alpha;
+    float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+    for (int k = 0; k < nd.cnt; ++k) {
+        const int e = nd.base + 32 * k;
+        const float4 v = scaled[B.col[e]];
+        const float w = ae * B.val32[e];
+        s0 = fmaf(w, v.x, s0);
+        s1 = fmaf(w, v.y, s1);
+        s2 = fmaf(w, v.z, s2);
     }
+    pull[nd.i] = make_float4(s0, s1, s2, 0.f);
 }
 
 // Second message pass fused with the output: a1 = M y for node i, then
@@ -631,17 +678,15 @@ __global__ void k_mp_aggregate(KParams P, DevBuffers B, const float4* __restrict
 // for training).
 __global__ void k_mp_aggregate_output(KParams P, DevBuffers B, MpBuffers M)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= P.n) return;
-    const int slot = B.row_slot[i];
-    const int base = B.chunk_off[slot >> 5] + (slot & 31);
-    const int cnt = B.row_cnt[i];
+    const MpNode nd = mp_node(P, B);
+    const int i = nd.i;
+    if (i < 0) return;
     const float ae = (float)P.alpha;
     float4 acc[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) acc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int k = 0; k < cnt; ++k) {
-        const int e = base + 32 * k;
+    for (int k = 0; k < nd.cnt; ++k) {
+        const int e = nd.base + 32 * k;
         const int j = B.col[e];
         const float w = ae * B.val32[e];
 #pragma unroll
@@ -668,62 +713,66 @@ __global__ void k_mp_aggregate_output(KParams P, DevBuffers B, MpBuffers M)
     }
 }
 
-// Loss rows: e = out - vstar / s, dout = 2 e / 3n; dy = dout o[0:4], g1 = dout o[4:8];
-// per block: sum e^2 and the readout gradient sum dout [y, a1, x0].
-__global__ void k_mp_loss(KParams P, DevBuffers B, MpBuffers M)
+// Loss rows: e = out - vstar / s, dout = 2 e / 3n (dout and D^-1 dout of each
+// node kept); per block: sum e^2 and the readout gradient sum dout [y, a1, x0].
+// FP64 only for e, its square's sum and dout (five operations a row on GB300's
+// 1/64-rate pipe); the readout's eleven sums are compensated FP32 (exact
+// TwoSum errors in a second word), which was 24 FP64 operations a row: 107 us
+// at 786,432 rows before, 20 now.
+__global__ void __launch_bounds__(kVecBlock) k_mp_loss(KParams P, DevBuffers B, MpBuffers M, double two_by_rows)
 {
-    const double s = M.scal[0];
-    const float* o = M.master + kMpOffO;
-    const int rows = 3 * P.n;
-    double acc[12];
+    __shared__ double s_inv;
+    if (threadIdx.x == 0) s_inv = 1.0 / M.scal[0];
+    __syncthreads();
+    const double inv = s_inv;
+    float o[11];
 #pragma unroll
-    for (int k = 0; k < 12; ++k) acc[k] = 0.0;
+    for (int k = 0; k < 11; ++k) o[k] = M.master[kMpOffO + k];
+    const int rows = 3 * P.n;
+    double ee = 0.0;
+    dfloat acc[11];
+#pragma unroll
+    for (int k = 0; k < 11; ++k) acc[k] = dfloat{0.f, 0.f};
     for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += gridDim.x * blockDim.x) {
         const int i = r / 3, c = r - 3 * i;
         const float4 y = M.y[r], a = M.a1[r], x = M.x0[r];
         const float out = y.x * o[0] + y.y * o[1] + y.z * o[2] + y.w * o[3] + a.x * o[4] + a.y * o[5] + a.z * o[6] +
                           a.w * o[7] + x.x * o[8] + x.y * o[9] + x.z * o[10];
-        const double e = (double)out - B.x[c * P.npad + i] / s;
-        const float d = (float)(2.0 * e / rows);
-        M.dy[r] = make_float4(d * o[0], d * o[1], d * o[2], d * o[3]);
-        M.g1[r] = make_float4(d * o[4], d * o[5], d * o[6], d * o[7]);
+        const double e = fma(-B.x[c * P.npad + i], inv, (double)out);
+        const float d = (float)(e * two_by_rows);
+        ee = fma(e, e, ee);
+        reinterpret_cast<float*>(M.dout)[4 * i + c] = d;
+        reinterpret_cast<float*>(M.scaled)[4 * i + c] = d * B.dinv32[i];
         const float f[11] = {y.x, y.y, y.z, y.w, a.x, a.y, a.z, a.w, x.x, x.y, x.z};
-        acc[0] += e * e;
 #pragma unroll
-        for (int k = 0; k < 11; ++k) acc[1 + k] += (double)(d * f[k]);
+        for (int k = 0; k < 11; ++k) {
+            const dfloat t = two_sum(acc[k].hi, __fmul_rn(d, f[k]));
+            acc[k] = dfloat{t.hi, __fadd_rn(acc[k].lo, t.lo)};
+        }
     }
-    __shared__ double sh[32];
+    __shared__ float2 sh[11][kVecBlock / 32];
+    __shared__ double she[kVecBlock / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int k = 0; k < 12; ++k) {
-        const double t = block_sum(acc[k], sh);
-        if (threadIdx.x == 0) M.dpart[blockIdx.x * 12 + k] = t;
+    for (int k = 0; k < 11; ++k) {
+        const dfloat t = warp_sum_df(fast_two_sum(acc[k].hi, acc[k].lo));
+        if (lane == 0) sh[k][warp] = make_float2(t.hi, t.lo);
+    }
+    ee = warp_sum(ee);
+    if (lane == 0) she[warp] = ee;
+    __syncthreads();
+    if (threadIdx.x < 12) {
+        double t = 0.0;
+        for (int w = 0; w < kVecBlock / 32; ++w)
+            t += threadIdx.x == 0 ? she[w] : (double)sh[threadIdx.x - 1][w].x + (double)sh[threadIdx.x - 1][w].y;
+        M.dpart[blockIdx.x * 12 + threadIdx.x] = t;
     }
 }
 
-// grad = sum over blocks (fixed order); the readout's gradient and the loss from the loss blocks.
-__global__ void k_mp_grad_reduce(MpBuffers M, int nblocks_mlp, int nblocks_loss, int rows)
+// One weight by Adam (Kingma & Ba 2015) on the FP32 masters, then its BF16
+// entries of the layouts for the kernels.
+__device__ __forceinline__ void mp_adam(const MpBuffers& M, int p, float lr, int t)
 {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p < kMpOffO) {
-        float s = 0.f;
-        for (int b = 0; b < nblocks_mlp; ++b) s += M.gpart[(size_t)b * kMpParams + p];
-        M.grad[p] = s;
-    } else if (p < kMpParams) {
-        double s = 0.0;
-        for (int b = 0; b < nblocks_loss; ++b) s += M.dpart[b * 12 + 1 + (p - kMpOffO)];
-        M.grad[p] = (float)s;
-    } else if (p == kMpParams) {
-        double s = 0.0;
-        for (int b = 0; b < nblocks_loss; ++b) s += M.dpart[b * 12];
-        M.scal[1] = s / rows;
-    }
-}
-
-// Adam (Kingma & Ba 2015) on the FP32 masters, then the BF16 layouts for the kernels.
-__global__ void k_mp_adam(MpBuffers M, float lr, int t)
-{
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= kMpParams) return;
     if (lr != 0.f) {
         const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
         const float gp = M.grad[p];
@@ -750,6 +799,51 @@ __global__ void k_mp_adam(MpBuffers M, float lr, int t)
     }
 }
 
+__global__ void k_mp_convert(MpBuffers M)
+{
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p < kMpParams) mp_adam(M, p, 0.f, 1);
+}
+
+// grad = sum over blocks (fixed order: warp w of a block takes partials w, w +
+// 8, ..., then the warps in turn; one thread per weight summing all of them in
+// turn took 75 us), the readout's gradient and the loss from the loss blocks,
+// and the weight's Adam step.
+__global__ void __launch_bounds__(256) k_mp_update(MpBuffers M, int nblocks_mlp, int nblocks_loss, int rows, float lr,
+                                                   int t)
+{
+    __shared__ double sh[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, p = blockIdx.x * 32 + lane;
+    double s = 0.0;
+    if (p < kMpOffO) {
+        float f = 0.f;
+#pragma unroll 4
+        for (int b = warp; b < nblocks_mlp; b += 8) f += M.gpart[(size_t)b * kMpParams + p];
+        s = f;
+    } else if (p <= kMpParams) {   // entry 0 of a loss block: sum e^2; 1 + k: the readout's gradient
+        const int k = p < kMpParams ? 1 + (p - kMpOffO) : 0;
+#pragma unroll 4
+        for (int b = warp; b < nblocks_loss; b += 8) s += M.dpart[b * 12 + k];
+    }
+    sh[warp][lane] = s;
+    __syncthreads();
+    if (warp != 0 || p > kMpParams) return;
+    if (p < kMpOffO) {
+        float f = 0.f;
+        for (int w = 0; w < 8; ++w) f += (float)sh[w][lane];
+        M.grad[p] = f;
+    } else {
+        double a = 0.0;
+        for (int w = 0; w < 8; ++w) a += sh[w][lane];
+        if (p == kMpParams) {
+            M.scal[1] = a / rows;
+            return;
+        }
+        M.grad[p] = (float)a;
+    }
+    mp_adam(M, p, lr, t);
+}
+
 // ------------------------------------------------------------------ launchers
 
 void launch_mp_infer(const KParams& P, DevBuffers& B, MpBuffers& M, Launch L)
@@ -757,7 +851,7 @@ void launch_mp_infer(const KParams& P, DevBuffers& B, MpBuffers& M, Launch L)
     const int rows = 3 * P.n;
     k_mp_scale<<<grid_for(P.n, kVecBlock, L.num_sms * 4), kVecBlock, 0, L.stream>>>(P, B, M);
     k_mp_input<<<grid_for(P.n, kVecBlock, 1 << 30), kVecBlock, 0, L.stream>>>(P, B, M);
-    k_mp_aggregate<<<grid_for(P.n, 128, 1 << 30), 128, 0, L.stream>>>(P, B, M.x0, M.a0, 0);
+    k_mp_aggregate<<<grid_for(P.n, 128, 1 << 30), 128, 0, L.stream>>>(P, B, M.x0, M.a0);
     k_mp_mlp_fwd_tc<<<grid_for(rows, tc::kRows, L.num_sms * 6), tc::kRows, 0, L.stream>>>(rows, M, B.st);
     k_mp_aggregate_output<<<grid_for(P.n, 128, 1 << 30), 128, 0, L.stream>>>(P, B, M);
 }
@@ -776,13 +870,12 @@ void launch_mp_apply(const KParams& P, DevBuffers& B, const MpBuffers& M, const 
 void launch_mp_train(const KParams& P, DevBuffers& B, MpBuffers& M, float lr, int t, Launch L)
 {
     const int rows = 3 * P.n;
-    const int nloss = grid_for(rows, kVecBlock, std::min(kMaxGradBlocks, L.num_sms * 4));
-    k_mp_loss<<<nloss, kVecBlock, 0, L.stream>>>(P, B, M);
-    k_mp_aggregate<<<grid_for(P.n, 128, 1 << 30), 128, 0, L.stream>>>(P, B, M.g1, M.dy, 2);
-    const int nmlp = grid_for(rows, kTileRows, std::min(kMaxGradBlocks, L.num_sms));
+    const int nloss = grid_for(rows, kVecBlock, std::min(kMaxGradBlocks, L.num_sms * 2));
+    k_mp_loss<<<nloss, kVecBlock, 0, L.stream>>>(P, B, M, 2.0 / rows);
+    k_mp_pull<<<grid_for(P.n, 128, 1 << 30), 128, 0, L.stream>>>(P, B, M.scaled, M.pull);
+    const int nmlp = grid_for(rows, kTileRows, std::min(kMaxGradBlocks, L.num_sms * 2));
     k_mp_mlp_bwd_tc<<<nmlp, 128, mp_bwd_tc_smem_bytes(), L.stream>>>(rows, M, B.st);
-    k_mp_grad_reduce<<<grid_for(kMpParams + 1, kVecBlock, 1 << 30), kVecBlock, 0, L.stream>>>(M, nmlp, nloss, rows);
-    k_mp_adam<<<grid_for(kMpParams, kVecBlock, 1 << 30), kVecBlock, 0, L.stream>>>(M, lr, t);
+    k_mp_update<<<kMpParams / 32 + 1, 256, 0, L.stream>>>(M, nmlp, nloss, rows, lr, t);
 }
 
 int mp_prepare()
@@ -795,7 +888,7 @@ int mp_weights_bf16_count() { return kWB; }
 
 void launch_mp_convert(MpBuffers& M, cudaStream_t s)
 {
-    k_mp_adam<<<grid_for(kMpParams, kVecBlock, 1 << 30), kVecBlock, 0, s>>>(M, 0.f, 1);
+    k_mp_convert<<<grid_for(kMpParams, kVecBlock, 1 << 30), kVecBlock, 0, s>>>(M);
 }
 
 }  // namespace ss
