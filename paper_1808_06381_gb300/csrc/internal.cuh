@@ -862,6 +862,7 @@ void launch_reset_step_stats(DevState* st, cudaStream_t s);
 cudaError_t device_code_version(int* binary_version, int* ptx_version);
 // sfactor.cu: S(q) at q_z = 0 for kx in [-nkx, nkx], ky in [-nky, nky] (kx slowest);
 // G = 0: direct sum over particles; G > 0: CIC grid of G x G in the sheared frame.
+// A_dev: (nkx + 1) G complex values, then max(nkx, nky) + 1 doubles.
 cudaError_t run_structure_factor(const KParams& P, const DevBuffers& B, double delta, int G, int nkx, int nky,
                                  const double* twiddle_dev, unsigned long long* grid_dev, double2* A_dev,
                                  double* S_dev, double* qx_dev, double* qy_dev, cudaStream_t s);

@@ -1703,7 +1703,7 @@ int sp_structure_factor(sp_sim* s, int32_t nkx, int32_t nky, int32_t grid, doubl
     if (grid > 0) {
         A_(dev_alloc(s, &tw, 2 * (size_t)grid));
         A_(dev_alloc(s, &g, (size_t)grid * grid));
-        A_(dev_alloc(s, &A, (size_t)(2 * nkx + 1) * grid));
+        A_(dev_alloc(s, &A, (size_t)(nkx + 1) * grid + std::max(nkx, nky) / 2 + 1));   // and the windows
     }
     if (rc == SP_OK && grid > 0) {
         // twiddle table (cos, sin)(2 pi m / G), m = 0..G-1
