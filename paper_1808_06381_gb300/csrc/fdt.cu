@@ -43,26 +43,41 @@ __global__ void k_cheb_bound(KParams P, DevBuffers B, unsigned long long* out)
 // that a whole step stays one graph): cs[0] = 2 / (b - a), cs[1] = (b + a) /
 // (b - a), cs[2 + k] = c_k, k <= degree; csf the same as double-floats.  With
 // no coupling (lambda_max = 1) p = 1: c_0 = 2, the rest 0.
-__global__ void k_cheb_coeffs(const unsigned long long* __restrict__ bound, int degree, double* __restrict__ cs,
-                              float2* __restrict__ csf)
+// c_k = 2 / N sum_j f_j cos(pi k (2 j + 1) / (2 N)), f_j = sqrt at the j-th point:
+// every cosine of the sum is one of cos(pi m / (2 N)), m = 0..N, so the block
+// forms that quarter wave and the f_j once (one cosine a thread; 33 x 2 FP64
+// cosines in turn in every thread took 76 us at degree 32, this 12).
+// Each block takes blockDim.x of the coefficients.
+__global__ void __launch_bounds__(128) k_cheb_coeffs(const unsigned long long* __restrict__ bound, int degree,
+                                                     double* __restrict__ cs, float2* __restrict__ csf)
 {
+    extern __shared__ double cheb_sm[];
     const double lmax = __longlong_as_double((long long)*bound);
     const bool ident = !(lmax - 1.0 > 1e-12);
     const int N = degree + 1;
-    const double pi = 3.141592653589793238462643383279502884;
+    double* f = cheb_sm;          // [N]
+    double* quarter = f + N;      // [N + 1] cos(pi m / (2 N))
+    for (int m = threadIdx.x; m <= N; m += blockDim.x) quarter[m] = cospi((double)m / (double)(2 * N));
+    __syncthreads();
+    auto cosine = [&](long long m) {   // cos(pi m / (2 N)), m >= 0
+        int r = (int)(m % (4 * N));
+        if (r > 2 * N) r = 4 * N - r;
+        return r <= N ? quarter[r] : -quarter[2 * N - r];
+    };
+    for (int j = threadIdx.x; j < N; j += blockDim.x)
+        f[j] = sqrt(0.5 * (lmax - 1.0) * cosine(2 * j + 1) + 0.5 * (lmax + 1.0));
+    __syncthreads();
     auto split = [](double x) { const float h = (float)x; return make_float2(h, (float)(x - (double)h)); };
-    for (int k = threadIdx.x; k < N; k += blockDim.x) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < N) {
         double acc = 0.0;
         if (!ident)
-            for (int j = 0; j < N; ++j) {
-                const double th = pi * (j + 0.5) / N;
-                acc += sqrt(0.5 * (lmax - 1.0) * cos(th) + 0.5 * (lmax + 1.0)) * cos(k * th);
-            }
+            for (int j = 0; j < N; ++j) acc = fma(f[j], cosine((long long)k * (2 * j + 1)), acc);
         const double c = ident ? (k == 0 ? 2.0 : 0.0) : 2.0 / N * acc;
         cs[2 + k] = c;
         csf[2 + k] = split(c);
     }
-    if (threadIdx.x == 0) {
+    if (k == 0) {
         const double s1 = ident ? 0.0 : 2.0 / (lmax - 1.0), s0 = ident ? 0.0 : (lmax + 1.0) / (lmax - 1.0);
         cs[0] = s1;
         cs[1] = s0;
@@ -106,7 +121,9 @@ __global__ void __launch_bounds__(256) k_cheb_step(KParams P, DevBuffers B, cons
 
 // The same degree step for the mixed path in double-float on the FP32 pipes:
 // T_k and xi as 32-byte records per row (hi float4, lo float4), the weights
-// and A_ii as their double-float pairs.
+// and A_ii as their double-float pairs.  Bound by the L1 wavefronts of the
+// gathered records, so a record is one 32-byte access (n = 262,144 clustered,
+// 18 entries a row: 57 us a step with two 16-byte accesses, 51.5 with one).
 __global__ void __launch_bounds__(256) k_cheb_step_df(KParams P, DevBuffers B, const float4* __restrict__ tc,
                                                       const float4* __restrict__ tp, float4* __restrict__ tn,
                                                       float4* __restrict__ y, const float2* __restrict__ csf, int kdeg)
@@ -123,11 +140,14 @@ __global__ void __launch_bounds__(256) k_cheb_step_df(KParams P, DevBuffers B, c
                   s);
     const dfloat d{B.diag32[row], B.diag32lo[row]}, al{P.alpha_hi, P.alpha_lo};
     const dfloat S1{s1.x, s1.y}, S0{s0.x, s0.y}, CK{ck.x, ck.y}, C0{c0h.x, c0h.y};
-    const float4 th = tc[2 * row], tl = tc[2 * row + 1];
+    float4 th, tl;
+    load_record(tc + 2 * row, th, tl);
     const dfloat t[3] = {{th.x, tl.x}, {th.y, tl.y}, {th.z, tl.z}};
     dfloat pv[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}}, yv[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
     if (!first) {
-        const float4 ph = tp[2 * row], pl = tp[2 * row + 1], yh = y[2 * row], yl = y[2 * row + 1];
+        float4 ph, pl, yh, yl;
+        load_record(tp + 2 * row, ph, pl);
+        load_record(y + 2 * row, yh, yl);
         pv[0] = dfloat{ph.x, pl.x};
         pv[1] = dfloat{ph.y, pl.y};
         pv[2] = dfloat{ph.z, pl.z};
@@ -143,10 +163,10 @@ __global__ void __launch_bounds__(256) k_cheb_step_df(KParams P, DevBuffers B, c
         v[c] = first ? u : df_add(dfloat{2.f * u.hi, 2.f * u.lo}, df_neg(pv[c]));
         yn[c] = first ? df_add(df_mul(C0, t[c]), df_mul(CK, v[c])) : df_add(yv[c], df_mul(CK, v[c]));
     }
-    tn[2 * row] = make_float4(v[0].hi, v[1].hi, v[2].hi, 0.f);
-    tn[2 * row + 1] = make_float4(v[0].lo, v[1].lo, v[2].lo, 0.f);
-    y[2 * row] = make_float4(yn[0].hi, yn[1].hi, yn[2].hi, 0.f);
-    y[2 * row + 1] = make_float4(yn[0].lo, yn[1].lo, yn[2].lo, 0.f);
+    store_record(tn + 2 * row, make_float4(v[0].hi, v[1].hi, v[2].hi, 0.f),
+                 make_float4(v[0].lo, v[1].lo, v[2].lo, 0.f));
+    store_record(y + 2 * row, make_float4(yn[0].hi, yn[1].hi, yn[2].hi, 0.f),
+                 make_float4(yn[0].lo, yn[1].lo, yn[2].lo, 0.f));
 }
 
 // FP64 planes [3][npad] to double-float records and back.
@@ -298,7 +318,12 @@ cudaError_t cheb_step_df(const KParams& P, DevBuffers& B, const float4* tc, cons
 
 cudaError_t cheb_coeffs(const unsigned long long* bound, int degree, double* cs, float2* csf, cudaStream_t s)
 {
-    k_cheb_coeffs<<<1, 128, 0, s>>>(bound, degree, cs, csf);
+    const int N = degree + 1, smem = (int)sizeof(double) * (2 * N + 1);   // 64 KB at the largest degree
+    if (smem > 40 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(k_cheb_coeffs, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+    }
+    k_cheb_coeffs<<<(N + 127) / 128, 128, smem, s>>>(bound, degree, cs, csf);
     return cudaGetLastError();
 }
 

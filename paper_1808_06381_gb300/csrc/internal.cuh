@@ -338,6 +338,24 @@ __device__ __forceinline__ float ld_stream(const float* p)
     return v;
 }
 
+// A 32-byte record (two float4, 32-byte aligned: one sector) in one load or
+// store.  A warp's gather of 32 records is bound by its L1 wavefronts, one per
+// line touched, and two 16-byte loads touch every line twice.  Ordered like a
+// plain access (volatile, memory clobber), so it stays behind a grid barrier.
+__device__ __forceinline__ void load_record(const float4* p, float4& h, float4& l)
+{
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(h.x), "=f"(h.y), "=f"(h.z), "=f"(h.w), "=f"(l.x), "=f"(l.y), "=f"(l.z), "=f"(l.w)
+                 : "l"(p)
+                 : "memory");
+}
+__device__ __forceinline__ void store_record(float4* p, float4 h, float4 l)
+{
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(h.x), "f"(h.y), "f"(h.z),
+                 "f"(h.w), "f"(l.x), "f"(l.y), "f"(l.z), "f"(l.w)
+                 : "memory");
+}
+
 // Philox4x64-10 (Salmon, Moraes, Dror, Shaw, SC'11).
 __device__ __forceinline__ void philox4x64_10(unsigned long long c[4], unsigned long long k0,
                                               unsigned long long k1)
@@ -632,10 +650,7 @@ __device__ __forceinline__ void row_sum_df(const int* __restrict__ col, const fl
 #pragma unroll
         for (int u = 0; u < KB; ++u) {
             xh[u] = xl[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (h[u] != 0.f) {
-                xh[u] = xdf[2 * j[u]];
-                xl[u] = xdf[2 * j[u] + 1];
-            }
+            if (h[u] != 0.f) load_record(xdf + 2 * j[u], xh[u], xl[u]);
         }
 #pragma unroll
         for (int u = 0; u < KB; ++u) {
