@@ -260,13 +260,15 @@ int sp_batch_step(sp_batch* b, int32_t nsteps, sp_step_info* info)
         if (rc != SP_OK) return rc;
     }
     for (int k = 0; k < nsteps; ++k) SB_CUDA(cudaGraphLaunch(b->exec, b->stream));
+    // every replica's state behind the steps, one synchronisation for all
+    for (sp_sim* s : b->sims)
+        SB_CUDA(cudaMemcpyAsync(s->st_host, s->B.st, sizeof(DevState), cudaMemcpyDeviceToHost, b->stream));
     SB_CUDA(cudaStreamSynchronize(b->stream));
     int status = SP_OK;
     bool regrown = false;
     for (int k = 0; k < b->R; ++k) {
         sp_sim* s = b->sims[k];
-        int rc = read_state(s);
-        if (rc != SP_OK) return rc;
+        int rc = SP_OK;
         long long done = s->st_host->steps_in_call;
         long long iters = s->st_host->iter_sum, checks = s->st_host->true_checks;
         int iter_max = s->st_host->iter_max;

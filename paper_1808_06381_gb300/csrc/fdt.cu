@@ -169,26 +169,26 @@ __global__ void __launch_bounds__(256) k_cheb_step_df(KParams P, DevBuffers B, c
                  make_float4(yn[0].lo, yn[1].lo, yn[2].lo, 0.f));
 }
 
-// FP64 planes [3][npad] to double-float records and back.
-__global__ void k_cheb_split(KParams P, const double* __restrict__ g, float4* __restrict__ t)
+// FP64 vectors by particle id ([n][3]) to double-float records in row order, and back.
+__global__ void k_cheb_split(int n, const int* __restrict__ ids, const double* __restrict__ g, float4* __restrict__ t)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= P.n) return;
-    const int np = P.npad;
-    const dfloat a = df_split(g[i]), b = df_split(g[np + i]), c = df_split(g[2 * np + i]);
-    t[2 * i] = make_float4(a.hi, b.hi, c.hi, 0.f);
-    t[2 * i + 1] = make_float4(a.lo, b.lo, c.lo, 0.f);
+    if (i >= n) return;
+    const double* v = g + 3ll * ids[i];
+    const dfloat a = df_split(v[0]), b = df_split(v[1]), c = df_split(v[2]);
+    store_record(t + 2 * i, make_float4(a.hi, b.hi, c.hi, 0.f), make_float4(a.lo, b.lo, c.lo, 0.f));
 }
 
-__global__ void k_cheb_join(KParams P, const float4* __restrict__ y, double* __restrict__ out)
+__global__ void k_cheb_join(int n, const int* __restrict__ ids, const float4* __restrict__ y, double* __restrict__ out)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= P.n) return;
-    const int np = P.npad;
-    const float4 h = y[2 * i], l = y[2 * i + 1];
-    out[i] = (double)h.x + (double)l.x;
-    out[np + i] = (double)h.y + (double)l.y;
-    out[2 * np + i] = (double)h.z + (double)l.z;
+    if (i >= n) return;
+    float4 h, l;
+    load_record(y + 2 * i, h, l);
+    double* v = out + 3ll * ids[i];
+    v[0] = (double)h.x + (double)l.x;
+    v[1] = (double)h.y + (double)l.y;
+    v[2] = (double)h.z + (double)l.z;
 }
 
 // The normals the assembly of this step used (drawn by the pair search,
@@ -327,15 +327,15 @@ cudaError_t cheb_coeffs(const unsigned long long* bound, int degree, double* cs,
     return cudaGetLastError();
 }
 
-cudaError_t cheb_split(const KParams& P, const double* g, float4* t, cudaStream_t s)
+cudaError_t cheb_split(int n, const int* ids, const double* g_n3, float4* t, cudaStream_t s)
 {
-    k_cheb_split<<<grid_for(P.n, 256, 1 << 30), 256, 0, s>>>(P, g, t);
+    k_cheb_split<<<grid_for(n, 256, 1 << 30), 256, 0, s>>>(n, ids, g_n3, t);
     return cudaGetLastError();
 }
 
-cudaError_t cheb_join(const KParams& P, const float4* y, double* out, cudaStream_t s)
+cudaError_t cheb_join(int n, const int* ids, const float4* y, double* out_n3, cudaStream_t s)
 {
-    k_cheb_join<<<grid_for(P.n, 256, 1 << 30), 256, 0, s>>>(P, y, out);
+    k_cheb_join<<<grid_for(n, 256, 1 << 30), 256, 0, s>>>(n, ids, y, out_n3);
     return cudaGetLastError();
 }
 

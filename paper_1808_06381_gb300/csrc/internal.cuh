@@ -882,6 +882,17 @@ cudaError_t run_structure_factor(const KParams& P, const DevBuffers& B, double d
                                  const double* twiddle_dev, unsigned long long* grid_dev, double2* A_dev,
                                  double* S_dev, double* qx_dev, double* qy_dev, cudaStream_t s);
 
+// Work arrays of the structure factor, kept by the simulation between calls
+// (grown when a call needs more; the twiddles are those of grid size G).
+struct SqBuffers {
+    double* out = nullptr;              // [3][modes] S, qx, qy
+    double* tw = nullptr;               // [2 G] (cos, sin)(2 pi m / G)
+    unsigned long long* grid = nullptr; // [G][G]
+    double2* A = nullptr;
+    size_t out_cap = 0, grid_cap = 0, A_cap = 0;
+    int G = 0;
+};
+
 // fdt.cu: xi = p(A) g ~ A^(1/2) g (Chebyshev interpolant of sqrt on [1, lambda_max])
 cudaError_t cheb_bound(const KParams& P, DevBuffers& B, unsigned long long* out_dev, cudaStream_t s);
 // Work arrays of xi = p(A) g: v[0] holds g, v[1..3] the rotating T_k, v[4] xi;
@@ -904,12 +915,16 @@ cudaError_t cheb_step(const KParams& P, DevBuffers& B, const double* tc, const d
                       const double* cs, int k, cudaStream_t s);
 cudaError_t cheb_step_df(const KParams& P, DevBuffers& B, const float4* tc, const float4* tp, float4* tn, float4* y,
                          const float2* csf, int k, cudaStream_t s);
-cudaError_t cheb_split(const KParams& P, const double* g, float4* t, cudaStream_t s);
-cudaError_t cheb_join(const KParams& P, const float4* y, double* out, cudaStream_t s);
+// [n][3] by particle id to records by row (ids: the rows' ids) and back
+cudaError_t cheb_split(int n, const int* ids, const double* g_n3, float4* t, cudaStream_t s);
+cudaError_t cheb_join(int n, const int* ids, const float4* y, double* out_n3, cudaStream_t s);
 
 // vcorr.cu: velocity cross-correlation versus distance (Fig. vv)
 constexpr int kVcMaxBins = 1024;
 struct VcBuffers {
+    unsigned long long* fixed = nullptr; // allocation of sum, cnt, part, scal, misc and the first band
+    float4* rows = nullptr;     // allocation of p4, u4, pos_n3 and v_n3
+    int2* band_own = nullptr;   // a grown band
     double* pos_n3 = nullptr;   // [n][3] positions (particle order of the caller)
     double* v_n3 = nullptr;     // [n][3] velocities
     float4* p4 = nullptr;       // [n] FP32 positions

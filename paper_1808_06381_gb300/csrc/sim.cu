@@ -80,6 +80,25 @@ void fdt_free(FdtBuffers& V)
     cudaFree(V.bound);
     V = FdtBuffers{};
 }
+
+void sq_free(SqBuffers& Q)
+{
+    void* ptrs[] = {Q.out, Q.tw, Q.grid, Q.A};
+    for (void* q : ptrs) cudaFree(q);
+    Q = SqBuffers{};
+}
+
+template <class T>
+int sq_grow(sp_sim* s, T** p, size_t* cap, size_t want)
+{
+    if (want <= *cap) return SP_OK;
+    cudaFree(*p);
+    *p = nullptr;
+    *cap = 0;
+    SS_TRY(dev_alloc(s, p, want));
+    *cap = want;
+    return SP_OK;
+}
 }  // namespace
 
 
@@ -634,6 +653,7 @@ int sp_sim_destroy(sp_sim* s)
     DevBuffers& B = s->B;
     vc_free(s->vc);
     fdt_free(s->fdt);
+    sq_free(s->sq);
     void* ptrs[] = {B.pos_s, B.id_s, B.v_s, B.pos_w, B.pos32, B.id_w, B.cell_of, B.slot, B.perm,
                     B.cell_count, B.cell_start, B.row_cnt, B.slot_row, B.row_slot, B.chunk_len32,
                     B.chunk_off, B.col, B.img, B.val, B.val32, B.val32lo, B.hcol, B.hval, B.diag, B.partials_df,
@@ -1546,22 +1566,24 @@ int sp_sqrt_apply(sp_sim* s, int32_t degree, const double* g_host, double* xi_ho
     const KParams& P = s->kp;
     DevBuffers& B = s->B;
     const int n = P.n, np = P.npad;
-    FdtBuffers V;
-    double* planes = nullptr;   // g, then xi, as FP64 planes in the rows' order
-    int rc = fdt_alloc(s, V);
-    if (rc == SP_OK) rc = dev_alloc(s, &planes, 3 * (size_t)np);
+    if (!s->fdt.v[0]) {   // kept for the next call and for sp_set_fdt_noise
+        const int rc = fdt_alloc(s, s->fdt);
+        if (rc != SP_OK) {
+            fdt_free(s->fdt);
+            return rc;
+        }
+    }
+    FdtBuffers& V = s->fdt;
+    int rc = SP_OK;
     unsigned long long bbits = 0;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
+    if (cudaMemcpyAsync(B.stage, g_host, sizeof(double) * 3 * n, cudaMemcpyHostToDevice, s->stream) != cudaSuccess)
+        rc = SP_ERR_CUDA;
     if (rc == SP_OK) {
-        if (cudaMemcpyAsync(B.stage, g_host, sizeof(double) * 3 * n, cudaMemcpyHostToDevice, s->stream) != cudaSuccess)
-            rc = SP_ERR_CUDA;
-    }
-    if (rc == SP_OK) {
-        launch_gather_by_id(B.stage, B.id_w, n, np, planes, s->stream);
         if (P.mixed)
-            cheb_split(P, planes, static_cast<float4*>(V.v[0]), s->stream);
+            cheb_split(n, B.id_w, B.stage, static_cast<float4*>(V.v[0]), s->stream);
         else
-            cudaMemcpyAsync(V.v[0], planes, sizeof(double) * 3 * np, cudaMemcpyDeviceToDevice, s->stream);
+            launch_gather_by_id(B.stage, B.id_w, n, np, static_cast<double*>(V.v[0]), s->stream);
         if (steps_ms) {
             cudaEventCreate(&e0);
             cudaEventCreate(&e1);
@@ -1570,10 +1592,9 @@ int sp_sqrt_apply(sp_sim* s, int32_t degree, const double* g_host, double* xi_ho
         enqueue_cheb(P, B, V, degree, s->stream);
         if (steps_ms) cudaEventRecord(e1, s->stream);
         if (P.mixed)
-            cheb_join(P, static_cast<float4*>(V.v[4]), planes, s->stream);
+            cheb_join(n, B.id_w, static_cast<float4*>(V.v[4]), B.stage, s->stream);
         else
-            cudaMemcpyAsync(planes, V.v[4], sizeof(double) * 3 * np, cudaMemcpyDeviceToDevice, s->stream);
-        launch_scatter_by_id(planes, np, B.id_w, n, B.stage, s->stream);
+            launch_scatter_by_id(static_cast<double*>(V.v[4]), np, B.id_w, n, B.stage, s->stream);
         if (cudaMemcpyAsync(xi_host, B.stage, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, s->stream) !=
                 cudaSuccess ||
             cudaMemcpyAsync(&bbits, V.bound, sizeof(bbits), cudaMemcpyDeviceToHost, s->stream) != cudaSuccess ||
@@ -1593,8 +1614,6 @@ int sp_sqrt_apply(sp_sim* s, int32_t degree, const double* g_host, double* xi_ho
     if (rc == SP_ERR_CUDA) s->err = std::string("sqrt_apply: ") + cudaGetErrorString(cudaGetLastError());
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
-    fdt_free(V);
-    cudaFree(planes);
     return rc;
 }
 
@@ -1607,7 +1626,13 @@ int sp_set_fdt_noise(sp_sim* s, int32_t degree)
     }
     SS_TRY(set_device(s));
     SS_CUDA(cudaStreamSynchronize(s->stream));
-    if (degree > 0 && !s->fdt.v[0]) SS_TRY(fdt_alloc(s, s->fdt));
+    if (degree > 0 && !s->fdt.v[0]) {
+        const int rc = fdt_alloc(s, s->fdt);
+        if (rc != SP_OK) {
+            fdt_free(s->fdt);
+            return rc;
+        }
+    }
     s->fdt_degree = degree;
     free_graphs(s);   // the step graph is captured again with (or without) the noise pass
     return SP_OK;
@@ -1692,36 +1717,32 @@ int sp_structure_factor(sp_sim* s, int32_t nkx, int32_t nky, int32_t grid, doubl
     SS_TRY(read_state(s));
     const double delta = s->st_host->delta;
     const size_t m = (size_t)(2 * nkx + 1) * (2 * nky + 1);
-    double *S = nullptr, *qx = nullptr, *qy = nullptr, *tw = nullptr;
-    unsigned long long* g = nullptr;
-    double2* A = nullptr;
-    int rc = SP_OK;
-    auto A_ = [&](int r) { if (rc == SP_OK) rc = r; };
-    A_(dev_alloc(s, &S, m));
-    A_(dev_alloc(s, &qx, m));
-    A_(dev_alloc(s, &qy, m));
+    SqBuffers& Q = s->sq;
+    SS_TRY(sq_grow(s, &Q.out, &Q.out_cap, 3 * m));
     if (grid > 0) {
-        A_(dev_alloc(s, &tw, 2 * (size_t)grid));
-        A_(dev_alloc(s, &g, (size_t)grid * grid));
-        A_(dev_alloc(s, &A, (size_t)(nkx + 1) * grid + std::max(nkx, nky) / 2 + 1));   // and the windows
-    }
-    if (rc == SP_OK && grid > 0) {
-        // twiddle table (cos, sin)(2 pi m / G), m = 0..G-1
-        std::vector<double> t(2 * (size_t)grid);
-        const double two_pi = 6.283185307179586476925286766559;
-        for (int k = 0; k < grid; ++k) {
-            t[2 * k] = std::cos(two_pi * k / grid);
-            t[2 * k + 1] = std::sin(two_pi * k / grid);
+        SS_TRY(sq_grow(s, &Q.grid, &Q.grid_cap, (size_t)grid * grid));
+        SS_TRY(sq_grow(s, &Q.A, &Q.A_cap, (size_t)(nkx + 1) * grid + std::max(nkx, nky) / 2 + 1));   // and the windows
+        if (Q.G != grid) {
+            // twiddle table (cos, sin)(2 pi m / G), m = 0..G-1
+            cudaFree(Q.tw);
+            Q.tw = nullptr;
+            Q.G = 0;
+            SS_TRY(dev_alloc(s, &Q.tw, 2 * (size_t)grid));
+            std::vector<double> t(2 * (size_t)grid);
+            const double two_pi = 6.283185307179586476925286766559;
+            for (int k = 0; k < grid; ++k) {
+                t[2 * k] = std::cos(two_pi * k / grid);
+                t[2 * k + 1] = std::sin(two_pi * k / grid);
+            }
+            SS_CUDA(cudaMemcpyAsync(Q.tw, t.data(), sizeof(double) * t.size(), cudaMemcpyHostToDevice, s->stream));
+            SS_CUDA(cudaStreamSynchronize(s->stream));
+            Q.G = grid;
         }
-        if (cudaMemcpyAsync(tw, t.data(), sizeof(double) * t.size(), cudaMemcpyHostToDevice, s->stream) !=
-            cudaSuccess)
-            rc = SP_ERR_CUDA;
-        if (rc == SP_OK) SS_CUDA(cudaStreamSynchronize(s->stream));
     }
-    if (rc == SP_OK) {
-        if (run_structure_factor(s->kp, s->B, delta, grid, nkx, nky, tw, g, A, S, qx, qy, s->stream) != cudaSuccess)
-            rc = SP_ERR_CUDA;
-    }
+    double *S = Q.out, *qx = Q.out + m, *qy = Q.out + 2 * m;
+    int rc = SP_OK;
+    if (run_structure_factor(s->kp, s->B, delta, grid, nkx, nky, Q.tw, Q.grid, Q.A, S, qx, qy, s->stream) != cudaSuccess)
+        rc = SP_ERR_CUDA;
     if (rc == SP_OK) {
         if (cudaMemcpyAsync(S_host, S, sizeof(double) * m, cudaMemcpyDeviceToHost, s->stream) != cudaSuccess ||
             (qx_host && cudaMemcpyAsync(qx_host, qx, sizeof(double) * m, cudaMemcpyDeviceToHost, s->stream) != cudaSuccess) ||
@@ -1730,9 +1751,6 @@ int sp_structure_factor(sp_sim* s, int32_t nkx, int32_t nky, int32_t grid, doubl
             rc = SP_ERR_CUDA;
     }
     if (rc == SP_ERR_CUDA && s->err.empty()) s->err = std::string("structure factor: ") + cudaGetErrorString(cudaGetLastError());
-    void* ptrs[] = {S, qx, qy, tw, g, A};
-    for (void* q : ptrs)
-        if (q) cudaFree(q);
     return rc;
 }
 

@@ -39,7 +39,9 @@ struct sp_sim {
     bool learned = false;         // run the network before every solve of a step
     int mp_t = 0;                 // Adam step counter
     ss::VcBuffers vc{};           // velocity correlation (allocated by its first call)
-    ss::FdtBuffers fdt{};         // A^(1/2)-correlated noise in the steps (sp_set_fdt_noise)
+    ss::FdtBuffers fdt{};         // A^(1/2) g (sp_set_fdt_noise's steps and sp_sqrt_apply, one at a time on the
+                                  // simulation's stream; allocated by the first of them)
+    ss::SqBuffers sq{};           // structure factor (allocated by its first call)
     int fdt_degree = 0;           // 0: independent noise per particle (the paper's)
     ss::FcgState* fcg = nullptr;  // flexible solve's device state (allocated by its first call)
     ss::FcgState fcg_host{};

@@ -398,30 +398,36 @@ cudaError_t vc_alloc(T** p, long long count)
 
 void vc_free(VcBuffers& V)
 {
-    void* ptrs[] = {V.pos_n3, V.v_n3, V.p4, V.u4, V.sum, V.cnt, V.band, V.misc, V.part, V.scal, V.tiles};
+    void* ptrs[] = {V.fixed, V.rows, V.band_own, V.tiles};
     for (void* q : ptrs) cudaFree(q);
     if (V.ev[0]) cudaEventDestroy(V.ev[0]);
     if (V.ev[1]) cudaEventDestroy(V.ev[1]);
     V = VcBuffers{};
 }
 
-// Buffers for n particles (kept and reused while n does not grow).
+// Buffers for n particles (kept and reused while n does not grow): one
+// allocation for the fixed-size part and one for the rows (an allocation and
+// its release cost ~10 us each, and the call from host arrays makes all anew).
 cudaError_t vc_reserve(VcBuffers& V, long long n)
 {
     cudaError_t e = cudaSuccess;
     auto T = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
-    if (!V.sum) {   // the fixed-size part
-        T(vc_alloc(&V.sum, kVcMaxBins));
-        T(vc_alloc(&V.cnt, kVcMaxBins));
-        T(vc_alloc(&V.misc, 4));
-        T(vc_alloc(&V.part, kVcPrepBlocks));
-        T(vc_alloc(&V.scal, 2));
+    if (!V.fixed) {
         // initial capacity of the boundary-pair list (grown on demand; a small
         // value set through the environment exercises the growth)
         long long bc = 1 << 20;
         if (const char* env = getenv("SHEARSIM_VCORR_BAND_CAP")) bc = std::max(1ll, atoll(env));
-        T(vc_alloc(&V.band, bc));
-        if (e == cudaSuccess) V.band_cap = bc;
+        constexpr size_t words = 2 * kVcMaxBins + kVcPrepBlocks + 2 + 2;   // sum, cnt, part, scal, misc (8 bytes each)
+        T(vc_alloc(&V.fixed, (long long)words + bc));
+        if (e == cudaSuccess) {
+            V.sum = V.fixed;
+            V.cnt = V.sum + kVcMaxBins;
+            V.part = reinterpret_cast<double*>(V.cnt + kVcMaxBins);
+            V.scal = V.part + kVcPrepBlocks;
+            V.misc = reinterpret_cast<unsigned int*>(V.scal + 2);
+            V.band = reinterpret_cast<int2*>(V.fixed + words);
+            V.band_cap = bc;
+        }
         T(cudaEventCreate(&V.ev[0]));
         T(cudaEventCreate(&V.ev[1]));
         if (e != cudaSuccess) {
@@ -431,11 +437,14 @@ cudaError_t vc_reserve(VcBuffers& V, long long n)
     }
     if (n > V.n_cap) {
         V.n_cap = 0;
-        T(vc_alloc(&V.pos_n3, 3 * n));
-        T(vc_alloc(&V.v_n3, 3 * n));
-        T(vc_alloc(&V.p4, n));
-        T(vc_alloc(&V.u4, n));
-        if (e == cudaSuccess) V.n_cap = n;
+        T(vc_alloc(&V.rows, 5 * n));   // p4, u4 (16 bytes a row), pos_n3, v_n3 (24)
+        if (e == cudaSuccess) {
+            V.p4 = V.rows;
+            V.u4 = V.p4 + n;
+            V.pos_n3 = reinterpret_cast<double*>(V.u4 + n);
+            V.v_n3 = V.pos_n3 + 3 * n;
+            V.n_cap = n;
+        }
     }
     return e;
 }
@@ -561,11 +570,12 @@ int run_velocity_correlation(VcBuffers& V, long long n, const double L[3], doubl
         // more pairs near a boundary than the list holds: grow it and run again
         const long long want = (long long)misc_h[0] + (misc_h[0] >> 2) + 1024;
         V.band_cap = 0;
-        if (attempt == 1 || vc_alloc(&V.band, want) != cudaSuccess) {
+        if (attempt == 1 || vc_alloc(&V.band_own, want) != cudaSuccess) {
             cudaGetLastError();
             if (err) *err = "velocity correlation: boundary pair list overflow";
             return SP_ERR_OOM;
         }
+        V.band = V.band_own;
         V.band_cap = want;
     }
     const double S = scal_h[1];
