@@ -98,29 +98,43 @@ void launch_integrate(const KParams& P, DevBuffers& B, Launch L, bool commit)
 // Eq. vc (times zeta): f_ij = c_ev R_ij w_ij + zeta alpha w_ij (v_j - v_i + V_ij).
 // y_ij f_ij,x is symmetric in (i, j), so each row sums its whole neighbour list
 // and the total is halved.  Separations come from the stored image codes and
-// weights from the assembled matrix.
+// weights from the assembled matrix.  Bound by GB300's FP64 pipe: the rows come
+// in slot order (a warp's rows equally long), kStressSplit threads share a row
+// (a small system's rows are chains too few to fill the SMs), and a warp whose
+// current entries all pair with the central image skips the image shifts (7
+// FP64 operations an entry instead of ~20): n = 500 53 us, n = 60,013 141 us with
+// one thread per row in row order, 20 and 51 us now.
+constexpr int kStressSplit = 4;
 __global__ void __launch_bounds__(kVecBlock) k_stress(KParams P, DevBuffers B)
 {
     DevState* st = B.st;
     if (st->error | st->overflow) return;
     const int np = P.npad;
-    const double delta = st->delta;
+    const double delta = st->delta, za = P.zeta * P.alpha, kl = P.kappa * P.L[1];
+    const int center = image_code(0, 0, 0);
     double acc = 0.0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P.n; i += gridDim.x * blockDim.x) {
-        const double xi = B.pos_w[i], yi = B.pos_w[np + i], zi = B.pos_w[2 * np + i];
-        const double vxi = B.x[i];
-        const int slot = B.row_slot[i];
-        const int base = B.chunk_off[slot >> 5] + (slot & 31);
-        const int cnt = B.row_cnt[i];
-        for (int k = 0; k < cnt; ++k) {
+    // thread t of a block: slot t % 32 of a chunk, entries (t / 32) % split, ... (whole warps share both)
+    for (int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < P.nchunks * kStressSplit;
+         c += (gridDim.x * blockDim.x) >> 5) {
+        const int chunk = c / kStressSplit, slot = 32 * chunk + (threadIdx.x & 31);
+        const int i = B.slot_row[slot];
+        if (i < 0) continue;
+        const double xi = B.pos_w[i], yi = B.pos_w[np + i], vxi = B.x[i];
+        const int base = B.chunk_off[chunk] + (slot & 31), cnt = B.row_cnt[i];
+        for (int k = c % kStressSplit; k < cnt; k += kStressSplit) {
             const int e = base + 32 * k;
-            const int j = B.col[e];
-            double dx, dy, dz;
-            const double nimg = image_separation(P, delta, xi, yi, zi, B.pos_w[j], B.pos_w[np + j],
-                                                 B.pos_w[2 * np + j], B.img[e], dx, dy, dz);
-            const double w = B.val[e];
-            const double fx = P.c_ev * dx * w + P.zeta * P.alpha * w * (B.x[j] - vxi + P.kappa * P.L[1] * nimg);
-            acc += dy * fx;
+            const int j = B.col[e], code = B.img[e];
+            double dx = xi - B.pos_w[j], dy = yi - B.pos_w[np + j], dv = B.x[j] - vxi;
+            if (!__all_sync(__activemask(), code == center)) {
+                const int a = (code & 7) - 2, m = ((code >> 3) & 3) - 1;
+                if (m != 0) {
+                    dx -= m > 0 ? delta : -delta;
+                    dy -= m > 0 ? P.L[1] : -P.L[1];
+                    dv += m > 0 ? kl : -kl;
+                }
+                if (a != 0) dx -= P.L[0] * (double)a;
+            }
+            acc = fma(dy, B.val[e] * fma(P.c_ev, dx, za * dv), acc);
         }
     }
     const double v[1] = {acc};
@@ -137,8 +151,13 @@ __global__ void __launch_bounds__(kVecBlock) k_stress(KParams P, DevBuffers B)
 // relative for the boxes used here), weights from the FP32 matrix, FP32
 // velocities, and a double-float accumulation.  Each pair once (the entry of
 // its lower row; y_ij f_ij,x is symmetric in i and j), so half the gathers.
+// In a small system SPLIT neighbouring lanes share a row (each batch's entries
+// are every SPLIT-th): n = 20,011 31 us -> 14, 48,000 31 -> 20, 100,000 33 -> 29;
+// from kStress32SplitRows on one thread per row fills the SMs by itself.
 constexpr int kStressBatch = 4;   // entries requested at a time
+constexpr int kStress32SplitRows = 130000;
 
+template <int SPLIT>
 __global__ void __launch_bounds__(kVecBlock) k_stress32(KParams P, DevBuffers B)
 {
     DevState* st = B.st;
@@ -154,22 +173,23 @@ __global__ void __launch_bounds__(kVecBlock) k_stress32(KParams P, DevBuffers B)
     // floats at the FP64 rate); velocities from the solver's double-float x
     auto sel = [](int k, float v) { return k == 0 ? 0.f : (k > 0 ? v : -v); };
     dfloat acc{0.f, 0.f};
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P.n; i += gridDim.x * blockDim.x) {
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < P.n * SPLIT; t += gridDim.x * blockDim.x) {
+        const int i = t / SPLIT, sub = t % SPLIT;
         const float xi = B.pos32[i], yi = B.pos32[np + i];
         const float vxi = B.xdf[2 * i].x;
         const int slot = B.row_slot[i];
         const int base = B.chunk_off[slot >> 5] + (slot & 31);
         const int cnt = B.row_cnt[i];
         float row = 0.f;
-        for (int kb = 0; kb < cnt; kb += kStressBatch) {
+        for (int kb = sub; kb < cnt; kb += kStressBatch * SPLIT) {
             int j[kStressBatch], code[kStressBatch];
             float w[kStressBatch];
 #pragma unroll
             for (int u = 0; u < kStressBatch; ++u) {
-                const int e = base + 32 * (kb + u);
-                j[u] = kb + u < cnt ? B.col[e] : i;
-                code[u] = kb + u < cnt ? (int)B.img[e] : image_code(0, 0, 0);
-                w[u] = kb + u < cnt ? B.val32[e] : 0.f;
+                const int k = kb + u * SPLIT, e = base + 32 * k;
+                j[u] = k < cnt ? B.col[e] : i;
+                code[u] = k < cnt ? (int)B.img[e] : image_code(0, 0, 0);
+                w[u] = k < cnt ? B.val32[e] : 0.f;
             }
 #pragma unroll
             for (int u = 0; u < kStressBatch; ++u) {
@@ -192,10 +212,12 @@ __global__ void __launch_bounds__(kVecBlock) k_stress32(KParams P, DevBuffers B)
 
 void launch_stress(const KParams& P, DevBuffers& B, bool mixed, Launch L)
 {
-    if (mixed)
-        k_stress32<<<grid_for(P.n, kVecBlock, L.num_sms * 8), kVecBlock, 0, L.stream>>>(P, B);
+    if (!mixed)
+        k_stress<<<grid_for(32ll * P.nchunks * kStressSplit, kVecBlock, L.num_sms * 8), kVecBlock, 0, L.stream>>>(P, B);
+    else if (P.n < kStress32SplitRows)
+        k_stress32<8><<<grid_for(8ll * P.n, kVecBlock, L.num_sms * 8), kVecBlock, 0, L.stream>>>(P, B);
     else
-        k_stress<<<grid_for(P.n, kVecBlock, L.num_sms * 8), kVecBlock, 0, L.stream>>>(P, B);
+        k_stress32<1><<<grid_for(P.n, kVecBlock, L.num_sms * 8), kVecBlock, 0, L.stream>>>(P, B);
 }
 
 __global__ void k_scatter_by_id(const double* __restrict__ planes, int npad, const int* __restrict__ ids,

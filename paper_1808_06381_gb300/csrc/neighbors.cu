@@ -10,6 +10,7 @@
 // close in memory for the solver's gathers.
 #include <array>
 #include <cmath>
+#include <type_traits>
 
 #include "internal.cuh"
 
@@ -426,13 +427,16 @@ __device__ __forceinline__ void for_each_neighbor_generic(const KParams& P, doub
 // edge is >= 3 r_c, so the image found here is the canonical minimum image of
 // every accepted pair.  FP32 arithmetic uses explicit round-to-nearest
 // intrinsics so that the counting and filling passes decide identically.
+// The nine (z, y) rows of three cells are numbered 0..8; rows zy0..zy1 - 1 are
+// visited (all of them, or one by each of nine threads that share a particle).
 template <class F>
 __device__ __forceinline__ void for_each_neighbor_fast(const KParams& P, double delta,
                                                        const double* __restrict__ pos,
                                                        const float* __restrict__ pos32,
                                                        const int* __restrict__ cell_start,
                                                        const int* __restrict__ cell_w, int i,
-                                                       double xi, double yi, double zi, F&& visit)
+                                                       double xi, double yi, double zi, F&& visit, int zy0 = 0,
+                                                       int zy1 = 9)
 {
     const int np = P.npad;
     const int nc0 = P.nc[0], nc1 = P.nc[1], nc2 = P.nc[2];
@@ -457,7 +461,7 @@ __device__ __forceinline__ void for_each_neighbor_fast(const KParams& P, double 
     // at the FP64 rate); every product below is exact, as before
     auto times = [](int k, float v) { return k == 0 ? 0.f : (k > 0 ? v : -v); };
     const float L2f = 2.f * P.Lf[0];
-    for (int dzc = -1; dzc <= 1; ++dzc) {
+    for (int dzc = zy0 / 3 - 1; dzc <= (zy1 - 1) / 3 - 1; ++dzc) {
         int czz = cz + dzc, c_img = 0;
         if (czz < 0) {
             czz += nc2;
@@ -467,7 +471,7 @@ __device__ __forceinline__ void for_each_neighbor_fast(const KParams& P, double 
             c_img = 1;
         }
         const float szf = times(c_img, P.Lf[2]);
-        for (int dyc = -1; dyc <= 1; ++dyc) {
+        for (int dyc = zy1 - zy0 == 1 ? zy0 % 3 - 1 : -1; dyc <= (zy1 - zy0 == 1 ? zy0 % 3 - 1 : 1); ++dyc) {
             int cyy = cy + dyc, m = 0;
             if (cyy < 0) {
                 cyy += nc1;
@@ -571,6 +575,54 @@ __global__ void k_nbr_collect(KParams P, DevBuffers B, int draw_noise)
     B.row_cnt[i] = cnt;
 }
 
+// The same search for small systems, nine threads per row: thread part of a row
+// walks one (z, y) row of three cells, counts, and after the counts of the parts
+// before it walks again and writes from there, so the list is the one of the
+// whole walk in its order.  With one thread per row a system of a few thousand
+// rows is a few warps per SM, each a chain of ~100 dependent loads (count, scan and
+// fill together: n = 500 67 us -> 46, n = 20,011 81 -> 57); at kSplitSearchRows both
+// take the same time, and beyond it the single threads fill the SMs and the second
+// walk costs more than it saves (n = 60,013: 94 us single, 107 split).
+constexpr int kSplitRows = 32;            // rows per block of 9 x 32 threads
+constexpr int kSplitSearchRows = 48000;
+__global__ void __launch_bounds__(9 * kSplitRows) k_nbr_collect_split(KParams P, DevBuffers B, int draw_noise)
+{
+    DevState* st = B.st;
+    if (st->error | st->overflow) return;
+    __shared__ int found[9][kSplitRows];
+    const int r = threadIdx.x % kSplitRows, part = threadIdx.x / kSplitRows;   // a warp: 32 rows, the same part
+    const int i = blockIdx.x * kSplitRows + r;
+    if (i == 0 && part == 0) {
+        st->nnz = 0;
+        st->noise_step = draw_noise == 2 ? st->noise_step : -1;   // 2: drawn by k_row_normals
+    }
+    const int np = P.npad;
+    const double delta = st->delta;
+    const double xi = i < P.n ? B.pos_w[i] : 0.0, yi = i < P.n ? B.pos_w[np + i] : 0.0, zi = i < P.n ? B.pos_w[2 * np + i] : 0.0;
+    int cnt = 0;
+    if (i < P.n)
+        for_each_neighbor_fast(P, delta, B.pos_w, B.pos32, B.cell_start, B.cell_of, i, xi, yi, zi,
+                               [&](int, unsigned char) { ++cnt; }, part, part + 1);
+    found[part][r] = cnt;
+    __syncthreads();
+    if (i >= P.n) return;
+    int at = 0;
+    for (int k = 0; k < part; ++k) at += found[k][r];
+    if (part == 8) B.row_cnt[i] = at + cnt;
+    if (cnt == 0 || at >= kCandCap) return;
+    int* __restrict__ cj = B.cand_j;
+    unsigned char* __restrict__ ci = B.cand_img;
+    for_each_neighbor_fast(P, delta, B.pos_w, B.pos32, B.cell_start, B.cell_of, i, xi, yi, zi,
+                           [&](int j, unsigned char code) {
+                               if (at < kCandCap) {
+                                   cj[(size_t)at * np + i] = j;
+                                   ci[(size_t)at * np + i] = code;
+                               }
+                               ++at;
+                           },
+                           part, part + 1);
+}
+
 // The step's normals of every row as the pair search draws them, in a kernel
 // of their own (so that they can run beside the search).
 __global__ void k_row_normals(KParams P, DevBuffers B)
@@ -598,14 +650,30 @@ __global__ void k_row_normals(KParams P, DevBuffers B)
 
 int launch_nbr_count(const KParams& P, DevBuffers& B, bool draw_noise, Launch L, cudaStream_t side, cudaEvent_t* ev)
 {
+    const bool split = P.fast_cells && P.n < kSplitSearchRows;
+    auto search = [&](int mode) {
+        if (split)
+            k_nbr_collect_split<<<grid_for(P.n, kSplitRows, 1 << 30), 9 * kSplitRows, 0, L.stream>>>(P, B, mode);
+        else
+            k_nbr_collect<<<grid_for(P.n, 128, 1 << 30), 128, 0, L.stream>>>(P, B, mode);
+    };
     if (draw_noise && side && ev) {   // the normals beside the search, joined before anything after it
         cudaEventRecord(ev[0], L.stream);
         cudaStreamWaitEvent(side, ev[0], 0);
         k_row_normals<<<grid_for(P.n, 256, 1 << 30), 256, 0, side>>>(P, B);
         cudaEventRecord(ev[1], side);
-        k_nbr_collect<<<grid_for(P.n, 128, 1 << 30), 128, 0, L.stream>>>(P, B, 2);
+        search(2);
         cudaStreamWaitEvent(L.stream, ev[1], 0);
         return 2;
+    }
+    if (split && draw_noise) {   // the normals as a kernel of their own
+        k_row_normals<<<grid_for(P.n, 256, 1 << 30), 256, 0, L.stream>>>(P, B);
+        search(2);
+        return 2;
+    }
+    if (split) {
+        search(0);
+        return 1;
     }
     k_nbr_collect<<<grid_for(P.n, 128, 1 << 30), 128, 0, L.stream>>>(P, B, draw_noise ? 1 : 0);
     return 1;
@@ -878,15 +946,41 @@ __device__ __forceinline__ dfloat sep_df(float ih, float il, float jh, float jl,
 // FP64 assembly to ~1e-12 relative (the 2^-48 representation of the
 // positions), far inside the mixed solver's tolerance.
 constexpr int kAsmBatch = 4;   // partners requested at a time by the double-float assembly
+constexpr int kAsmSplit = 4;   // warps per chunk of 32 rows in systems below kSplitAssemblyRows
+constexpr int kSplitAssemblyRows = 1 << 19;
 
-template <bool DF>
+// SPLIT warps share a chunk of 32 rows, each taking every SPLIT-th entry, and
+// the first of them sums their sums and finishes the rows: in a small system
+// one thread per row leaves most SMs without a warp and every warp with one
+// long chain (FP64: ~25 operations an entry at GB300's 1/64 rate).  n = 500 FP64:
+// 74 us with one thread per row, 31 now; n = 4,096 FP64 105 -> 35, n = 60,013 FP64
+// 186 -> 105, n = 20,011 mixed 127 -> 21, n = 262,144 mixed 112 -> 100.  From
+// kSplitAssemblyRows on the SMs are full either way and the sums through shared
+// memory only cost (n = 4,194,304 mixed: 1,407 us split, 1,163 single).
+template <bool DF, int SPLIT>
 __global__ void __launch_bounds__(256, 3) k_assemble_slots(KParams P, DevBuffers B, int use_inj)
 {
     const DevState* st = B.st;
     if (st->error | st->overflow) return;
-    const int slot = blockIdx.x * 256 + threadIdx.x;
+    const int sub = (threadIdx.x >> 5) % SPLIT;
+    const int slot = blockIdx.x * (256 / SPLIT) + ((threadIdx.x >> 5) / SPLIT) * 32 + (threadIdx.x & 31);
     const int i = B.slot_row[slot];
-    if (i < 0) return;
+    if (SPLIT == 1 && i < 0) return;
+    using Sum = typename std::conditional<DF, dfloat, double>::type;
+    __shared__ Sum part[SPLIT > 1 ? SPLIT - 1 : 1][5][SPLIT > 1 ? 256 / SPLIT : 1];
+    const int in_block = ((threadIdx.x >> 5) / SPLIT) * 32 + (threadIdx.x & 31);
+    bool wide = false;   // a row with more than kCandCap partners: searched again by its first thread
+    if (SPLIT > 1) {
+        if (i >= 0 && B.row_cnt[i] > kCandCap) {
+            wide = true;
+            if (sub == 0)
+                search_row_into_slots(P, B, i, st->delta, B.chunk_off[slot >> 5] + (slot & 31), B.row_cnt[i]);
+        }
+        __syncthreads();
+    }
+    double sw = 0.0, fx = 0.0, fy = 0.0, fz = 0.0, nw = 0.0;
+    dfloat dsw{0.f, 0.f}, dsx{0.f, 0.f}, dsy{0.f, 0.f}, dsz{0.f, 0.f}, dsn{0.f, 0.f};
+    if (SPLIT == 1 || i >= 0) {
     const double delta = st->delta;
     const int np = P.npad;
     const double xi = B.pos_w[i], yi = B.pos_w[np + i], zi = B.pos_w[2 * np + i];
@@ -899,14 +993,12 @@ __global__ void __launch_bounds__(256, 3) k_assemble_slots(KParams P, DevBuffers
     const int* __restrict__ pj = B.cand_j + i;
     const unsigned char* __restrict__ pimg = B.cand_img + i;
     size_t pstride = (size_t)np;
-    if (cnt > kCandCap) {
-        search_row_into_slots(P, B, i, delta, base, cnt);
+    if (SPLIT == 1 ? cnt > kCandCap : wide) {
+        if (SPLIT == 1) search_row_into_slots(P, B, i, delta, base, cnt);
         pj = B.col + base;
         pimg = B.img + base;
         pstride = 32;
     }
-    double sw = 0.0, fx = 0.0, fy = 0.0, fz = 0.0, nw = 0.0;
-    dfloat dsw{0.f, 0.f}, dsx{0.f, 0.f}, dsy{0.f, 0.f}, dsz{0.f, 0.f}, dsn{0.f, 0.f};
     if (DF) {
         const float* __restrict__ ph = B.pos32;
         const float* __restrict__ pl = B.pos32lo;
@@ -919,13 +1011,13 @@ __global__ void __launch_bounds__(256, 3) k_assemble_slots(KParams P, DevBuffers
         dfloat s_w = zero, s_x = zero, s_y = zero, s_z = zero, s_n = zero;
         // partners in batches of kAsmBatch: their indices, then their positions,
         // are requested together (one latency per batch, not per partner)
-        for (int k0 = 0; k0 < cnt; k0 += kAsmBatch) {
+        for (int k0 = sub; k0 < cnt; k0 += kAsmBatch * SPLIT) {
         int jb[kAsmBatch], cb[kAsmBatch];
 #pragma unroll
         for (int u = 0; u < kAsmBatch; ++u) {
-            const bool in = k0 + u < cnt;
-            jb[u] = in ? pj[(k0 + u) * pstride] : i;
-            cb[u] = in ? pimg[(k0 + u) * pstride] : center;
+            const int k = k0 + u * SPLIT;
+            jb[u] = k < cnt ? pj[k * pstride] : i;
+            cb[u] = k < cnt ? pimg[k * pstride] : center;
         }
         float pxh[kAsmBatch], pxl[kAsmBatch], pyh[kAsmBatch], pyl[kAsmBatch], pzh[kAsmBatch], pzl[kAsmBatch];
 #pragma unroll
@@ -940,7 +1032,7 @@ __global__ void __launch_bounds__(256, 3) k_assemble_slots(KParams P, DevBuffers
         }
 #pragma unroll
         for (int u = 0; u < kAsmBatch; ++u) {
-            const int k = k0 + u;
+            const int k = k0 + u * SPLIT;
             if (k >= cnt) break;
             const int e = base + 32 * k;
             const int j = jb[u];
@@ -987,7 +1079,7 @@ __global__ void __launch_bounds__(256, 3) k_assemble_slots(KParams P, DevBuffers
     } else {
         const double Lx = P.L[0], Ly = P.L[1], Lz = P.L[2];
         const double* __restrict__ pos = B.pos_w;
-        for (int k = 0; k < cnt; ++k) {
+        for (int k = sub; k < cnt; k += SPLIT) {
             const int e = base + 32 * k;
             const int j = pj[k * pstride];
             const int code = pimg[k * pstride];
@@ -1020,7 +1112,7 @@ __global__ void __launch_bounds__(256, 3) k_assemble_slots(KParams P, DevBuffers
             if (shifted) nw += m == 0 ? 0.0 : (m > 0 ? w : -w);
         }
     }
-    for (int k = cnt; k < clen; ++k) {
+    for (int k = cnt + sub; k < clen; k += SPLIT) {
         B.col[base + 32 * k] = i;
         B.img[base + 32 * k] = (unsigned char)center;
         B.val32[base + 32 * k] = 0.f;
@@ -1029,12 +1121,42 @@ __global__ void __launch_bounds__(256, 3) k_assemble_slots(KParams P, DevBuffers
         else
             B.val[base + 32 * k] = 0.0;
     }
+    }
+    const int np = P.npad;
+    if constexpr (SPLIT > 1) {   // the row's sums in the order of the warps
+        if (sub > 0) {
+            if constexpr (DF) {
+                const dfloat v[5] = {dsw, dsx, dsy, dsz, dsn};
+                for (int q = 0; q < 5; ++q) part[sub - 1][q][in_block] = v[q];
+            } else {
+                const double v[5] = {sw, fx, fy, fz, nw};
+                for (int q = 0; q < 5; ++q) part[sub - 1][q][in_block] = v[q];
+            }
+        }
+        __syncthreads();
+        if (sub > 0 || i < 0) return;
+        for (int w = 0; w < SPLIT - 1; ++w) {
+            if constexpr (DF) {
+                dsw = df_add(dsw, part[w][0][in_block]);
+                dsx = df_add(dsx, part[w][1][in_block]);
+                dsy = df_add(dsy, part[w][2][in_block]);
+                dsz = df_add(dsz, part[w][3][in_block]);
+                dsn = df_add(dsn, part[w][4][in_block]);
+            } else {
+                sw += part[w][0][in_block];
+                fx += part[w][1][in_block];
+                fy += part[w][2][in_block];
+                fz += part[w][3][in_block];
+                nw += part[w][4][in_block];
+            }
+        }
+    }
     if (DF)
         finish_row_df(P, B, i, dfloat{B.pos32[np + i], B.pos32lo[np + i]}, (unsigned long long)st->step, use_inj,
                       st->noise_step == st->step, dsw, dsx, dsy, dsz, dsn);
     else
-        finish_row(P, B, i, yi, (unsigned long long)st->step, use_inj, st->noise_step == st->step, sw, fx, fy, fz,
-                   nw);
+        finish_row(P, B, i, B.pos_w[np + i], (unsigned long long)st->step, use_inj, st->noise_step == st->step, sw, fx,
+                   fy, fz, nw);
 }
 
 // Pair search writing the sliced columns and image codes (FP32 decisions).
@@ -1082,10 +1204,18 @@ int launch_nbr_fill(const KParams& P, DevBuffers& B, bool assemble, bool use_inj
 // Assembly from existing pairs (df: double-float entries, the mixed-precision path).
 void launch_assemble_only(const KParams& P, DevBuffers& B, bool use_inj, bool df, Launch L)
 {
-    if (df)
-        k_assemble_slots<true><<<P.nslots / 256, 256, 0, L.stream>>>(P, B, use_inj ? 1 : 0);
-    else
-        k_assemble_slots<false><<<P.nslots / 256, 256, 0, L.stream>>>(P, B, use_inj ? 1 : 0);
+    const int inj = use_inj ? 1 : 0;
+    if (P.n < kSplitAssemblyRows) {
+        const int grid = P.nslots / (256 / kAsmSplit);
+        if (df)
+            k_assemble_slots<true, kAsmSplit><<<grid, 256, 0, L.stream>>>(P, B, inj);
+        else
+            k_assemble_slots<false, kAsmSplit><<<grid, 256, 0, L.stream>>>(P, B, inj);
+    } else if (df) {
+        k_assemble_slots<true, 1><<<P.nslots / 256, 256, 0, L.stream>>>(P, B, inj);
+    } else {
+        k_assemble_slots<false, 1><<<P.nslots / 256, 256, 0, L.stream>>>(P, B, inj);
+    }
 }
 
 // ------------------------------------------------------ generator utilities
