@@ -154,50 +154,16 @@ __device__ __forceinline__ f2 f2_rint(f2 x)
     return f2_add(f2_add(x, f2_both(12582912.f)), f2_both(-12582912.f));
 }
 
+__device__ __forceinline__ f2 f2_add_rd(f2 a, f2 b)   // both rounded down
+{
+    f2 r;
+    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
 constexpr int kVcSegment = 64;    // tile particles between two emptyings of the histograms
 constexpr int kVcListed = 1024;   // listed pairs held in shared memory per segment
 constexpr int kVcCountBit = 19;   // histogram word A: 7 low bits of the product (sum below 2^19), count from here
-
-// The decisions of one pair (separation d, squared length r2, product bits qb
-// = 0x4B400000 + round(dot S)): the pair goes to the warp's histogram, or to
-// the FP64 list when one of its decisions lies within the FP32 error bound of a
-// boundary (an image index taken within the FP32 error of a tie leaves that
-// component within the same error of half the box edge).
-__device__ __forceinline__ void vc_pair(const VcConst& C, float dx, float dy, float dz, float r2, unsigned int qb,
-                                        unsigned int* hw, int hb, unsigned int code, unsigned int* listed,
-                                        unsigned int* nlisted, int2* band, unsigned int* band_n,
-                                        unsigned int band_cap, int i, int j)
-{
-    const bool tie = fabsf(dx) > C.half[0] || fabsf(dy) > C.half[1] || fabsf(dz) > C.half[2];
-    bool push = tie;
-    if (!tie && r2 < C.r2_hi) {
-        // |R| from the reciprocal square root (within 3 ulp; the bands allow for it)
-        float rs;
-        asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rs) : "f"(fmaxf(r2, 1e-30f)));
-        const float r = r2 * rs;
-        const float t = r * C.inv_f;
-        const float tk = __fadd_rd(t, 8388608.f);   // 2^23 + floor(t) (0 <= t < 2^23)
-        const float fr = t - (tk - 8388608.f);      // exact
-        if (r > C.r_band || fr < C.eb || fr > 1.f - C.eb) {
-            push = true;
-        } else {
-            const int k = __float_as_int(tk) - 0x4B000000;
-            // m = round(dot S) + 2^22 (|dot S| < 2^21): its low 7 bits and a count
-            // of 1 in word A, its high 16 bits in word B
-            atomicAdd(hw + k, (qb & 127u) | (1u << kVcCountBit));
-            atomicAdd(hw + hb + k, (qb >> 7) & 0xffffu);
-        }
-    }
-    if (push) {   // rare (a few per thousand pairs)
-        const unsigned int at = atomicAdd(nlisted, 1u);
-        if (at < kVcListed) {
-            listed[at] = code;
-        } else {   // a dense segment: straight to the list
-            const unsigned int idx = atomicAdd(band_n, 1u);
-            if (idx < band_cap) band[idx] = make_int2(i, j);
-        }
-    }
-}
 
 // Block (I, J0): particles i = 512 I + tid and 512 I + 256 + tid against the
 // c' tiles J0 .. J0 + chunk - 1 (256 particles each).
@@ -210,9 +176,11 @@ __global__ void __launch_bounds__(kVcTile) k_vc_pairs(VcConst C, const float4* _
                                                         unsigned int band_cap)
 {
     extern __shared__ float4 vc_smem[];
-    float4* sp = vc_smem;                  // [kVcTile] positions of the c' tile, negated
-    float4* su = sp + kVcTile;             // [kVcTile] their u
-    unsigned int* listed = reinterpret_cast<unsigned int*>(su + kVcTile);   // [kVcListed] local codes of listed pairs
+    // the c' tile with every value twice, as the packed operations take it:
+    // (-x, -x, -y, -y), (-z, -z, u_x, u_x), (u_y, u_y, u_z, u_z)
+    float4* sp = vc_smem;
+    const ulonglong2* spd = reinterpret_cast<const ulonglong2*>(sp);
+    unsigned int* listed = reinterpret_cast<unsigned int*>(sp + 3 * kVcTile);   // [kVcListed] local codes of listed pairs
     // per-warp histograms of a segment, two 32-bit words per bin: a warp adds at
     // most 64 x 64 = 2^12 pairs to a bin, so word A holds the count above its 7
     // low bits' sum and word B (16 bits a pair) stays below 2^28
@@ -240,41 +208,85 @@ __global__ void __launch_bounds__(kVcTile) k_vc_pairs(VcConst C, const float4* _
     unsigned long long cnt[kOwn];
 #pragma unroll
     for (int u = 0; u < kOwn; ++u) sum[u] = 0, cnt[u] = 0ull;
+    const f2 nLx = f2_both(-C.Lf[0]), nLy = f2_both(-C.Lf[1]), nLz = f2_both(-C.Lf[2]), nDf = f2_both(-C.df);
+    const f2 iLx = f2_both(C.iLf[0]), iLy = f2_both(C.iLf[1]), iLz = f2_both(C.iLf[2]);
+    const f2 S2 = f2_both(S), magic = f2_both(12582912.f), inv2 = f2_both(C.inv_f), p23 = f2_both(8388608.f);
+    const f2 m23 = f2_both(-8388608.f), neg1 = f2_both(-1.f);
+    const float hx = C.half[0], hy = C.half[1], hz = C.half[2], one_eb = 1.f - C.eb;
+    // a rare pair (a few per thousand) to the segment's list, or straight to the global one
+    auto list = [&](unsigned int code, int i, int j) {
+        const unsigned int at = atomicAdd(&nlisted, 1u);
+        if (at < kVcListed) {
+            listed[at] = code;
+        } else {
+            const unsigned int idx = atomicAdd(band_n, 1u);
+            if (idx < band_cap) band[idx] = make_int2(i, j);
+        }
+    };
     auto segment = [&](auto diag, int J, int b, int e) {
         for (int jj = b; jj < e; ++jj) {
             const int j = J * kVcTile + jj;
-            const float4 pj = sp[jj], uj = su[jj];
-            f2 dx = f2_add(X, f2_both(pj.x)), dy = f2_add(Y, f2_both(pj.y)), dz = f2_add(Z, f2_both(pj.z));
-            const f2 ny = f2_rint(f2_mul(dy, f2_both(C.iLf[1])));
-            dy = f2_fma(ny, f2_both(-C.Lf[1]), dy);
-            dx = f2_fma(ny, f2_both(-C.df), dx);
-            dx = f2_fma(f2_rint(f2_mul(dx, f2_both(C.iLf[0]))), f2_both(-C.Lf[0]), dx);
-            dz = f2_fma(f2_rint(f2_mul(dz, f2_both(C.iLf[2]))), f2_both(-C.Lf[2]), dz);
+            const ulonglong2 ja = spd[jj], jb = spd[kVcTile + jj], jc = spd[2 * kVcTile + jj];
+            f2 dx = f2_add(X, ja.x), dy = f2_add(Y, ja.y), dz = f2_add(Z, jb.x);
+            const f2 ny = f2_rint(f2_mul(dy, iLy));
+            dy = f2_fma(ny, nLy, dy);
+            dx = f2_fma(ny, nDf, dx);
+            dx = f2_fma(f2_rint(f2_mul(dx, iLx)), nLx, dx);
+            dz = f2_fma(f2_rint(f2_mul(dz, iLz)), nLz, dz);
             const f2 r2 = f2_fma(dx, dx, f2_fma(dy, dy, f2_mul(dz, dz)));
-            const f2 dot = f2_fma(UX, f2_both(uj.x), f2_fma(UY, f2_both(uj.y), f2_mul(UZ, f2_both(uj.z))));
-            const f2 q = f2_fma(dot, f2_both(S), f2_both(12582912.f));
-            float ax, ay, az, ar, aq, bx, by, bz, br, bq;
+            const f2 q = f2_fma(f2_fma(UX, jb.y, f2_fma(UY, jc.x, f2_mul(UZ, jc.y))), S2, magic);
+            float ax, ay, az, ar, aq, bx, by, bz, br, bq, as, bs;
             f2_get(dx, ax, bx);
             f2_get(dy, ay, by);
             f2_get(dz, az, bz);
             f2_get(r2, ar, br);
             f2_get(q, aq, bq);
-            const unsigned int code = (unsigned int)tid | ((unsigned int)jj << 9);
-            if (!decltype(diag)::value || j > i0)
-                vc_pair(C, ax, ay, az, ar, __float_as_uint(aq), hw, hb, code, listed, &nlisted, band, band_n, band_cap,
-                        i0, j);
-            if (!decltype(diag)::value || j > i1)
-                vc_pair(C, bx, by, bz, br, __float_as_uint(bq), hw, hb, code | kVcTile, listed, &nlisted, band, band_n,
-                        band_cap, i1, j);
+            // |R| from the reciprocal square root (within 3 ulp; the bands allow for it),
+            // its bin position t, 2^23 + floor(t) (0 <= t < 2^23) and t's fraction (exact)
+            asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(as) : "f"(fmaxf(ar, 1e-30f)));
+            asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(bs) : "f"(fmaxf(br, 1e-30f)));
+            const f2 r = f2_mul(r2, f2_make(as, bs)), t = f2_mul(r, inv2);
+            const f2 tk = f2_add_rd(t, p23), fr = f2_fma(f2_add(tk, m23), neg1, t);
+            float ra, rb, ta, tb2, fa, fb;
+            f2_get(r, ra, rb);
+            f2_get(tk, ta, tb2);
+            f2_get(fr, fa, fb);
+            // an image index taken within the FP32 error of a tie leaves that component
+            // within the same error of half the box edge
+            const bool in_a = !decltype(diag)::value || j > i0, in_b = !decltype(diag)::value || j > i1;
+            const bool tie_a = fabsf(ax) > hx || fabsf(ay) > hy || fabsf(az) > hz;
+            const bool tie_b = fabsf(bx) > hx || fabsf(by) > hy || fabsf(bz) > hz;
+            const bool near_a = ra > C.r_band || fa < C.eb || fa > one_eb;
+            const bool near_b = rb > C.r_band || fb < C.eb || fb > one_eb;
+            const bool cut_a = ar < C.r2_hi, cut_b = br < C.r2_hi;
+            // m = round(dot S) + 2^22 (|dot S| < 2^21): its low 7 bits and a count of 1
+            // in word A, its high 16 bits in word B
+            if (in_a && !tie_a && cut_a && !near_a) {
+                unsigned int* h = hw + (__float_as_int(ta) - 0x4B000000);
+                atomicAdd(h, (__float_as_uint(aq) & 127u) | (1u << kVcCountBit));
+                atomicAdd(h + hb, (__float_as_uint(aq) >> 7) & 0xffffu);
+            }
+            if (in_b && !tie_b && cut_b && !near_b) {
+                unsigned int* h = hw + (__float_as_int(tb2) - 0x4B000000);
+                atomicAdd(h, (__float_as_uint(bq) & 127u) | (1u << kVcCountBit));
+                atomicAdd(h + hb, (__float_as_uint(bq) >> 7) & 0xffffu);
+            }
+            const bool push_a = in_a && (tie_a || (cut_a && near_a)), push_b = in_b && (tie_b || (cut_b && near_b));
+            if (push_a || push_b) {
+                const unsigned int code = (unsigned int)tid | ((unsigned int)jj << 9);
+                if (push_a) list(code, i0, j);
+                if (push_b) list(code | kVcTile, i1, j);
+            }
         }
     };
     for (int J = J0; J <= J1; ++J) {
         const int jt = J * kVcTile + tid;
         __syncthreads();   // the histograms are zeroed; the previous tile is no longer read
         if (jt < C.n) {
-            const float4 p = p4[jt];
-            sp[tid] = make_float4(-p.x, -p.y, -p.z, 0.f);
-            su[tid] = u4[jt];
+            const float4 p = p4[jt], u = u4[jt];
+            sp[tid] = make_float4(-p.x, -p.x, -p.y, -p.y);
+            sp[kVcTile + tid] = make_float4(-p.z, -p.z, u.x, u.x);
+            sp[2 * kVcTile + tid] = make_float4(u.y, u.y, u.z, u.z);
         }
         __syncthreads();
         const int jn = min(kVcTile, C.n - J * kVcTile);
@@ -337,19 +349,31 @@ __device__ __forceinline__ double round_quotient(double a, double L, double invL
     return fabs(f - 0.5) < 0x1p-46 ? round(__ddiv_rn(a, L)) : round(q);
 }
 
+// round(a / L) for |a| < L (the quotient rounds to 1/2 or more exactly when a
+// >= L / 2: the next double below L / 2 has a quotient of at most 1/2 - 2^-54):
+// two comparisons instead of a product, a truncation and a rounding
+__device__ __forceinline__ double round_near(double a, double halfL)
+{
+    return a >= halfL ? 1.0 : (a <= -halfL ? -1.0 : 0.0);
+}
+
 // The Lees-Edwards minimum image with every operation of the definition
-// (the same results as min_image()).
+// (the same results as min_image(); a product by 0 or +-1 is exact and its
+// subtraction of 0 changes nothing).
 __device__ __forceinline__ void vc_min_image(const KParams& P, const VcConst& C, double xi, double yi, double zi,
                                              double xj, double yj, double zj, double& dx, double& dy, double& dz)
 {
     dx = __dsub_rn(xi, xj);
     dy = __dsub_rn(yi, yj);
     dz = __dsub_rn(zi, zj);
-    const double n = round_quotient(dy, P.L[1], C.invL[1]);
-    dy = __dsub_rn(dy, __dmul_rn(n, P.L[1]));
-    dx = __dsub_rn(dx, __dmul_rn(n, C.delta));
-    dx = __dsub_rn(dx, __dmul_rn(P.L[0], round_quotient(dx, P.L[0], C.invL[0])));
-    dz = __dsub_rn(dz, __dmul_rn(P.L[2], round_quotient(dz, P.L[2], C.invL[2])));
+    const double n = round_near(dy, 0.5 * P.L[1]), c = round_near(dz, 0.5 * P.L[2]);
+    if (n != 0.0) {
+        dy = __dsub_rn(dy, n > 0.0 ? P.L[1] : -P.L[1]);
+        dx = __dsub_rn(dx, n > 0.0 ? C.delta : -C.delta);
+    }
+    const double a = fabs(dx) < P.L[0] ? round_near(dx, 0.5 * P.L[0]) : round_quotient(dx, P.L[0], C.invL[0]);
+    if (a != 0.0) dx = __dsub_rn(dx, __dmul_rn(P.L[0], a));
+    if (c != 0.0) dz = __dsub_rn(dz, c > 0.0 ? P.L[2] : -P.L[2]);
 }
 
 // The listed pairs with the FP64 operations of the definition (the minimum
@@ -383,7 +407,7 @@ __global__ void k_vc_band(VcConst C, KParams P, const double* __restrict__ pos, 
 
 size_t pairs_smem(int nbins)
 {
-    return sizeof(float4) * 2 * kVcTile + sizeof(unsigned int) * (kVcListed + 2 * kVcWarps * nbins);
+    return sizeof(float4) * 3 * kVcTile + sizeof(unsigned int) * (kVcListed + 2 * kVcWarps * nbins);
 }
 
 template <class T>
