@@ -40,6 +40,7 @@ struct PShared {
     double bcast[4];
     float bcastf[2];     // the same totals rounded to FP32 (the on-chip iteration's scalars)
     int flag;
+    int win[2];          // the block's windows (streaming solve)
     // decided by thread 0 (FP64 scalars once per block, not once per thread)
     float alpha_f, beta_f;
     int action;   // 0 continue, 1 replace the residual, 2 stop
@@ -498,6 +499,29 @@ __device__ __forceinline__ int chunk_lane(int k, int t)
     return (k & 1) ? (t ^ 0xE0) : t;
 }
 
+// First window of block b of nb: the first whose entries and rows before it cost
+// at least b / nb of all (8 bytes an entry, ~160 a row: in units of 8 bytes,
+// 256 x 20 a window plus its entries).  With equal numbers of windows the
+// densest block set the pace of a clustered system: a batch of 8 replicas,
+// 351,946 rows, 3.24 -> 2.60 ms (at 4.2 M rows, 108 windows a block, no change).  One warp, by a search 32 points at a time.
+__device__ __forceinline__ int window_at(const KParams& P, const DevBuffers& B, int b, int nb)
+{
+    const int nwin = P.nslots / 256, lane = threadIdx.x & 31;
+    auto cost = [&](int w) { return 5120ll * w + B.chunk_off[8 * w]; };
+    const long long T = cost(nwin) * b / nb;
+    int lo = 0, hi = nwin;   // cost(lo) <= T, the answer in [lo, hi]
+    while (hi - lo > 1) {
+        const int step = (hi - lo + 31) / 32, w = min(lo + step * (lane + 1), hi);
+        const unsigned int below = __ballot_sync(0xffffffffu, cost(w) <= T);
+        const int k = __popc(below);   // the points are non-decreasing
+        const int nlo = k > 0 ? min(lo + step * k, hi) : lo;
+        hi = min(lo + step * (k + 1), hi);
+        lo = nlo;
+        if (lo >= hi) break;
+    }
+    return cost(lo) >= T ? lo : hi;
+}
+
 // The solve of one system by blocks bid = 0..nb-1 of the launch (all of the
 // launch for a single system; a share of it in a batch).  Expects r4 = (r, D^-1)
 // with r = b - A x, p4 = q4 = d4 = 0 and the scalars, from the set-up kernel.
@@ -513,9 +537,12 @@ __device__ __forceinline__ void persistent_solve(const KParams& P, const DevBuff
     if (st->error | st->overflow | st->done) return;   // uniform: set before the launch
     unsigned int gen = 0u;   // barriers passed in this launch (the counter starts at 0)
 
-    const int nwin = P.nslots / 256;
-    const int wb = (int)((long long)bid * nwin / nb);
-    const int we = (int)((long long)(bid + 1) * nwin / nb);
+    if (threadIdx.x < 64) {
+        const int side = threadIdx.x >> 5, w = window_at(P, B, bid + side, nb);
+        if ((threadIdx.x & 31) == 0) sh.win[side] = w;
+    }
+    __syncthreads();
+    const int wb = sh.win[0], we = sh.win[1];
     const int G = blockDim.x >> 8;                              // window groups
     const int t = threadIdx.x & 255, wg = wb + (threadIdx.x >> 8);   // lane in window, first window
     const int np = P.npad;
