@@ -1741,7 +1741,21 @@ __global__ void __launch_bounds__(BS, 1) k32_cg_resident(KParams P, DevBuffers B
 // Small systems (k64_cg_pipelined, below): pipelined CG on chip.
 constexpr int kBatch64 = 6;
 
-// s_a = sum over the row's entries of w_k v_a[col_k]
+// A 32-byte record (x, y, z, 0) in FP64 in one access (one sector; the gathers'
+// L1 wavefronts, one per line touched, were three times as many with a plane
+// per component), ordered like a plain access.
+__device__ __forceinline__ void load_record64(const double* p, double& x, double& y, double& z)
+{
+    double w;
+    asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(x), "=d"(y), "=d"(z), "=d"(w) : "l"(p) : "memory");
+}
+__device__ __forceinline__ void store_record64(double* p, double x, double y, double z)
+{
+    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(x), "d"(y), "d"(z), "d"(0.0) : "memory");
+}
+
+// s_a = sum over the row's entries of w_k v_a[col_k]; v is planes, or records (REC)
+template <bool REC>
 __device__ __forceinline__ void p_row_sum64(const int* __restrict__ col, const double* __restrict__ val,
                                             const double* v, int np, int e0, int e1, bool active, double& s0,
                                             double& s1, double& s2)
@@ -1766,9 +1780,13 @@ __device__ __forceinline__ void p_row_sum64(const int* __restrict__ col, const d
             for (int u = 0; u < kBatch64; ++u) {
                 g0[u] = g1[u] = g2[u] = 0.0;
                 if (w[u] != 0.0) {
-                    g0[u] = v[j[u]];
-                    g1[u] = v[np + j[u]];
-                    g2[u] = v[2 * np + j[u]];
+                    if (REC) {
+                        load_record64(v + 4 * (size_t)j[u], g0[u], g1[u], g2[u]);
+                    } else {
+                        g0[u] = v[j[u]];
+                        g1[u] = v[np + j[u]];
+                        g2[u] = v[2 * np + j[u]];
+                    }
                 }
             }
 #pragma unroll
@@ -1781,12 +1799,10 @@ __device__ __forceinline__ void p_row_sum64(const int* __restrict__ col, const d
     }
 }
 
-// The block's rows in slot order.
+// The rows of the block's windows [wb, we) in slot order.
 template <class F>
-__device__ __forceinline__ void for_each_slot64(const KParams& P, int bid, int nb, F f)
+__device__ __forceinline__ void for_each_slot64(int wb, int we, F f)
 {
-    const int nwin = P.nslots / 256;
-    const int wb = (int)((long long)bid * nwin / nb), we = (int)((long long)(bid + 1) * nwin / nb);
     const int G = blockDim.x >> 8, t = threadIdx.x & 255;
     for (int w = wb + (int)(threadIdx.x >> 8), k = 0; w < we; w += G, ++k) f(w * 256 + chunk_lane(k, t));
 }
@@ -1802,9 +1818,15 @@ __device__ __forceinline__ void persistent_solve64(const KParams& P, const DevBu
     const int np = P.npad;
     double* x = B.x;
     double* r = B.r;
-    double* z = B.z;
+    double* z = B.s64;   // records
     double* p = B.p;
     double* q = B.q;
+    if (threadIdx.x < 64) {
+        const int side = threadIdx.x >> 5, w = window_at(P, B, bid + side, nb);
+        if ((threadIdx.x & 31) == 0) sh.win[side] = w;
+    }
+    __syncthreads();
+    const int wb = sh.win[0], we = sh.win[1];
     auto row_of = [&](int slot) { return B.slot_row[slot]; };
     auto ends = [&](int slot, int& e0, int& e1) {
         e0 = B.chunk_off[slot >> 5] + (slot & 31);
@@ -1814,16 +1836,16 @@ __device__ __forceinline__ void persistent_solve64(const KParams& P, const DevBu
     // r = b - A x0 (or b, x = 0); z = D^-1 r; p = q = 0; ||b||^2, r.r, r.z
     {
         double bb = 0.0, rr = 0.0, rz = 0.0;
-        for_each_slot64(P, bid, nb, [&](int slot) {
+        for_each_slot64(wb, we, [&](int slot) {
             const int row = row_of(slot);
             int e0 = 0, e1 = 0;
             if (row >= 0) ends(slot, e0, e1);
             double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-            if (from_x) p_row_sum64(B.col, B.val, x, np, e0, e1, row >= 0, s0, s1, s2);
+            if (from_x) p_row_sum64<false>(B.col, B.val, x, np, e0, e1, row >= 0, s0, s1, s2);
             if (row < 0) return;
             const double sv[3] = {s0, s1, s2};
             const double d = B.diag[row], di = B.dinv[row];
-            double rs = 0.0;
+            double rs = 0.0, zn[3];
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 const int k2 = c * np + row;
@@ -1834,12 +1856,13 @@ __device__ __forceinline__ void persistent_solve64(const KParams& P, const DevBu
                 else
                     x[k2] = 0.0;
                 r[k2] = rk;
-                z[k2] = di * rk;
+                zn[c] = di * rk;
                 p[k2] = 0.0;
                 q[k2] = 0.0;
                 bb += bk * bk;
                 rs += rk * rk;
             }
+            store_record64(z + 4 * (size_t)row, zn[0], zn[1], zn[2]);
             rr += rs;
             rz += di * rs;
         });
@@ -1874,19 +1897,21 @@ __device__ __forceinline__ void persistent_solve64(const KParams& P, const DevBu
         // ---- q = A z + beta q; p = z + beta p; p.q
         const double beta = sh.bcast[3];
         double pq = 0.0;
-        for_each_slot64(P, bid, nb, [&](int slot) {
+        for_each_slot64(wb, we, [&](int slot) {
             const int row = row_of(slot);
             int e0 = 0, e1 = 0;
             if (row >= 0) ends(slot, e0, e1);
             double s0, s1, s2;
-            p_row_sum64(B.col, B.val, z, np, e0, e1, row >= 0, s0, s1, s2);
+            p_row_sum64<true>(B.col, B.val, z, np, e0, e1, row >= 0, s0, s1, s2);
             if (row < 0) return;
             const double sv[3] = {s0, s1, s2};
             const double d = B.diag[row];
+            double zo[3];
+            load_record64(z + 4 * (size_t)row, zo[0], zo[1], zo[2]);
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 const int k2 = c * np + row;
-                const double zk = z[k2];
+                const double zk = zo[c];
                 const double az = d * zk - P.alpha * sv[c];
                 const double qk = beta == 0.0 ? az : az + beta * q[k2];
                 const double pk = beta == 0.0 ? zk : zk + beta * p[k2];
@@ -1914,20 +1939,21 @@ __device__ __forceinline__ void persistent_solve64(const KParams& P, const DevBu
         // ---- x += alpha p; r -= alpha q; z = D^-1 r (own rows); r.r, r.z
         const double a = sh.bcast[2];
         double rr = 0.0, rz = 0.0;
-        for_each_slot64(P, bid, nb, [&](int slot) {
+        for_each_slot64(wb, we, [&](int slot) {
             const int i = row_of(slot);
             if (i < 0) return;
             const double di = B.dinv[i];
-            double rs = 0.0;
+            double rs = 0.0, zn[3];
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 const int k2 = c * np + i;
                 x[k2] += a * p[k2];
                 const double rk = r[k2] - a * q[k2];
                 r[k2] = rk;
-                z[k2] = di * rk;
+                zn[c] = di * rk;
                 rs += rk * rk;
             }
+            store_record64(z + 4 * (size_t)i, zn[0], zn[1], zn[2]);
             rr += rs;
             rz += di * rs;
         });
@@ -1954,24 +1980,25 @@ __device__ __forceinline__ void persistent_solve64(const KParams& P, const DevBu
         // ---- the FP64 true residual r = b - A x (z = D^-1 r): accept, restart or give up
         {
             double trr = 0.0, trz = 0.0;
-            for_each_slot64(P, bid, nb, [&](int slot) {
+            for_each_slot64(wb, we, [&](int slot) {
                 const int row = row_of(slot);
                 int e0 = 0, e1 = 0;
                 if (row >= 0) ends(slot, e0, e1);
                 double s0, s1, s2;
-                p_row_sum64(B.col, B.val, x, np, e0, e1, row >= 0, s0, s1, s2);
+                p_row_sum64<false>(B.col, B.val, x, np, e0, e1, row >= 0, s0, s1, s2);
                 if (row < 0) return;
                 const double sv[3] = {s0, s1, s2};
                 const double d = B.diag[row], di = B.dinv[row];
-                double rs = 0.0;
+                double rs = 0.0, zn[3];
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
                     const int k2 = c * np + row;
                     const double rk = B.b[k2] - (d * x[k2] - P.alpha * sv[c]);
                     r[k2] = rk;
-                    z[k2] = di * rk;
+                    zn[c] = di * rk;
                     rs += rk * rk;
                 }
+                store_record64(z + 4 * (size_t)row, zn[0], zn[1], zn[2]);
                 trr += rs;
                 trz += di * rs;
             });

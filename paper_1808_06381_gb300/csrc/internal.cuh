@@ -160,8 +160,8 @@ struct DevBuffers {
     double* p;       // [3][npad]
     double* q;       // [3][npad]
     double* z;       // [3][npad] D^-1 r (FP64 solver)
-    double* s64;     // [2][npad][4] FP64 on-chip solve of small systems: the two buffers of its published
-                     // records (x, y, z, 0 of a row)
+    double* s64;     // [2][npad][4] FP64 persistent solves: records (x, y, z, 0 of a row) of the gathered vector
+                     // (the on-chip form publishes into the two buffers in turn)
     uint4* posfix;   // [npad] mixed: positions in 32-bit fixed point of the box edges (x, y, z, 0), built
                      // before each matrix-free solve
     float4* r4;      // [npad] mixed solver vectors, (x, y, z, 0) per row
