@@ -119,24 +119,28 @@ __global__ void __launch_bounds__(256) k_cheb_step(KParams P, DevBuffers B, cons
     }
 }
 
+constexpr int kChebThreads = 128;
 // The same degree step for the mixed path in double-float on the FP32 pipes:
 // T_k and xi as 32-byte records per row (hi float4, lo float4), the weights
 // and A_ii as their double-float pairs.  Bound by the L1 wavefronts of the
 // gathered records, so a record is one 32-byte access (n = 262,144 clustered,
 // 18 entries a row: 57 us a step with two 16-byte accesses, 51.5 with one).
-__global__ void __launch_bounds__(256) k_cheb_step_df(KParams P, DevBuffers B, const float4* __restrict__ tc,
-                                                      const float4* __restrict__ tp, float4* __restrict__ tn,
-                                                      float4* __restrict__ y, const float2* __restrict__ csf, int kdeg)
+// Blocks of 128 with six on an SM leave 85 registers a thread, enough for six
+// entries in flight without a spill: 39 us (256 threads and four entries: 51;
+// two entries 59; eight entries at half the warps 50).
+__global__ void __launch_bounds__(kChebThreads, 768 / kChebThreads)
+k_cheb_step_df(KParams P, DevBuffers B, const float4* __restrict__ tc, const float4* __restrict__ tp,
+               float4* __restrict__ tn, float4* __restrict__ y, const float2* __restrict__ csf, int kdeg)
 {
     const int first = kdeg == 1;
     const float2 s1 = csf[0], s0 = csf[1], ck = csf[2 + kdeg], c0 = csf[2];
     const float2 c0h = make_float2(0.5f * c0.x, 0.5f * c0.y);   // exact halving
-    const int slot = blockIdx.x * 256 + threadIdx.x;
+    const int slot = blockIdx.x * kChebThreads + threadIdx.x;
     if (slot >= P.nslots) return;
     const int row = B.slot_row[slot];
     if (row < 0) return;
     dfloat s[3];
-    row_sum_df<4>(B.col, B.val32, B.val32lo, tc, B.chunk_off[slot >> 5] + (slot & 31), B.chunk_off[(slot >> 5) + 1],
+    row_sum_df<6>(B.col, B.val32, B.val32lo, tc, B.chunk_off[slot >> 5] + (slot & 31), B.chunk_off[(slot >> 5) + 1],
                   s);
     const dfloat d{B.diag32[row], B.diag32lo[row]}, al{P.alpha_hi, P.alpha_lo};
     const dfloat S1{s1.x, s1.y}, S0{s0.x, s0.y}, CK{ck.x, ck.y}, C0{c0h.x, c0h.y};
@@ -312,7 +316,7 @@ int enqueue_fdt_noise(const KParams& P, DevBuffers& B, FdtBuffers& V, int degree
 cudaError_t cheb_step_df(const KParams& P, DevBuffers& B, const float4* tc, const float4* tp, float4* tn, float4* y,
                          const float2* csf, int k, cudaStream_t s)
 {
-    k_cheb_step_df<<<P.nslots / 256, 256, 0, s>>>(P, B, tc, tp, tn, y, csf, k);
+    k_cheb_step_df<<<P.nslots / kChebThreads, kChebThreads, 0, s>>>(P, B, tc, tp, tn, y, csf, k);
     return cudaGetLastError();
 }
 
