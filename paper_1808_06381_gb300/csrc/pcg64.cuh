@@ -147,6 +147,7 @@ __device__ __forceinline__ void stage(const Sys& S, Shared& sh, unsigned char* d
         const int pad = max(__shfl_sync(0xffffffffu, row, 0), 0);
         bool bad = !at.valid();
         for (int kb = 0; kb < len; kb += KS) {
+            if (__any_sync(0xffffffffu, bad)) break;   // refused: no read beyond a malformed row's first bad column
             int j[KS];
             V w[KS];
 #pragma unroll
