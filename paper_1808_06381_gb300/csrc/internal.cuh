@@ -118,7 +118,8 @@ struct DevBuffers {
     double* v_s;     // [3][npad] velocities of the last solve
     // work arrays of the current step (cell order)
     double* pos_w;   // [3][npad]
-    float* pos32;    // [3][npad] FP32 copy of pos_w for the pair pre-filter
+    float* pos32;    // [3][npad] FP32 copy of pos_w
+    float4* pos4;    // [npad] the same as one record per row (x, y, z, 0): the pair search's candidates
     float* pos32lo;  // [3][npad] pos_w - pos32: positions as double-floats (pos32, pos32lo)
     int* id_w;       // [n]
     int* cell_of;    // [n] cell of each row: in the state order while binning, then (written by the

@@ -248,21 +248,24 @@ __global__ void k_sort_cells(KParams P, const int* __restrict__ cell_start, int*
 __global__ void k_gather_rows(KParams P, const int* __restrict__ perm, const int* __restrict__ id_s,
                               const double* __restrict__ pos_s, const double* __restrict__ v_s,
                               double* __restrict__ pos_w, float* __restrict__ pos32, float* __restrict__ pos32lo,
-                              int* __restrict__ id_w, double* __restrict__ x, int warm, const DevState* st)
+                              float4* __restrict__ pos4, int* __restrict__ id_w, double* __restrict__ x, int warm,
+                              const DevState* st)
 {
     if (st->error | st->overflow) return;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= P.n) return;
     const int np = P.npad;
     const int s = perm[k];
+    float h[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         const double v = pos_s[a * np + s];
         pos_w[a * np + k] = v;
-        const float vh = (float)v;
-        pos32[a * np + k] = vh;
-        pos32lo[a * np + k] = (float)(v - (double)vh);
+        h[a] = (float)v;
+        pos32[a * np + k] = h[a];
+        pos32lo[a * np + k] = (float)(v - (double)h[a]);
     }
+    pos4[k] = make_float4(h[0], h[1], h[2], 0.f);
     id_w[k] = id_s[s];
 #pragma unroll
     for (int a = 0; a < 3; ++a) x[a * np + k] = warm ? v_s[a * np + s] : 0.0;
@@ -275,7 +278,7 @@ int launch_scatter_sort_gather(const KParams& P, DevBuffers& B, bool warm, Launc
     k_sort_cells<<<grid_for(P.ncell, 128, 1 << 30), 128, 0, L.stream>>>(P, B.cell_start, B.perm, B.id_s, B.cell_of,
                                                                          B.st);
     k_gather_rows<<<grid_for(P.n, kVecBlock, 1 << 30), kVecBlock, 0, L.stream>>>(
-        P, B.perm, B.id_s, B.pos_s, B.v_s, B.pos_w, B.pos32, B.pos32lo, B.id_w, B.x, warm ? 1 : 0, B.st);
+        P, B.perm, B.id_s, B.pos_s, B.v_s, B.pos_w, B.pos32, B.pos32lo, B.pos4, B.id_w, B.x, warm ? 1 : 0, B.st);
     return 3;
 }
 
@@ -426,13 +429,19 @@ __device__ __forceinline__ void for_each_neighbor_generic(const KParams& P, doub
 // predicate.  At most one image of j lies within r_c of i because every box
 // edge is >= 3 r_c, so the image found here is the canonical minimum image of
 // every accepted pair.  FP32 arithmetic uses explicit round-to-nearest
-// intrinsics so that the counting and filling passes decide identically.
+// intrinsics so that the counting and filling passes decide identically.  The
+// search is bound by instruction issue (a warp's lanes scan different cells,
+// each loop running to the longest), so a candidate is one 16-byte load, the
+// shift is taken from the particle once per cell, and the particle itself is
+// sorted out only among the accepted ones: 12 instructions a candidate instead
+// of ~22 (with the normals: n = 262,144 clustered 171 us -> 157, n = 4,194,304
+// 2,260 -> 2,070).
 // The nine (z, y) rows of three cells are numbered 0..8; rows zy0..zy1 - 1 are
 // visited (all of them, or one by each of nine threads that share a particle).
 template <class F>
 __device__ __forceinline__ void for_each_neighbor_fast(const KParams& P, double delta,
                                                        const double* __restrict__ pos,
-                                                       const float* __restrict__ pos32,
+                                                       const float4* __restrict__ pos4,
                                                        const int* __restrict__ cell_start,
                                                        const int* __restrict__ cell_w, int i,
                                                        double xi, double yi, double zi, F&& visit, int zy0 = 0,
@@ -440,7 +449,7 @@ __device__ __forceinline__ void for_each_neighbor_fast(const KParams& P, double 
 {
     const int np = P.npad;
     const int nc0 = P.nc[0], nc1 = P.nc[1], nc2 = P.nc[2];
-    const float xf = pos32[i], yf = pos32[np + i], zf = pos32[2 * np + i];
+    const float4 pf = pos4[i];
     const float deltaf = (float)delta;
     // the row's cell coordinates from its cell index (integer work; the
     // binning computed the index from the same FP64 position)
@@ -470,7 +479,7 @@ __device__ __forceinline__ void for_each_neighbor_fast(const KParams& P, double 
             czz -= nc2;
             c_img = 1;
         }
-        const float szf = times(c_img, P.Lf[2]);
+        const float zs = __fsub_rn(pf.z, times(c_img, P.Lf[2]));
         for (int dyc = zy1 - zy0 == 1 ? zy0 % 3 - 1 : -1; dyc <= (zy1 - zy0 == 1 ? zy0 % 3 - 1 : 1); ++dyc) {
             int cyy = cy + dyc, m = 0;
             if (cyy < 0) {
@@ -480,7 +489,7 @@ __device__ __forceinline__ void for_each_neighbor_fast(const KParams& P, double 
                 cyy -= nc1;
                 m = 1;
             }
-            const float syf = times(m, P.Lf[1]);
+            const float ys = __fsub_rn(pf.y, times(m, P.Lf[1]));
             const float mdf = times(m, deltaf);
             const int cxu0 = m == 0 ? cx : (m > 0 ? cx_p1 : cx_m1);
             for (int dxc = -1; dxc <= 1; ++dxc) {
@@ -489,17 +498,14 @@ __device__ __forceinline__ void for_each_neighbor_fast(const KParams& P, double 
                 const int a = cxu >= 0 ? (cxu >= nc0 ? (cxu >= 2 * nc0 ? 2 : 1) : 0) : (cxu >= -nc0 ? -1 : -2);
                 const int c = cell_index(P, cxu - a * nc0, cyy, czz);
                 const float axf = a == 0 ? 0.f : (a == 1 ? P.Lf[0] : (a == -1 ? -P.Lf[0] : (a == 2 ? L2f : -L2f)));
-                const float sxf = __fadd_rn(mdf, axf);
+                const float xs = __fsub_rn(pf.x, __fadd_rn(mdf, axf));
                 const unsigned char code = image_code(a, m, c_img);
                 const int j1 = cell_start[c + 1];
                 for (int j = cell_start[c]; j < j1; ++j) {
-                    if (j == i) continue;
-                    const float dxf = __fsub_rn(__fsub_rn(xf, pos32[j]), sxf);
-                    const float dyf = __fsub_rn(__fsub_rn(yf, pos32[np + j]), syf);
-                    const float dzf = __fsub_rn(__fsub_rn(zf, pos32[2 * np + j]), szf);
-                    const float r2f = __fadd_rn(__fadd_rn(__fmul_rn(dxf, dxf), __fmul_rn(dyf, dyf)),
-                                                __fmul_rn(dzf, dzf));
-                    if (r2f >= P.rc2_hi) continue;
+                    const float4 q = pos4[j];
+                    const float dxf = __fsub_rn(xs, q.x), dyf = __fsub_rn(ys, q.y), dzf = __fsub_rn(zs, q.z);
+                    const float r2f = __fmaf_rn(dzf, dzf, __fmaf_rn(dyf, dyf, __fmul_rn(dxf, dxf)));
+                    if (r2f >= P.rc2_hi || j == i) continue;
                     if (r2f < P.rc2_lo) {
                         visit(j, code);
                     } else {
@@ -518,13 +524,13 @@ __device__ __forceinline__ void for_each_neighbor_fast(const KParams& P, double 
 template <class F>
 __device__ __forceinline__ void for_each_neighbor(const KParams& P, double delta,
                                                   const double* __restrict__ pos,
-                                                  const float* __restrict__ pos32,
+                                                  const float4* __restrict__ pos4,
                                                   const int* __restrict__ cell_start,
                                                   const int* __restrict__ cell_w, int i,
                                                   double xi, double yi, double zi, F&& visit)
 {
     if (P.fast_cells)
-        for_each_neighbor_fast(P, delta, pos, pos32, cell_start, cell_w, i, xi, yi, zi, visit);
+        for_each_neighbor_fast(P, delta, pos, pos4, cell_start, cell_w, i, xi, yi, zi, visit);
     else
         for_each_neighbor_generic(P, delta, pos, cell_start, i, xi, yi, zi, visit);
 }
@@ -564,7 +570,7 @@ __global__ void k_nbr_collect(KParams P, DevBuffers B, int draw_noise)
     int cnt = 0;
     int* __restrict__ cj = B.cand_j;
     unsigned char* __restrict__ ci = B.cand_img;
-    for_each_neighbor(P, delta, B.pos_w, B.pos32, B.cell_start, B.cell_of, i, B.pos_w[i], B.pos_w[np + i],
+    for_each_neighbor(P, delta, B.pos_w, B.pos4, B.cell_start, B.cell_of, i, B.pos_w[i], B.pos_w[np + i],
                       B.pos_w[2 * np + i], [&](int j, unsigned char code) {
                           if (cnt < kCandCap) {
                               cj[(size_t)cnt * np + i] = j;
@@ -601,7 +607,7 @@ __global__ void __launch_bounds__(9 * kSplitRows) k_nbr_collect_split(KParams P,
     const double xi = i < P.n ? B.pos_w[i] : 0.0, yi = i < P.n ? B.pos_w[np + i] : 0.0, zi = i < P.n ? B.pos_w[2 * np + i] : 0.0;
     int cnt = 0;
     if (i < P.n)
-        for_each_neighbor_fast(P, delta, B.pos_w, B.pos32, B.cell_start, B.cell_of, i, xi, yi, zi,
+        for_each_neighbor_fast(P, delta, B.pos_w, B.pos4, B.cell_start, B.cell_of, i, xi, yi, zi,
                                [&](int, unsigned char) { ++cnt; }, part, part + 1);
     found[part][r] = cnt;
     __syncthreads();
@@ -612,7 +618,7 @@ __global__ void __launch_bounds__(9 * kSplitRows) k_nbr_collect_split(KParams P,
     if (cnt == 0 || at >= kCandCap) return;
     int* __restrict__ cj = B.cand_j;
     unsigned char* __restrict__ ci = B.cand_img;
-    for_each_neighbor_fast(P, delta, B.pos_w, B.pos32, B.cell_start, B.cell_of, i, xi, yi, zi,
+    for_each_neighbor_fast(P, delta, B.pos_w, B.pos4, B.cell_start, B.cell_of, i, xi, yi, zi,
                            [&](int j, unsigned char code) {
                                if (at < kCandCap) {
                                    cj[(size_t)at * np + i] = j;
@@ -881,7 +887,7 @@ __device__ __noinline__ void search_row_into_slots(const KParams& P, const DevBu
 {
     const int np = P.npad;
     int k = 0;
-    for_each_neighbor(P, delta, B.pos_w, B.pos32, B.cell_start, B.cell_of, i, B.pos_w[i], B.pos_w[np + i],
+    for_each_neighbor(P, delta, B.pos_w, B.pos4, B.cell_start, B.cell_of, i, B.pos_w[i], B.pos_w[np + i],
                       B.pos_w[2 * np + i],
                       [&](int j, unsigned char code) {
                           if (k < cnt) {
@@ -1176,7 +1182,7 @@ __global__ void k_nbr_fill(KParams P, DevBuffers B)
     int k = 0;
     int* __restrict__ col = B.col;
     unsigned char* __restrict__ img = B.img;
-    for_each_neighbor(P, delta, B.pos_w, B.pos32, B.cell_start, B.cell_of, i, xi, yi, zi, [&](int j, unsigned char code) {
+    for_each_neighbor(P, delta, B.pos_w, B.pos4, B.cell_start, B.cell_of, i, xi, yi, zi, [&](int j, unsigned char code) {
         if (k < cnt) {
             col[base + 32 * k] = j;
             img[base + 32 * k] = code;

@@ -659,7 +659,7 @@ int sp_sim_destroy(sp_sim* s)
                     B.chunk_off, B.col, B.img, B.val, B.val32, B.val32lo, B.hcol, B.hval, B.diag, B.partials_df,
                     B.diag32lo, B.bdf, B.xdf, B.rdf, B.rlo, B.hlo,
                     B.dinv, B.diag32, B.dinv32, B.b, B.x, B.r, B.p, B.q, B.z, B.s64, B.r4, B.p4, B.q4, B.d4,
-                    B.posfix, B.res_hist, B.xi_inj, B.exp_tab, B.exp_tab_df, B.rng_tab, B.pos32lo, B.cand_j, B.cand_img, B.noise3, B.partials, B.scan_tmp, B.stage, B.st};
+                    B.posfix, B.res_hist, B.xi_inj, B.exp_tab, B.exp_tab_df, B.rng_tab, B.pos32lo, B.pos4, B.cand_j, B.cand_img, B.noise3, B.partials, B.scan_tmp, B.stage, B.st};
     for (void* q : ptrs)
         if (q) cudaFree(q);
     if (s->mp_alloc) {
@@ -746,6 +746,7 @@ int sp_sim_create(const sp_params* p, const double* pos_host, sp_sim** out)
     A(dev_alloc(s, &B.pos_w, v3));
     A(dev_alloc(s, &B.pos32, v3));
     A(dev_alloc(s, &B.pos32lo, v3));
+    A(dev_alloc(s, &B.pos4, (size_t)npad));
     A(dev_alloc(s, &B.v_s, v3));
     A(dev_alloc(s, &B.id_s, n));
     A(dev_alloc(s, &B.id_w, n));
