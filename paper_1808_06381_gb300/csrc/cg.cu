@@ -405,8 +405,10 @@ __global__ void __launch_bounds__(kBlock) k32_split_x(KParams P, DevBuffers B)
 // r = b - A x0 in double-float from the double-float matrix, b and x0 (or
 // r = b and x = 0); r4 = (fp32(r), D^-1); d = p = q = 0.  ||b||^2 from the
 // high parts of b (FP32 squares summed in FP64: the relative tolerance needs
-// a few digits of it).
-__global__ void __launch_bounds__(kBlock) k32_init(KParams P, DevBuffers B, int from_x)
+// a few digits of it).  Bound by the L1 wavefronts of the gathered 32-byte
+// records: three blocks on an SM leave 85 registers a thread for six entries in
+// flight (n = 4,194,304: 915 us, with eight in flight and no bound 957).
+__global__ void __launch_bounds__(kBlock, 3) k32_init(KParams P, DevBuffers B, int from_x)
 {
     DevState* st = B.st;
     if (st->error | st->overflow) return;
@@ -417,7 +419,7 @@ __global__ void __launch_bounds__(kBlock) k32_init(KParams P, DevBuffers B, int 
         dfloat r[3];
         if (from_x) {
             dfloat s[3];
-            row_sum_df<8>(B.col, B.val32, B.val32lo, B.xdf, e0, e1, s);
+            row_sum_df<6>(B.col, B.val32, B.val32lo, B.xdf, e0, e1, s);
             residual_df(P, B, row, s, r);
         } else {
             const float4 bh = B.bdf[2 * row], bl = B.bdf[2 * row + 1];
