@@ -453,7 +453,10 @@ def main():
     if prof["persistent_ms"] > 0 and args.precision == "fp64":
         plan = plan_algorithmic_bytes(prof["n"], prof["cg_iterations"], "fp64")
         pach = plan / (prof["persistent_ms"] * 1e-3) / 1e9
-        persistent = {"kernel": "k64_cg_persistent", "bound": "latency", "achieved": pach, "peak": peak,
+        # the on-chip form takes up to 16 chunks of 32 rows per SM
+        onchip = prof["n"] <= 512 * torch.cuda.get_device_properties(local_rank).multi_processor_count
+        persistent = {"kernel": "k64_cg_pipelined" if onchip else "k64_cg_persistent", "bound": "latency",
+                      "achieved": pach, "peak": peak,
                       "unit": "GB/s", "frac": pach / peak, "traffic": None,
                       "peak_source": f"hbm_gbs {peak_kind} (burst copy)",
                       "algorithmic_bytes_per_launch": plan,
@@ -461,10 +464,11 @@ def main():
                                                 "iteration x n x iterations",
                       "avg_launch_ms": prof["persistent_ms"], "cg_iterations": prof["cg_iterations"],
                       "true_residual_checks": prof["true_checks"], "grid": prof["persistent_blocks"],
-                      "note": "one cooperative launch per solve; the system stays in L2 and GB300 issues FP64 at "
+                      "note": "one cooperative launch per solve; the system stays on the chip (shared memory and "
+                              "registers, or L2 for systems of more than 512 rows per SM) and GB300 issues FP64 at "
                               "~2 FMA per clock per SM: bound by the FP64 pipe, the gathers' latency and the grid "
-                              "reductions (two per iteration; one in the pipelined form that systems of fewer "
-                              "than 512 rows per SM take), so frac is an algorithmic-equivalent bandwidth"}
+                              "reductions (one per iteration on chip, two beyond), so frac is an "
+                              "algorithmic-equivalent bandwidth"}
     elif prof["persistent_ms"] > 0:
         pbytes = persistent_algorithmic_bytes(prof["n"], prof["nnz"], prof["cg_iterations"], prof["true_checks"],
                                               bool(prof.get("persistent_init")))

@@ -417,6 +417,9 @@ __device__ __forceinline__ void for_each_neighbor_generic(const KParams& P, doub
     }
 }
 
+constexpr int kSearchBatch = 3;   // candidates requested at a time (1: n = 60,013 85 us, 2: 77, 3: 74, 4: 70; n = 4,194,304
+                                  // 2,083, 2,065, 1,965, 2,015; 6: 71 and 2,123)
+
 // The same pair set as for_each_neighbor_generic for boxes with >= 3 cells per
 // axis, with almost no FP64 work.  Each candidate cell is visited as one image
 // of the box (integer shifts a, m, c along x, y, z), so the image separation
@@ -434,8 +437,10 @@ __device__ __forceinline__ void for_each_neighbor_generic(const KParams& P, doub
 // each loop running to the longest), so a candidate is one 16-byte load, the
 // shift is taken from the particle once per cell, and the particle itself is
 // sorted out only among the accepted ones: 12 instructions a candidate instead
-// of ~22 (with the normals: n = 262,144 clustered 171 us -> 157, n = 4,194,304
-// 2,260 -> 2,070).
+// of ~22 (with the normals: n = 262,144 clustered 171 us -> 160, n = 4,194,304
+// 2,260 -> 2,020).  What remains is the latency of the cell bounds and of the
+// candidates (4.2 warps waiting on a load per issue), so the three cells of a
+// row of cells are one run: 160 -> 156 us, 2,020 -> 1,960, n = 60,013 83 -> 74.
 // The nine (z, y) rows of three cells are numbered 0..8; rows zy0..zy1 - 1 are
 // visited (all of them, or one by each of nine threads that share a particle).
 template <class F>
@@ -492,29 +497,50 @@ __device__ __forceinline__ void for_each_neighbor_fast(const KParams& P, double 
             const float ys = __fsub_rn(pf.y, times(m, P.Lf[1]));
             const float mdf = times(m, deltaf);
             const int cxu0 = m == 0 ? cx : (m > 0 ? cx_p1 : cx_m1);
-            for (int dxc = -1; dxc <= 1; ++dxc) {
-                const int cxu = cxu0 + dxc;
+            // the three cells of the row as one run of candidates: all bounds are
+            // requested together, the lanes of a warp differ in the sum of three
+            // cells' particles (not in each), and kSearchBatch candidates are in flight
+            int base[3], part[3];     // a candidate's position is base + k, k counting through the row
+            float xs[3];
+            unsigned char code[3];
+#pragma unroll
+            for (int u = 0; u < 3; ++u) {
+                const int cxu = cxu0 + u - 1;
                 // floor(cxu / nc0) for cxu in [-2 nc0, 3 nc0)
                 const int a = cxu >= 0 ? (cxu >= nc0 ? (cxu >= 2 * nc0 ? 2 : 1) : 0) : (cxu >= -nc0 ? -1 : -2);
                 const int c = cell_index(P, cxu - a * nc0, cyy, czz);
                 const float axf = a == 0 ? 0.f : (a == 1 ? P.Lf[0] : (a == -1 ? -P.Lf[0] : (a == 2 ? L2f : -L2f)));
-                const float xs = __fsub_rn(pf.x, __fadd_rn(mdf, axf));
-                const unsigned char code = image_code(a, m, c_img);
-                const int j1 = cell_start[c + 1];
-                for (int j = cell_start[c]; j < j1; ++j) {
-                    const float4 q = pos4[j];
-                    const float dxf = __fsub_rn(xs, q.x), dyf = __fsub_rn(ys, q.y), dzf = __fsub_rn(zs, q.z);
+                xs[u] = __fsub_rn(pf.x, __fadd_rn(mdf, axf));
+                code[u] = image_code(a, m, c_img);
+                base[u] = cell_start[c];
+                part[u] = cell_start[c + 1] - base[u];
+            }
+            part[1] += part[0];
+            part[2] += part[1];
+            base[1] -= part[0];
+            base[2] -= part[1];
+            for (int k0 = 0; k0 < part[2]; k0 += kSearchBatch) {
+                float4 q[kSearchBatch];
+#pragma unroll
+                for (int u = 0; u < kSearchBatch; ++u) {
+                    const int k = min(k0 + u, part[2] - 1);
+                    q[u] = pos4[k + (k < part[0] ? base[0] : (k < part[1] ? base[1] : base[2]))];
+                }
+#pragma unroll
+                for (int u = 0; u < kSearchBatch; ++u) {
+                    const int k = k0 + u;
+                    const float dxf = __fsub_rn(k < part[0] ? xs[0] : (k < part[1] ? xs[1] : xs[2]), q[u].x);
+                    const float dyf = __fsub_rn(ys, q[u].y), dzf = __fsub_rn(zs, q[u].z);
                     const float r2f = __fmaf_rn(dzf, dzf, __fmaf_rn(dyf, dyf, __fmul_rn(dxf, dxf)));
-                    if (r2f >= P.rc2_hi || j == i) continue;
-                    if (r2f < P.rc2_lo) {
-                        visit(j, code);
-                    } else {
-                        // the margin band: the exact FP64 predicate at the image the walk
-                        // found, which is the canonical one of min_image_code for any |R|
-                        // below L / 2 (bit-identical, without its three FP64 divisions:
-                        // GB300 issues FP64 at 1/64 of the FP32 rate, and the warp waits)
-                        if (band_pair(P, delta, xi, yi, zi, pos, np, j, code)) visit(j, code);
-                    }
+                    if (r2f >= P.rc2_hi || k >= part[2]) continue;
+                    const int j = k + (k < part[0] ? base[0] : (k < part[1] ? base[1] : base[2]));
+                    const unsigned char img = k < part[0] ? code[0] : (k < part[1] ? code[1] : code[2]);
+                    if (j == i) continue;
+                    // inside the margin band the exact FP64 predicate at the image the walk
+                    // found, which is the canonical one of min_image_code for any |R|
+                    // below L / 2 (bit-identical, without its three FP64 divisions:
+                    // GB300 issues FP64 at 1/64 of the FP32 rate, and the warp waits)
+                    if (r2f < P.rc2_lo || band_pair(P, delta, xi, yi, zi, pos, np, j, img)) visit(j, img);
                 }
             }
         }
