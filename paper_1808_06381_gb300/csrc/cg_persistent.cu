@@ -503,7 +503,8 @@ __device__ __forceinline__ int chunk_lane(int k, int t)
 // at least b / nb of all (8 bytes an entry, ~160 a row: in units of 8 bytes,
 // 256 x 20 a window plus its entries).  With equal numbers of windows the
 // densest block set the pace of a clustered system: a batch of 8 replicas,
-// 351,946 rows, 3.24 -> 2.60 ms (at 4.2 M rows, 108 windows a block, no change).  One warp, by a search 32 points at a time.
+// 351,946 rows, 3.24 -> 2.60 ms (at 4.2 M rows, 108 windows a block, no change).
+// One warp, by a search 32 points at a time.
 __device__ __forceinline__ int window_at(const KParams& P, const DevBuffers& B, int b, int nb)
 {
     const int nwin = P.nslots / 256, lane = threadIdx.x & 31;
