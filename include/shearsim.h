@@ -322,7 +322,10 @@ int sp_profile_step(sp_sim* sim, sp_kernel_profile* out);
  * whole solve: their solver vectors in registers, their z = D^-1 r and the
  * matrix entries between two of them in shared memory, so that only entries
  * to other blocks' rows are gathered from global memory; it serves systems of
- * at most 2048 rows per SM and is not timed (ms 0) for larger ones.
+ * at most 2048 rows per SM and is not timed (ms 0) for larger ones; up to 768
+ * rows per SM it runs as pipelined CG with one grid reduction per iteration.
+ * A simulation for which no configuration was chosen takes the on-chip form
+ * where it serves the system and configuration 0 beyond.
  * Two configurations (matrix_free = 1) stream only the columns in the
  * iteration and recompute each pair weight w_ij = exp(-|R_ij|^2 / 2 lambda^2)
  * (arXiv 1808.06381, §Method) in FP32 from the positions in 32-bit fixed
@@ -336,7 +339,8 @@ int sp_profile_step(sp_sim* sim, sp_kernel_profile* out);
  * variable SHEARSIM_TUNE_CACHE naming a file, choices are looked up there
  * first, keyed by device name, SM count, n and the mean row length, and new
  * choices are appended (one line per key).  For SP_PREC_FP64, or with
- * trials < 1, nothing is timed and configuration 0 is kept.  Errors:
+ * trials < 1, nothing is timed and the present choice is kept (reported as
+ * configuration 0 where none was made).  Errors:
  * SP_ERR_INVALID_ARG (NULL sim), SP_ERR_CUDA, and those of the solve. */
 #define SP_TUNE_MAX_CONFIGS 12
 typedef struct sp_tune_info {
