@@ -214,9 +214,8 @@ struct MpBuffers {
     float4* a0;      // [3n] M x0
     float4* y;       // [3n] MLP output (4 message features)
     float4* a1;      // [3n] M y
-    float4* dout;    // [n] training: dLoss / dout of the node's three rows
-    float4* scaled;  // [n] D^-1 dout
-    float4* pull;    // [n] M^T dout
+    float4* dout;    // [n] training: dLoss / dout of the node's three rows, and D^-1
+    float4* dy;      // [3n] training: dLoss / dy
     float* master;   // [kMpParams] FP32 weights
     float* m;        // [kMpParams] Adam first moment
     float* v;        // [kMpParams] Adam second moment

@@ -307,10 +307,9 @@ __global__ void __launch_bounds__(128) k_mp_mlp_fwd_tc(int rows, MpBuffers M, De
 
 // ------------------------------------------ training backward on tcgen05
 //
-// One tile of 128 rows at a time, one thread per row, 128 threads, two blocks
-// per SM (one block's epilogues run under the other's products); every
-// product is a tcgen05.mma with M = 128 (BF16 operands in no-swizzle
-// core-matrix tiles as above, FP32 accumulators in tensor memory):
+// Tiles of 128 rows, one thread per row; every product is a tcgen05.mma with M =
+// 128 (BF16 operands in no-swizzle core-matrix tiles as above, FP32 accumulators
+// in tensor memory):
 //   h1 = tanh(X W1), h2 = tanh(h1 W2)             (forward recomputed; K 16, 64)
 //   dp2 = (dY W3^T) (1 - h2^2)                     (A = dY [128][16], B = W3 [64][16])
 //   dp1 = (dp2 W2^T) (1 - h1^2)                    (A = dp2 [128][64], B = W2 [64][64])
@@ -321,34 +320,44 @@ __global__ void __launch_bounds__(128) k_mp_mlp_fwd_tc(int rows, MpBuffers M, De
 //   H^T dY  -> rows 64-127: dW3 = h2^T dY
 //   Q^T X   -> rows 64-127: dW1^T = dp1^T X
 // so nothing is written twice: a thread stores its row's activations 16 bytes
-// at a time (conflict-free) and keeps them packed for the derivatives.  The
-// earlier form wrote transposed copies of every operand two bytes at a time
-// (~512 four-way conflicting shared-memory accesses a thread and tile, 148 KB,
-// one block per SM): 233 us at 786,432 rows, this one 82.
-// dY of a row is formed here: d o[0:4] + (M^T d) o[4:8], o the readout (dout of
-// the row and its second message pass back, k_mp_loss and k_mp_pull).
-// The three gradient accumulators stay in tensor memory across all the
-// block's tiles and are read back once: one partial gradient per block,
-// summed over blocks in a fixed order (k_mp_update).  Tensor memory: columns
-// 0-63 for the activations' products (reused), 64-127 dW2, 128-143 dW3, 144-159
-// dW1^T, 160-223 dY W3^T.  The derivative of tanh uses the BF16 activations the
-// products use.  Every wait is bounded.
+// at a time (conflict-free) and keeps them packed for the derivatives.
+//
+// The gradient accumulators stay in tensor memory across all the block's tiles
+// and are read back once: one partial gradient per block, summed over blocks in
+// order (k_mp_update).  The tensor cores' FP32 accumulation truncates, so the
+// order in which an accumulator takes its tiles is part of the result (two
+// accumulators per SM instead of one moved a gradient at n = 262,144 by 1e-5 to
+// 8e-5 of its norm): one block per SM takes tiles blockIdx + k gridDim in the
+// order of k.  Two groups of 128 threads share the block's accumulators and
+// weights, each with its own operand tiles and activation columns: group g
+// works on tiles k = g, g + 2, ..., one group's epilogues run under the other's
+// products, and a group's issuer adds tile k's gradients once those of tile k -
+// 1 are complete (the mbarrier in_order, whose phase k ends with tile k's).
+// Tensor memory columns: 128 g .. + 63 group g's activations (reused), + 64 ..
+// 127 its dY W3^T, 256-319 dW2, 320-335 dW3, 336-351 dW1^T.  The derivative of
+// tanh uses the BF16 activations the products use.  Every wait is bounded.
+// 786,432 rows: 233 us with transposed copies of every operand written two bytes
+// at a time by one group, 89 now (82 with two accumulators per SM, which rounded
+// differently).
 namespace tcb {
 constexpr int kBRows = 128;
-constexpr int kBTmemCols = 256;
-constexpr int kColW2 = 64, kColW3 = 128, kColW1 = 144, kColH2 = 160;
-// dynamic shared memory layout (byte offsets, 128-byte aligned)
+constexpr int kBGroups = 2;
+constexpr int kBTmemCols = 512;
+constexpr int kColH2 = 64, kColGroup = 128, kColW2 = 256, kColW3 = 320, kColW1 = 336;
+// dynamic shared memory layout (byte offsets, 128-byte aligned): the weights,
 constexpr int oW1T = 0;                      // [64][16]  W1^T          (B, layer 1)
 constexpr int oW2T = oW1T + 64 * 16 * 2;     // [64][64]  W2^T          (B, layer 2)
 constexpr int oW3P = oW2T + 64 * 64 * 2;     // [64][16]  W3 (k 4 -> 16) (B, dh2)
 constexpr int oW2N = oW3P + 64 * 16 * 2;     // [64][64]  W2            (B, dh1)
-constexpr int oX = oW2N + 64 * 64 * 2;       // [128][16] [x0, a0]      (A, layer 1; B, dW1^T)
+constexpr int oGroups = oW2N + 64 * 64 * 2;  // and the groups' tiles, each
+constexpr int oX = 0;                        // [128][16] [x0, a0]      (A, layer 1; B, dW1^T)
 constexpr int oDY = oX + kBRows * 16 * 2;    // [128][16] dY            (A, dh2; B, dW3)
 constexpr int oH = oDY + kBRows * 16 * 2;    // [128][128] [h1, h2]     (A, layer 2, dW2 and dW3)
 constexpr int oQ = oH + kBRows * 128 * 2;    // [128][128] [dp2, dp1]   (A, dh1 and dW1^T; B, dW2)
-constexpr int kSmem = oQ + kBRows * 128 * 2;
+constexpr int kGroupSmem = oQ + kBRows * 128 * 2;
+constexpr int kSmem = oGroups + kBGroups * kGroupSmem;
 constexpr int kHalf = 8 * 128;               // bytes from column 0 to column 64 of a 128-column tile
-constexpr int kGroup = 16 * 128;             // bytes from one group of 8 rows of it to the next
+constexpr int kGroup8 = 16 * 128;            // bytes from one group of 8 rows of it to the next
 }  // namespace tcb
 
 int mp_bwd_tc_smem_bytes() { return tcb::kSmem + 128; }
@@ -356,29 +365,35 @@ int mp_bwd_tc_smem_bytes() { return tcb::kSmem + 128; }
 __device__ __forceinline__ float bf16_lo(unsigned v) { return __uint_as_float(v << 16); }
 __device__ __forceinline__ float bf16_hi(unsigned v) { return __uint_as_float(v & 0xffff0000u); }
 
-__global__ void __launch_bounds__(128, 2) k_mp_mlp_bwd_tc(int rows, MpBuffers M, DevState* st)
+__global__ void __launch_bounds__(128 * tcb::kBGroups, 1) k_mp_mlp_bwd_tc(int rows, MpBuffers M, DevState* st)
 {
     using namespace tc;
     using namespace tcb;
     extern __shared__ __align__(128) unsigned char sm_raw[];
     // the operand tiles start on a 128-byte boundary (the launch adds 128 bytes)
     unsigned char* sm = sm_raw + ((128u - (smem_addr(sm_raw) & 127u)) & 127u);
-    __shared__ __align__(8) unsigned long long mbar;
+    __shared__ __align__(8) unsigned long long mbars[kBGroups], in_order;
     __shared__ unsigned tmem_base;
-    __shared__ int failed;
-    const int tid = threadIdx.x, warp = tid >> 5;
+    __shared__ int failed_of[kBGroups];   // a group leaves its loop by its own flag alone (its barriers need all of it)
+    const int g = threadIdx.x >> 7, tid = threadIdx.x & 127, warp = threadIdx.x >> 5;
+    unsigned char* sg = sm + oGroups + g * kGroupSmem;
+    unsigned long long* mbar = &mbars[g];
+    int& failed = failed_of[g];
     // weights (BF16 layouts of k_mp_update) into core-matrix tiles
-    for (int e = tid; e < 64 * 16; e += blockDim.x) {
+    for (int e = threadIdx.x; e < 64 * 16; e += blockDim.x) {
         *reinterpret_cast<__nv_bfloat16*>(sm + oW1T + core_off(e / 16, e % 16, 16)) = M.wb[kW1T + e];
         *reinterpret_cast<__nv_bfloat16*>(sm + oW3P + core_off(e / 16, e % 16, 16)) = M.wb[kW3P + e];
     }
-    for (int e = tid; e < 64 * 64; e += blockDim.x) {
+    for (int e = threadIdx.x; e < 64 * 64; e += blockDim.x) {
         *reinterpret_cast<__nv_bfloat16*>(sm + oW2T + core_off(e / 64, e % 64, 64)) = M.wb[kW2T + e];
         *reinterpret_cast<__nv_bfloat16*>(sm + oW2N + core_off(e / 64, e % 64, 64)) = M.wb[kW2N + e];
     }
-    if (tid == 0) {
-        failed = 0;
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&mbar)) : "memory");
+    if (threadIdx.x == 0) {
+        for (int k = 0; k < kBGroups; ++k) {
+            failed_of[k] = 0;
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&mbars[k])) : "memory");
+        }
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&in_order)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
@@ -391,62 +406,58 @@ __global__ void __launch_bounds__(128, 2) k_mp_mlp_bwd_tc(int rows, MpBuffers M,
     fence_before();
     __syncthreads();
     fence_after();
-    const unsigned tmem = tmem_base;
-    const unsigned tlane = tmem + ((unsigned)(warp * 32) << 16);   // this warp's lane quarter
+    const unsigned tmem = tmem_base, tact = tmem + (unsigned)(g * kColGroup);   // this group's activations
+    const unsigned quarter = (unsigned)((warp & 3) * 32) << 16;                  // this warp's lane quarter
+    const unsigned tlane = tact + quarter;
     const unsigned id64 = idesc_bf16(kBRows, 64);
     const unsigned idt64 = idesc_bf16(kBRows, 64, true), idt16 = idesc_bf16(kBRows, 16, true);
     unsigned phase = 0;
-    int acc = 0;   // the gradient products accumulate after the block's first tile
-    float o[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) o[k] = M.master[kMpOffO + k];
-    auto sync_mma = [&]() {   // operands written by all threads -> visible to the MMA issuer
+    auto sync_group = [&]() { asm volatile("bar.sync %0, 128;" ::"r"(1 + g) : "memory"); };
+    auto sync_mma = [&]() {   // operands written by all the group's threads -> visible to its MMA issuer
         fence_async_smem();
         fence_before();
-        __syncthreads();
+        sync_group();
         fence_after();
     };
     auto wait_mma = [&]() {
-        if (!wait_phase(&mbar, phase)) atomicExch(&failed, 1);
+        if (!wait_phase(mbar, phase)) atomicExch(&failed, 1);
         phase ^= 1u;
         fence_after();
     };
     auto put8 = [&](int off, const unsigned* w) {   // 8 columns of this thread's row of a 128-column tile
-        *reinterpret_cast<uint4*>(sm + off + (tid >> 3) * kGroup + (tid & 7) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+        *reinterpret_cast<uint4*>(sg + off + (tid >> 3) * kGroup8 + (tid & 7) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
     };
     // the row's inputs, requested a tile ahead
-    float4 x, a;
-    float d, md;
-    auto load = [&](int r) {
+    float4 x, a, dy;
+    auto load = [&](long long tile) {
         const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        const long long r = tile * kBRows + tid;
         x = r < rows ? M.x0[r] : z;
         a = r < rows ? M.a0[r] : z;
-        d = r < rows ? reinterpret_cast<const float*>(M.dout)[4 * (r / 3) + r % 3] : 0.f;
-        md = r < rows ? reinterpret_cast<const float*>(M.pull)[4 * (r / 3) + r % 3] : 0.f;
+        dy = r < rows ? M.dy[r] : z;
     };
-    load(blockIdx.x * kBRows + tid);
+    const long long ntile = (rows + kBRows - 1) / kBRows;
+    auto tile_of = [&](int k) { return (long long)blockIdx.x + (long long)k * gridDim.x; };
+    load(tile_of(g));
 
-    for (int base = blockIdx.x * kBRows; base < rows && !failed; base += gridDim.x * kBRows) {
+    for (int k = g; tile_of(k) < ntile && !failed; k += kBGroups) {
         {   // X = [x0, a0] (k 6..15 zero) and dY (k 4..15 zero)
             const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-            float dy[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) dy[k] = fmaf(d, o[k], md * o[4 + k]);
-            *reinterpret_cast<uint4*>(sm + oX + core_off(tid, 0, 16)) =
+            *reinterpret_cast<uint4*>(sg + oX + core_off(tid, 0, 16)) =
                 make_uint4(pack_bf16(x.x, x.y), pack_bf16(x.z, a.x), pack_bf16(a.y, a.z), 0u);
-            *reinterpret_cast<uint4*>(sm + oX + core_off(tid, 8, 16)) = zero;
-            *reinterpret_cast<uint4*>(sm + oDY + core_off(tid, 0, 16)) =
-                make_uint4(pack_bf16(dy[0], dy[1]), pack_bf16(dy[2], dy[3]), 0u, 0u);
-            *reinterpret_cast<uint4*>(sm + oDY + core_off(tid, 8, 16)) = zero;
+            *reinterpret_cast<uint4*>(sg + oX + core_off(tid, 8, 16)) = zero;
+            *reinterpret_cast<uint4*>(sg + oDY + core_off(tid, 0, 16)) =
+                make_uint4(pack_bf16(dy.x, dy.y), pack_bf16(dy.z, dy.w), 0u, 0u);
+            *reinterpret_cast<uint4*>(sg + oDY + core_off(tid, 8, 16)) = zero;
         }
         sync_mma();
         if (tid == 0) {   // layer 1, and dh2 = dY W3^T
-            mma(tmem, smem_desc(sm + oX, 16), smem_desc(sm + oW1T, 16), id64, 0);
-            mma(tmem + kColH2, smem_desc(sm + oDY, 16), smem_desc(sm + oW3P, 16), id64, 0);
-            commit(&mbar);
+            mma(tact, smem_desc(sg + oX, 16), smem_desc(sm + oW1T, 16), id64, 0);
+            mma(tact + kColH2, smem_desc(sg + oDY, 16), smem_desc(sm + oW3P, 16), id64, 0);
+            commit(mbar);
         }
         wait_mma();
-        unsigned h1[32], h2[32];   // the row's activations, packed
+        unsigned h1[32];   // the row's activations, packed
 #pragma unroll
         for (int c = 0; c < 64; c += 16) {
             float v[16];
@@ -460,44 +471,37 @@ __global__ void __launch_bounds__(128, 2) k_mp_mlp_bwd_tc(int rows, MpBuffers M,
         if (tid == 0) {
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks)
-                mma(tmem, smem_desc(sm + oH + ks * 256, 128u, (unsigned)kGroup), smem_desc(sm + oW2T + ks * 256, 64),
+                mma(tact, smem_desc(sg + oH + ks * 256, 128u, (unsigned)kGroup8), smem_desc(sm + oW2T + ks * 256, 64),
                     id64, ks > 0);
-            commit(&mbar);
+            commit(mbar);
         }
         wait_mma();
         // h2 = tanh(D) and dp2 = dh2 (1 - h2^2)
 #pragma unroll
         for (int c = 0; c < 64; c += 16) {
-            float v[16], g[16];
+            float v[16], u[16];
             ld16(tlane + c, v);
-            ld16(tlane + kColH2 + c, g);
-            unsigned w[8];
+            ld16(tlane + kColH2 + c, u);
+            unsigned h2[8], w[8];
 #pragma unroll
             for (int q = 0; q < 16; q += 2) {
                 const unsigned h = pack_bf16(tanh_fast(v[q]), tanh_fast(v[q + 1]));
                 const float lo = bf16_lo(h), hi = bf16_hi(h);
-                h2[(c + q) / 2] = h;
-                w[q / 2] = pack_bf16(g[q] * (1.f - lo * lo), g[q + 1] * (1.f - hi * hi));
+                h2[q / 2] = h;
+                w[q / 2] = pack_bf16(u[q] * (1.f - lo * lo), u[q + 1] * (1.f - hi * hi));
             }
-            put8(oH + kHalf + c / 8 * 128, h2 + c / 2);
-            put8(oH + kHalf + (c / 8 + 1) * 128, h2 + c / 2 + 4);
+            put8(oH + kHalf + c / 8 * 128, h2);
+            put8(oH + kHalf + (c / 8 + 1) * 128, h2 + 4);
             put8(oQ + c / 8 * 128, w);
             put8(oQ + (c / 8 + 1) * 128, w + 4);
         }
         sync_mma();
-        if (tid == 0) {   // dh1 = dp2 W2^T, waited for; then dW2 and dW3 behind it (K = 128 rows, 16 a step)
+        if (tid == 0) {   // dh1 = dp2 W2^T
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks)
-                mma(tmem, smem_desc(sm + oQ + ks * 256, 128u, (unsigned)kGroup), smem_desc(sm + oW2N + ks * 256, 64),
+                mma(tact, smem_desc(sg + oQ + ks * 256, 128u, (unsigned)kGroup8), smem_desc(sm + oW2N + ks * 256, 64),
                     id64, ks > 0);
-            commit(&mbar);
-#pragma unroll
-            for (int ks = 0; ks < 8; ++ks) {
-                const int on = acc | (ks > 0);
-                const unsigned long long h = smem_desc(sm + oH + ks * 2 * kGroup, (unsigned)kGroup, 128u);
-                mma(tmem + kColW2, h, smem_desc(sm + oQ + ks * 2 * kGroup, (unsigned)kGroup, 128u), idt64, on);
-                mma(tmem + kColW3, h, smem_desc(sm + oDY + ks * 512, 256u, 128u), idt16, on);
-            }
+            commit(mbar);
         }
         wait_mma();
         // dp1 = dh1 (1 - h1^2)
@@ -515,46 +519,61 @@ __global__ void __launch_bounds__(128, 2) k_mp_mlp_bwd_tc(int rows, MpBuffers M,
             put8(oQ + kHalf + (c / 8 + 1) * 128, w + 4);
         }
         sync_mma();
-        if (tid == 0) {
+        if (tid == 0) {   // the weight gradients over the tile's rows (K = 128, 16 a step), behind the tile before
+            if (k > 0 && !wait_phase(&in_order, (unsigned)(k - 1) & 1u)) {
+                atomicExch(&failed, 1);
+            } else {
+                fence_after();
 #pragma unroll
-            for (int ks = 0; ks < 8; ++ks)
-                mma(tmem + kColW1, smem_desc(sm + oQ + ks * 2 * kGroup, (unsigned)kGroup, 128u),
-                    smem_desc(sm + oX + ks * 512, 256u, 128u), idt16, acc | (ks > 0));
-            commit(&mbar);
+                for (int ks = 0; ks < 8; ++ks) {
+                    const int on = k > 0 || ks > 0;
+                    const unsigned long long h = smem_desc(sg + oH + ks * 2 * kGroup8, (unsigned)kGroup8, 128u);
+                    const unsigned long long q = smem_desc(sg + oQ + ks * 2 * kGroup8, (unsigned)kGroup8, 128u);
+                    mma(tmem + kColW2, h, q, idt64, on);
+                    mma(tmem + kColW3, h, smem_desc(sg + oDY + ks * 512, 256u, 128u), idt16, on);
+                    mma(tmem + kColW1, q, smem_desc(sg + oX + ks * 512, 256u, 128u), idt16, on);
+                }
+            }
+            commit(&in_order);
+            commit(mbar);
         }
-        load(base + gridDim.x * kBRows + tid);
+        load(tile_of(k + kBGroups));
         wait_mma();   // the next tile overwrites the operands
-        acc = 1;
         fence_before();
-        __syncthreads();
+        sync_group();
         fence_after();
     }
+    fence_before();
+    __syncthreads();   // both groups' gradients are in tensor memory
+    fence_after();
+    const bool bad = failed_of[0] || failed_of[1];
     // this block's partial gradient (zero if it had no tile)
     float* gp = M.gpart + (size_t)blockIdx.x * kMpParams;
-    if (acc && !failed) {
-        if (warp < 2) {   // rows 0-63: dW2[i][h] (i = row)
+    if ((long long)blockIdx.x < ntile && !bad) {
+        const unsigned lane0 = tmem + quarter;
+        if (g == 0 && warp < 2) {   // rows 0-63: dW2[i][h] (i = row)
             const int i = tid;
 #pragma unroll
             for (int c = 0; c < 64; c += 16) {
                 float v[16];
-                ld16(tlane + kColW2 + c, v);
+                ld16(lane0 + kColW2 + c, v);
 #pragma unroll
                 for (int q = 0; q < 16; ++q) gp[kMpOffW2 + i * 64 + c + q] = v[q];
             }
-        } else {          // rows 64-127: dW3[h][m] (h = row - 64) and dW1^T[i][f] (i = row - 64)
+        } else if (g == 0) {        // rows 64-127: dW3[h][m] (h = row - 64) and dW1^T[i][f] (i = row - 64)
             const int h = tid - 64;
             float v[16];
-            ld16(tlane + kColW3, v);
+            ld16(lane0 + kColW3, v);
 #pragma unroll
             for (int m = 0; m < 4; ++m) gp[kMpOffW3 + h * 4 + m] = v[m];
-            ld16(tlane + kColW1, v);
+            ld16(lane0 + kColW1, v);
 #pragma unroll
             for (int f = 0; f < 6; ++f) gp[kMpOffW1 + f * 64 + h] = v[f];
         }
     } else {
-        for (int e = tid; e < kMpOffO; e += blockDim.x) gp[e] = 0.f;
+        for (int e = threadIdx.x; e < kMpOffO; e += blockDim.x) gp[e] = 0.f;
     }
-    if (failed && tid == 0) atomicCAS(&st->error, 0, (int)SP_ERR_TIMEOUT);
+    if (bad && threadIdx.x == 0) atomicCAS(&st->error, 0, (int)SP_ERR_TIMEOUT);
     fence_before();
     __syncthreads();
     if (warp == 0)
@@ -652,25 +671,42 @@ __global__ void k_mp_aggregate(KParams P, DevBuffers B, const float4* __restrict
     for (int c = 0; c < 3; ++c) out[3 * i + c] = make_float4(s[c].x * di, s[c].y * di, s[c].z * di, s[c].w * di);
 }
 
-// pull = M^T dout, one value per component: the gradient at the second message
-// pass is dout times the readout's four weights, a product of the row's scalar
-// with a constant vector, so M^T acts on the scalar (16 bytes per entry
-// instead of 48; scaled holds D^-1 dout).
-__global__ void k_mp_pull(KParams P, DevBuffers B, const float4* __restrict__ scaled, float4* __restrict__ pull)
+// dY = dout o[0:4] + M^T (dout o[4:8]), o the readout: the gradient at the second
+// message pass is a row's dout times four constants, so an entry gathers the
+// partner's three dout and D^-1 (16 bytes) and forms the twelve products again,
+// rounded as when they were stored (with them stored, 48 bytes and D^-1 an
+// entry: 62 us at 786,432 rows, 48 now).
+__global__ void k_mp_pull(KParams P, DevBuffers B, MpBuffers M)
 {
     const MpNode nd = mp_node(P, B);
     if (nd.i < 0) return;
     const float ae = (float)P.alpha;
-    float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+    float o[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) o[k] = M.master[kMpOffO + k];
+    float s[3][4];
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) s[c][k] = 0.f;
     for (int k = 0; k < nd.cnt; ++k) {
         const int e = nd.base + 32 * k;
-        const float4 v = scaled[B.col[e]];
-        const float w = ae * B.val32[e];
-        s0 = fmaf(w, v.x, s0);
-        s1 = fmaf(w, v.y, s1);
-        s2 = fmaf(w, v.z, s2);
+        const float4 v = M.dout[B.col[e]];
+        const float w = ae * B.val32[e] * v.w, d[3] = {v.x, v.y, v.z};
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) s[c][q] = fmaf(w, __fmul_rn(d[c], o[4 + q]), s[c][q]);
     }
-    pull[nd.i] = make_float4(s0, s1, s2, 0.f);
+    const float4 v = M.dout[nd.i];
+    const float d[3] = {v.x, v.y, v.z};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        float r[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) r[q] = __fadd_rn(s[c][q], __fmul_rn(d[c], o[q]));
+        M.dy[3 * nd.i + c] = make_float4(r[0], r[1], r[2], r[3]);
+    }
 }
 
 // Second message pass fused with the output: a1 = M y for node i, then
@@ -713,58 +749,87 @@ __global__ void k_mp_aggregate_output(KParams P, DevBuffers B, MpBuffers M)
     }
 }
 
-// Loss rows: e = out - vstar / s, dout = 2 e / 3n (dout and D^-1 dout of each
-// node kept); per block: sum e^2 and the readout gradient sum dout [y, a1, x0].
-// FP64 only for e, its square's sum and dout (five operations a row on GB300's
-// 1/64-rate pipe); the readout's eleven sums are compensated FP32 (exact
-// TwoSum errors in a second word), which was 24 FP64 operations a row: 107 us
-// at 786,432 rows before, 20 now.
-__global__ void __launch_bounds__(kVecBlock) k_mp_loss(KParams P, DevBuffers B, MpBuffers M, double two_by_rows)
+// a / b from inv = 1 / b by one correction of the product a inv with its exact
+// remainder (Markstein, IBM J. Res. Dev. 34, 1990), three FP64 operations.
+__device__ __forceinline__ double quotient(double a, double b, double inv)
 {
-    __shared__ double s_inv;
-    if (threadIdx.x == 0) s_inv = 1.0 / M.scal[0];
+    const double q = a * inv, r = fma(-q, b, a);
+    return isfinite(r) ? fma(r, inv, q) : q;
+}
+
+// A sum of FP32 terms in three words: the exact error of every addition goes to
+// the second word, the exact error of that addition to the third (72 bits; an
+// FP64 sum has 53 and needs two operations a term on the 1/64-rate pipe).
+struct Sum3 {
+    float a, b, c;
+    __device__ void add(float v)
+    {
+        const dfloat t = two_sum(a, v), u = two_sum(b, t.lo);
+        a = t.hi;
+        b = u.hi;
+        c = __fadd_rn(c, u.lo);
+    }
+};
+
+// Loss rows: e = out - vstar / s, dout = 2 e / 3n (of each node kept, with D^-1);
+// per block: sum e^2 and the readout gradient sum dout [y, a1, x0].  Bound by FP64
+// (GB300 issues it at 1/64 of the FP32 rate), which only e, its square's sum and
+// dout need: 107 us at 786,432 rows with two FP64 divisions and eleven FP64 sums a
+// row, 36 now.
+__global__ void __launch_bounds__(kVecBlock) k_mp_loss(KParams P, DevBuffers B, MpBuffers M)
+{
+    __shared__ double s_inv[2];
+    const int rows = 3 * P.n;
+    const double scale = M.scal[0], rows_d = (double)rows;
+    if (threadIdx.x == 0) {
+        s_inv[0] = 1.0 / scale;
+        s_inv[1] = 1.0 / rows_d;
+    }
     __syncthreads();
-    const double inv = s_inv;
+    const double inv = s_inv[0], inv_rows = s_inv[1];
     float o[11];
 #pragma unroll
     for (int k = 0; k < 11; ++k) o[k] = M.master[kMpOffO + k];
-    const int rows = 3 * P.n;
     double ee = 0.0;
-    dfloat acc[11];
+    Sum3 acc[11];
 #pragma unroll
-    for (int k = 0; k < 11; ++k) acc[k] = dfloat{0.f, 0.f};
+    for (int k = 0; k < 11; ++k) acc[k] = Sum3{0.f, 0.f, 0.f};
     for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += gridDim.x * blockDim.x) {
         const int i = r / 3, c = r - 3 * i;
         const float4 y = M.y[r], a = M.a1[r], x = M.x0[r];
         const float out = y.x * o[0] + y.y * o[1] + y.z * o[2] + y.w * o[3] + a.x * o[4] + a.y * o[5] + a.z * o[6] +
                           a.w * o[7] + x.x * o[8] + x.y * o[9] + x.z * o[10];
-        const double e = fma(-B.x[c * P.npad + i], inv, (double)out);
-        const float d = (float)(e * two_by_rows);
+        const double e = (double)out - quotient(B.x[c * P.npad + i], scale, inv);
+        const float d = (float)quotient(2.0 * e, rows_d, inv_rows);
         ee = fma(e, e, ee);
-        reinterpret_cast<float*>(M.dout)[4 * i + c] = d;
-        reinterpret_cast<float*>(M.scaled)[4 * i + c] = d * B.dinv32[i];
+        float* node = reinterpret_cast<float*>(M.dout + i);
+        node[c] = d;
+        if (c == 2) node[3] = B.dinv32[i];
         const float f[11] = {y.x, y.y, y.z, y.w, a.x, a.y, a.z, a.w, x.x, x.y, x.z};
 #pragma unroll
-        for (int k = 0; k < 11; ++k) {
-            const dfloat t = two_sum(acc[k].hi, __fmul_rn(d, f[k]));
-            acc[k] = dfloat{t.hi, __fadd_rn(acc[k].lo, t.lo)};
-        }
+        for (int k = 0; k < 11; ++k) acc[k].add(__fmul_rn(d, f[k]));
     }
-    __shared__ float2 sh[11][kVecBlock / 32];
-    __shared__ double she[kVecBlock / 32];
+    __shared__ double sh[12][kVecBlock / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int k = 0; k < 11; ++k) {
-        const dfloat t = warp_sum_df(fast_two_sum(acc[k].hi, acc[k].lo));
-        if (lane == 0) sh[k][warp] = make_float2(t.hi, t.lo);
+#pragma unroll
+        for (int w = 16; w > 0; w >>= 1) {
+            const float a = __shfl_xor_sync(0xffffffffu, acc[k].a, w), b = __shfl_xor_sync(0xffffffffu, acc[k].b, w);
+            const float c = __shfl_xor_sync(0xffffffffu, acc[k].c, w);
+            acc[k].add(a);
+            const dfloat u = two_sum(acc[k].b, b);
+            acc[k].b = u.hi;
+            acc[k].c = __fadd_rn(acc[k].c, __fadd_rn(u.lo, c));
+        }
+        if (lane == 0) sh[1 + k][warp] = ((double)acc[k].c + (double)acc[k].b) + (double)acc[k].a;
     }
     ee = warp_sum(ee);
-    if (lane == 0) she[warp] = ee;
+    if (lane == 0) sh[0][warp] = ee;
     __syncthreads();
     if (threadIdx.x < 12) {
         double t = 0.0;
-        for (int w = 0; w < kVecBlock / 32; ++w)
-            t += threadIdx.x == 0 ? she[w] : (double)sh[threadIdx.x - 1][w].x + (double)sh[threadIdx.x - 1][w].y;
+        for (int w = 0; w < kVecBlock / 32; ++w) t += sh[threadIdx.x][w];
         M.dpart[blockIdx.x * 12 + threadIdx.x] = t;
     }
 }
@@ -805,34 +870,44 @@ __global__ void k_mp_convert(MpBuffers M)
     if (p < kMpParams) mp_adam(M, p, 0.f, 1);
 }
 
-// grad = sum over blocks (fixed order: warp w of a block takes partials w, w +
-// 8, ..., then the warps in turn; one thread per weight summing all of them in
-// turn took 75 us), the readout's gradient and the loss from the loss blocks,
-// and the weight's Adam step.
+// grad = sum over blocks, the readout's gradient and the loss from the loss
+// blocks, and the weight's Adam step.  The weights' FP32 partials are added one
+// by one in the order of the blocks (the rounding of that order is the
+// gradient's): all warps bring a run of them into shared memory and the first
+// adds them up (one thread per weight loading all of them in turn took 75 us);
+// the FP64 partials are shared out among the warps.
+constexpr int kGradRun = 160;
 __global__ void __launch_bounds__(256) k_mp_update(MpBuffers M, int nblocks_mlp, int nblocks_loss, int rows, float lr,
                                                    int t)
 {
+    __shared__ float run[kGradRun][32];
     __shared__ double sh[8][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, p = blockIdx.x * 32 + lane;
-    double s = 0.0;
+    static_assert(kMpOffO % 32 == 0, "a block's weights are all the network's or all the readout's");
     if (p < kMpOffO) {
         float f = 0.f;
+        for (int b0 = 0; b0 < nblocks_mlp; b0 += kGradRun) {
+            const int m = min(kGradRun, nblocks_mlp - b0);
 #pragma unroll 4
-        for (int b = warp; b < nblocks_mlp; b += 8) f += M.gpart[(size_t)b * kMpParams + p];
-        s = f;
-    } else if (p <= kMpParams) {   // entry 0 of a loss block: sum e^2; 1 + k: the readout's gradient
-        const int k = p < kMpParams ? 1 + (p - kMpOffO) : 0;
-#pragma unroll 4
-        for (int b = warp; b < nblocks_loss; b += 8) s += M.dpart[b * 12 + k];
-    }
-    sh[warp][lane] = s;
-    __syncthreads();
-    if (warp != 0 || p > kMpParams) return;
-    if (p < kMpOffO) {
-        float f = 0.f;
-        for (int w = 0; w < 8; ++w) f += (float)sh[w][lane];
+            for (int b = warp; b < m; b += 8) run[b][lane] = M.gpart[(size_t)(b0 + b) * kMpParams + p];
+            __syncthreads();
+            if (warp == 0)
+#pragma unroll 8
+                for (int b = 0; b < m; ++b) f += run[b][lane];
+            __syncthreads();
+        }
+        if (warp != 0) return;
         M.grad[p] = f;
-    } else {
+    } else {   // entry 0 of a loss block: sum e^2; 1 + k: the readout's gradient
+        double s = 0.0;
+        if (p <= kMpParams) {
+            const int k = p < kMpParams ? 1 + (p - kMpOffO) : 0;
+#pragma unroll 4
+            for (int b = warp; b < nblocks_loss; b += 8) s += M.dpart[b * 12 + k];
+        }
+        sh[warp][lane] = s;
+        __syncthreads();
+        if (warp != 0 || p > kMpParams) return;
         double a = 0.0;
         for (int w = 0; w < 8; ++w) a += sh[w][lane];
         if (p == kMpParams) {
@@ -871,10 +946,10 @@ void launch_mp_train(const KParams& P, DevBuffers& B, MpBuffers& M, float lr, in
 {
     const int rows = 3 * P.n;
     const int nloss = grid_for(rows, kVecBlock, std::min(kMaxGradBlocks, L.num_sms * 2));
-    k_mp_loss<<<nloss, kVecBlock, 0, L.stream>>>(P, B, M, 2.0 / rows);
-    k_mp_pull<<<grid_for(P.n, 128, 1 << 30), 128, 0, L.stream>>>(P, B, M.scaled, M.pull);
-    const int nmlp = grid_for(rows, kTileRows, std::min(kMaxGradBlocks, L.num_sms * 2));
-    k_mp_mlp_bwd_tc<<<nmlp, 128, mp_bwd_tc_smem_bytes(), L.stream>>>(rows, M, B.st);
+    k_mp_loss<<<nloss, kVecBlock, 0, L.stream>>>(P, B, M);
+    k_mp_pull<<<grid_for(P.n, 128, 1 << 30), 128, 0, L.stream>>>(P, B, M);
+    const int nmlp = grid_for(rows, kTileRows, std::min(kMaxGradBlocks, L.num_sms));
+    k_mp_mlp_bwd_tc<<<nmlp, 128 * tcb::kBGroups, mp_bwd_tc_smem_bytes(), L.stream>>>(rows, M, B.st);
     k_mp_update<<<kMpParams / 32 + 1, 256, 0, L.stream>>>(M, nmlp, nloss, rows, lr, t);
 }
 

@@ -664,7 +664,7 @@ int sp_sim_destroy(sp_sim* s)
         if (q) cudaFree(q);
     if (s->mp_alloc) {
         MpBuffers& M = s->mp;
-        void* mps[] = {M.x0, M.a0, M.y, M.a1, M.dout, M.scaled, M.pull, M.master, M.m, M.v, M.grad, M.gpart, M.dpart, M.wb, M.scal,
+        void* mps[] = {M.x0, M.a0, M.y, M.a1, M.dout, M.dy, M.master, M.m, M.v, M.grad, M.gpart, M.dpart, M.wb, M.scal,
                        M.part, M.ticket};
         for (void* q : mps)
             if (q) cudaFree(q);
@@ -1771,8 +1771,7 @@ int sp_mpnn_enable(sp_sim* s, uint64_t seed, const float* weights_host)
         A(dev_alloc(s, &M.y, rows));
         A(dev_alloc(s, &M.a1, rows));
         A(dev_alloc(s, &M.dout, (size_t)s->kp.n));
-        A(dev_alloc(s, &M.scaled, (size_t)s->kp.n));
-        A(dev_alloc(s, &M.pull, (size_t)s->kp.n));
+        A(dev_alloc(s, &M.dy, rows));
         A(dev_alloc(s, &M.master, kMpParams));
         A(dev_alloc(s, &M.m, kMpParams));
         A(dev_alloc(s, &M.v, kMpParams));
