@@ -21,6 +21,7 @@
 #include <math.h>
 
 #include "internal.cuh"
+#include "sfactor_cell.cuh"
 
 namespace ss {
 
@@ -28,31 +29,22 @@ namespace {
 
 constexpr double kFix = 4294967296.0;   // 2^32
 
-// Fractions of a cell in 2^-40, weights in 2^-32: products of 40-bit integers,
-// rounded to nearest like the FP64 products they replace (their error, below
-// 2^-39, is 1/100 of that rounding), three FP64 operations and two conversions a
-// particle instead of ~150 (four divisions, eight products and four roundings):
-// 33.6 us at n = 262,144 before, 9.3 now.
+// Fractions of a cell in 2^-50, weights in 2^-32: integer products rounded to
+// nearest like the FP64 products they replace, three FP64 operations and two
+// conversions a particle instead of ~150 (four divisions, eight products and four
+// roundings): 33.6 us at n = 262,144 before, 10.0 now.  Every value of a
+// coordinate lands on the grid (grid_cell).
 __global__ void k_sq_deposit(KParams P, const double* __restrict__ pos, double gamma, double sx, double sy, int G,
                              unsigned long long* __restrict__ grid)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= P.n) return;
     const double x = pos[i], y = pos[P.npad + i];
-    constexpr long long kOne = 1ll << 40;
-    const long long u = __double2ll_rd(fma(-gamma, y, x) * sx), v = __double2ll_rd(y * sy);   // grid units x 2^40
-    int i0 = (int)(u >> 40), j0 = (int)(v >> 40);
-    const unsigned long long fu = (unsigned long long)(u & (kOne - 1)) << 12, fv = (unsigned long long)(v & (kOne - 1)) << 12;
-    const unsigned long long gu = ((unsigned long long)kOne << 12) - fu, gv = ((unsigned long long)kOne << 12) - fv;
-    if (i0 < 0) i0 += G;        // x - gamma y lies in (-L_x, L_x)
-    if (i0 >= G) i0 -= G;
-    if (j0 >= G) j0 -= G;
-    const int i1 = i0 + 1 < G ? i0 + 1 : 0, j1 = j0 + 1 < G ? j0 + 1 : 0;
-    auto weight = [](unsigned long long a, unsigned long long b) { return (__umul64hi(a, b) + 128ull) >> 8; };
-    atomicAdd(grid + (size_t)j0 * G + i0, weight(gu, gv));
-    atomicAdd(grid + (size_t)j0 * G + i1, weight(fu, gv));
-    atomicAdd(grid + (size_t)j1 * G + i0, weight(gu, fv));
-    atomicAdd(grid + (size_t)j1 * G + i1, weight(fu, fv));
+    const GridCell u = grid_cell(fma(-gamma, y, x) * sx, G), v = grid_cell(y * sy, G);
+    atomicAdd(grid + (size_t)v.i0 * G + u.i0, cell_weight(u.g, v.g));
+    atomicAdd(grid + (size_t)v.i0 * G + u.i1, cell_weight(u.f, v.g));
+    atomicAdd(grid + (size_t)v.i1 * G + u.i0, cell_weight(u.g, v.f));
+    atomicAdd(grid + (size_t)v.i1 * G + u.i1, cell_weight(u.f, v.f));
 }
 
 // Block gy: A[kx][gy] = sum_gx rho[gy][gx] exp(-2 pi i kx gx / G) for kx =
@@ -225,7 +217,7 @@ cudaError_t run_structure_factor(const KParams& P, const DevBuffers& B, double d
         return cudaGetLastError();
     }
     cudaMemsetAsync(grid_dev, 0, sizeof(unsigned long long) * (size_t)G * G, s);
-    const double unit = 1099511627776.0 * G;   // 2^40 per grid cell
+    const double unit = kCellUnit * G;
     k_sq_deposit<<<grid_for(P.n, kVecBlock, 1 << 30), kVecBlock, 0, s>>>(P, B.pos_s, delta / P.L[1], unit / P.L[0],
                                                                             unit / P.L[1], G, grid_dev);
     const double2* tw = reinterpret_cast<const double2*>(twiddle_dev);

@@ -51,3 +51,25 @@ def test_grid_structure_factor_matches_numpy(G, nkx, nky, n, delta):
     ky = np.arange(-nky, nky + 1)[None, :]
     assert np.allclose(qx, 2 * np.pi * kx / L + 0 * ky, rtol=1e-14, atol=1e-14)
     assert np.allclose(qy, 2 * np.pi * ky / L - delta * 2 * np.pi * kx / L, rtol=1e-13, atol=1e-13)
+
+
+def test_refused_positions_leave_the_call_usable():
+    """Refused positions stay stored ("undefined until valid ones are set"): the deposit puts every
+    value on the grid, and after valid positions the call gives what a new simulation gives."""
+    n, G, k = 3000, 64, 8
+    L = synth.box_length(n)
+    pos = synth.uniform_positions(n, (L,) * 3, 2)
+    ref = ss.Simulation(n, (L,) * 3, 1.0, seed=1, positions=pos)
+    ref.set_positions(pos, 0.3 * L)
+    want = ref.structure_factor(k, k, grid=G)[0]
+    ref.close()
+    bad = pos.copy()
+    bad[:8, 1] = (-0.5 * L, -1e9, 3.7 * L, 1e12, 1e300, np.inf, -np.inf, np.nan)
+    bad[8:14, 0] = (-2.5 * L, 9.0 * L, -1e300, np.inf, np.nan, L)
+    sim = ss.Simulation(n, (L,) * 3, 1.0, seed=1, positions=pos)
+    with pytest.raises(ss.ShearsimError):
+        sim.set_positions(bad, 0.3 * L)
+    assert np.all(np.isfinite(sim.structure_factor(k, k, grid=G)[0]))
+    sim.set_positions(pos, 0.3 * L)
+    assert np.array_equal(sim.structure_factor(k, k, grid=G)[0], want)
+    sim.close()
