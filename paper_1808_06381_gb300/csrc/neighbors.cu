@@ -561,6 +561,15 @@ __device__ __forceinline__ void for_each_neighbor(const KParams& P, double delta
         for_each_neighbor_generic(P, delta, pos, cell_start, i, xi, yi, zi, visit);
 }
 
+// The step's words that the search resets (one thread).  In mode 2 k_row_normals
+// draws the normals beside the search and is the only one to write noise_step
+// (not even its own value is written back here: that could overwrite the new one).
+__device__ __forceinline__ void begin_search(DevState* st, int draw_noise)
+{
+    st->nnz = 0;
+    if (draw_noise != 2) st->noise_step = draw_noise ? st->step : -1;
+}
+
 // The pair search of a step, run once: counts the partners of every row and
 // keeps the first kCandCap of them (partner and image code, k-major so that a
 // warp's stores are coalesced) for the assembly, which places them in the
@@ -570,10 +579,7 @@ __global__ void k_nbr_collect(KParams P, DevBuffers B, int draw_noise)
     DevState* st = B.st;
     if (st->error | st->overflow) return;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0) {
-        st->nnz = 0;
-        if (draw_noise != 2) st->noise_step = draw_noise ? st->step : -1;   // 2: drawn by k_row_normals
-    }
+    if (i == 0) begin_search(st, draw_noise);
     if (i >= P.n) return;
     if (draw_noise == 1) {   // the step's normals of this row (the assembly uses them)
         if (P.mixed) {   // double-float arithmetic; stored as (hi, lo) pairs in the same space
@@ -624,10 +630,7 @@ __global__ void __launch_bounds__(9 * kSplitRows) k_nbr_collect_split(KParams P,
     __shared__ int found[9][kSplitRows];
     const int r = threadIdx.x % kSplitRows, part = threadIdx.x / kSplitRows;   // a warp: 32 rows, the same part
     const int i = blockIdx.x * kSplitRows + r;
-    if (i == 0 && part == 0) {
-        st->nnz = 0;
-        st->noise_step = draw_noise == 2 ? st->noise_step : -1;   // 2: drawn by k_row_normals
-    }
+    if (i == 0 && part == 0) begin_search(st, draw_noise);   // mode 0 or 2: this kernel draws no normals
     const int np = P.npad;
     const double delta = st->delta;
     const double xi = i < P.n ? B.pos_w[i] : 0.0, yi = i < P.n ? B.pos_w[np + i] : 0.0, zi = i < P.n ? B.pos_w[2 * np + i] : 0.0;
