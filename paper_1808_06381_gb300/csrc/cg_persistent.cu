@@ -2323,7 +2323,22 @@ __global__ void __launch_bounds__(p64::max_threads(U), 1) k64_cg_pipelined(KPara
 // b - A x in double-float from the sliced layout, after every reduction of the
 // recursive residual by 10^-4 (KParams::inner2) and at the end.  The sums
 // behind the scalars are FP64 from the row products on.  Bound by the barrier
-// (~2.3 us) and the gathers' latency.  Measured (whole solve of a clustered
+// (~2.3 us) and the gathers' latency.
+// The recurrences for w, s and z carry FP32 rounding that the coupling alpha
+// amplifies: where the matrix is ill conditioned the recursive residual runs
+// away from the true one and the restarts gain little (n = 20,011 clustered, FP32
+// recurrences restated on the host: true over recursive residual 1.02 at alpha = 4,
+// 1.7 at 40, 3.3 at 150, 12 at 1,000; at 4,000 a thousand iterations do not reach
+// 1e-8).  So the solve watches each replacement: when the true residual exceeds the
+// recursive one by kPipelinedDrift, when a cycle between two replacements is longer
+// than kPipelinedCycle iterations (31 at alpha = 4), or when the recurrences break
+// down, the rest of the solve runs the standard recurrence (q = A u + beta q, p = u
+// + beta p; two reductions an iteration, its vectors a subset of these).  On the
+// GPU at alpha = 4, 40, 150, 1,000, 4,000: 64, 158, 239, 335, 310 iterations of
+// the streaming solve, 64, 160, 246, 292, 318 here.  The scalars are FP64, as in
+// the streaming solve (in FP32 1,000 and 4,000 did not converge; they cost 10 us a
+// step at n = 20,011).
+// Measured (whole solve of a clustered
 // system to 1e-8; streaming form / k32_cg_resident / this one): n = 500 0.52 /
 // 0.33 / 0.19 ms, n = 20,011 1.02 / 0.75 / 0.38, n = 48,000 1.03 / 0.69 / 0.43,
 // n = 72,960 1.12 / 0.80 / 0.54, n = 100,000 1.13 / 0.84 / 0.79, n = 145,000
@@ -2378,10 +2393,15 @@ __device__ __forceinline__ void row_product32(const Sys& S, const p64::Shared& s
 }
 
 struct Cg32Scalars {
-    double bnorm2, rr_restart, target, last_res;
-    float rho, den, alpha, beta;
+    double bnorm2, target, last_res, rho, den;
+    double rr_rec;       // ||r||^2 of the recurrences when they were left for the true residual
+    float alpha, beta;   // the step lengths, rounded once
     int iter, restarts, status, first;
+    int plain, cycle;    // 1: two-reduction recurrence; the iteration at which the residual was last replaced
 };
+
+constexpr int kPipelinedCycle = 100;         // iterations between two replacements, at most
+constexpr double kPipelinedDrift2 = 2.0;     // true over recursive ||r||^2 beyond which the recurrences are given up
 
 template <int U, int KB>
 __device__ __forceinline__ void pipelined_solve32(const KParams& P, const DevBuffers& B, const p64::Grid& G,
@@ -2399,7 +2419,7 @@ __device__ __forceinline__ void pipelined_solve32(const KParams& P, const DevBuf
         sh.flag = 0;
         sh.action = 0;
         cg.status = SP_OK;
-        cg.iter = cg.restarts = 0;
+        cg.iter = cg.restarts = cg.plain = cg.cycle = 0;
         cg.last_res = 0.0;
     }
     p64::stage(S, sh, dyn, smem_bytes, nc);
@@ -2412,8 +2432,8 @@ __device__ __forceinline__ void pipelined_solve32(const KParams& P, const DevBuf
     auto publish = [&](int u, const float (&v)[3]) {
         rec[cur ^ 1][row[u]] = make_float4(di[u] * v[0], di[u] * v[1], di[u] * v[2], 0.f);
     };
-    // r = b - A x of the own rows in double-float, u = D^-1 r published; ||r||^2 into v0
-    auto residual = [&](bool product) {
+    // r = b - A x of the own rows in double-float, u = D^-1 r published; ||r||^2 into v0 (and r.u into v1)
+    auto residual = [&](bool product, bool with_ru) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             if (row[u] < 0) continue;
@@ -2431,6 +2451,7 @@ __device__ __forceinline__ void pipelined_solve32(const KParams& P, const DevBuf
                 rs += r[u][c] * r[u][c];
             }
             v0 += (double)rs;
+            if (with_ru) v1 += (double)(di[u] * rs);   // r.u (at the start v1 is ||b||^2; the standard recurrence begins later)
             publish(u, r[u]);
         }
         cur ^= 1;
@@ -2454,11 +2475,12 @@ __device__ __forceinline__ void pipelined_solve32(const KParams& P, const DevBuf
     if (threadIdx.x == 0)   // blocks that read a chunk's entries from memory
         for (int i = 0; i < nc; ++i)
             if (sh.off[i] < 0) v2 = 1.0;
-    residual(from_x);
-    enum { kStart, kIterate, kX, kTrue };   // the values the next reduction carries (kX: none, x was folded)
+    residual(from_x, false);
+    // the values the next reduction carries (kX: none, x was folded); kDirection and kUpdate: the standard recurrence's
+    enum { kStart, kIterate, kX, kTrue, kDirection, kUpdate };
     int phase = kStart;
     auto product = [&] {   // sum_j alpha w_ij of the published vector
-        if (phase == kX) return;
+        if (phase == kX || phase == kDirection) return;
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int i = warp + ncw * u;
@@ -2469,25 +2491,52 @@ __device__ __forceinline__ void pipelined_solve32(const KParams& P, const DevBuf
         sh.action = 0;
         if (phase == kIterate) {
             const double g = sh.tot[0], dl = sh.tot[1], rr = sh.tot[2];
+            cg.rr_rec = rr;
             if (!isfinite(g) || !isfinite(dl) || !isfinite(rr)) {
-                cg.status = SP_ERR_NONFINITE;
-                sh.action = 2;
+                sh.action = 3;   // the cycle's correction is dropped, the standard recurrence goes on from x
+                cg.plain = 1;
             } else if (rr <= cg.target || cg.iter >= P.max_iter) {
                 sh.action = 1;   // the true residual decides
+            } else if (cg.iter - cg.cycle >= kPipelinedCycle) {
+                sh.action = 1;
+                cg.plain = 1;
             } else {
-                const float gf = (float)g, df = (float)dl;
-                const float beta = cg.first ? 0.f : gf / cg.rho;
-                const float den = cg.first ? df : fmaf(-beta * beta, cg.den, df);   // (p, A p) of the new direction
-                if (!(den > 0.f)) {
+                const double beta = cg.first ? 0.0 : g / cg.rho;
+                const double den = cg.first ? dl : fma(-beta * beta, cg.den, dl);   // (p, A p) of the new direction
+                if (!(den > 0.0)) {
                     sh.action = 1;   // lost to rounding: the true residual decides
+                    cg.plain = 1;
                 } else {
-                    cg.beta = beta;
-                    cg.alpha = gf / den;
-                    cg.rho = gf;
+                    cg.beta = (float)beta;
+                    cg.alpha = (float)(g / den);
+                    cg.rho = g;
                     cg.den = den;
                     cg.first = 0;
                     ++cg.iter;
                 }
+            }
+            return;
+        }
+        if (phase == kDirection) {   // p.q
+            const double pq = sh.tot[0];
+            if (!(pq > 0.0) || !isfinite(pq)) {
+                cg.status = SP_ERR_NONFINITE;
+                sh.action = 2;
+            } else {
+                cg.alpha = (float)(cg.rho / pq);
+            }
+            return;
+        }
+        if (phase == kUpdate) {      // r.r, r.u
+            const double rr = sh.tot[0], rz = sh.tot[1];
+            ++cg.iter;
+            if (!isfinite(rr) || !isfinite(rz)) {
+                cg.status = SP_ERR_NONFINITE;
+                sh.action = 2;
+            } else {
+                cg.beta = (float)(rz / cg.rho);
+                cg.rho = rz;
+                if (rr <= cg.target || cg.iter >= P.max_iter) sh.action = 1;
             }
             return;
         }
@@ -2523,30 +2572,70 @@ __device__ __forceinline__ void pipelined_solve32(const KParams& P, const DevBuf
                 sh.action = 2;
             } else {
                 ++cg.restarts;
+                if (rr > kPipelinedDrift2 * cg.rr_rec) cg.plain = 1;
             }
+            cg.rho = sh.tot[1];
         }
         cg.first = 1;
+        cg.cycle = cg.iter;
+        cg.beta = 0.f;
         cg.target = fmax(P.inner2 * rr, kInnerFinal2 * P.tol2 * cg.bnorm2);
     };
     for (;;) {
-        const int K = phase == kX ? 0 : (phase == kTrue ? 1 : 3);
+        const int K = phase == kX ? 0 : (phase == kDirection ? 1 : (phase == kTrue || phase == kUpdate ? 2 : 3));
         if (!p64::reduce_overlapped(G, sh, gen, K, v0, v1, v2, product, scalars)) break;
         if (K > 0 && sh.action == 2) break;
         v0 = v1 = v2 = 0.0;
         if (phase == kX) {
-            residual(true);
+            residual(true, true);
             phase = kTrue;
             continue;
         }
-        if (phase == kIterate && sh.action == 1) {   // x += d (own rows)
+        if (sh.action != 0 && (phase == kIterate || phase == kUpdate)) {   // x += d (own rows)
 #pragma unroll
             for (int u = 0; u < U; ++u)
-                if (row[u] >= 0) fold_correction(B, row[u], make_float4(d[u][0], d[u][1], d[u][2], 0.f));
+                if (row[u] >= 0 && sh.action == 1) fold_correction(B, row[u], make_float4(d[u][0], d[u][1], d[u][2], 0.f));
             phase = kX;
             continue;
         }
-        const bool start = phase != kIterate;   // w = A u (A_ii u = r); else the recurrences
         const float a = cg.alpha, beta = cg.beta;
+        if (phase == kDirection) {   // d += alpha p; r -= alpha q (in s); u published
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (row[u] < 0) continue;
+                float rs = 0.f;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    d[u][c] = fmaf(a, p[u][c], d[u][c]);
+                    r[u][c] = fmaf(-a, s[u][c], r[u][c]);
+                    rs = fmaf(r[u][c], r[u][c], rs);
+                }
+                publish(u, r[u]);
+                v0 += (double)rs;
+                v1 += (double)(di[u] * rs);
+            }
+            cur ^= 1;
+            phase = kUpdate;
+            continue;
+        }
+        if (cg.plain) {   // q = A u + beta q (A_ii u = r); p = u + beta p (beta = 0 after a replacement)
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (row[u] < 0) continue;
+                float pq = 0.f;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const float qk = r[u][c] - sm[u][c], pk = di[u] * r[u][c];
+                    s[u][c] = beta != 0.f ? fmaf(beta, s[u][c], qk) : qk;   // (what stood there may be infinite)
+                    p[u][c] = beta != 0.f ? fmaf(beta, p[u][c], pk) : pk;
+                    pq = fmaf(p[u][c], s[u][c], pq);
+                }
+                v0 += (double)pq;
+            }
+            phase = kDirection;
+            continue;
+        }
+        const bool start = phase != kIterate;   // w = A u (A_ii u = r); else the recurrences
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             if (row[u] < 0) continue;
