@@ -324,8 +324,8 @@ int sp_profile_step(sp_sim* sim, sp_kernel_profile* out);
  * to other blocks' rows are gathered from global memory; it serves systems of
  * at most 2048 rows per SM and is not timed (ms 0) for larger ones; up to 768
  * rows per SM it runs as pipelined CG with one grid reduction per iteration.
- * A simulation for which no configuration was chosen takes the on-chip form
- * where it serves the system and configuration 0 beyond.
+ * A simulation for which no configuration was chosen takes that pipelined form
+ * up to 768 rows per SM and configuration 0 beyond.
  * Two configurations (matrix_free = 1) stream only the columns in the
  * iteration and recompute each pair weight w_ij = exp(-|R_ij|^2 / 2 lambda^2)
  * (arXiv 1808.06381, §Method) in FP32 from the positions in 32-bit fixed

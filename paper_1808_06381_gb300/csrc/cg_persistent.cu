@@ -2780,7 +2780,7 @@ PCfg g_pcfg[kPersistentConfigs] = {   // entry 0: the default without autotuning
     {4, 1, 0, 512, (const void*)k32_cg_persistent<4, 1, false, 512, true>, 0, 0, 1},
     {4, 3, 0, 256, (const void*)k32_cg_persistent<4, 3, false, 256, true>, 0, 0, 1},
 };
-constexpr int kResidentConfig = 9;    // the on-chip solve that a system without a chosen configuration takes
+constexpr int kResidentConfig = 9;    // the on-chip solve that a small system without a chosen configuration takes
 constexpr int kSmall32ChunkSmem = 7 * 1024;   // shared memory planned per chunk (28 entries a row)
 constexpr int kSmall32SpareSmem = 48 * 1024;
 constexpr int kSmall32MaxChunks = 24; // chunks of 32 rows per SM up to which the on-chip configurations run pipelined
@@ -2850,22 +2850,14 @@ p64::Shape small32_shape(const KParams& P, Launch L)
 
 // The configuration a launch uses: the chosen one, or entry 0 where the
 // chosen one is the on-chip solve and the system does not fit it.  Without a
-// choice (pcfg < 0): on chip where the system fits and the entries of a
-// uniform configuration of this density, half as many again for clustering,
-// fit beside the rows' records (else many chunks would be gathered from
-// memory, where the streaming form is the faster one).  Solve, streaming entry
-// 0 against on chip: n = 145,000 1.20 / 0.92 ms, n = 262,144 1.58 / 1.23, n =
-// 311,000 1.62 / 1.45; smaller systems at k32_cg_pipelined.
+// choice (pcfg < 0): the pipelined on-chip form where it serves the system
+// (figures there), else the streaming entry 0.  k32_cg_resident (n = 145,000: 0.92
+// ms, entry 0 1.20; n = 311,000 1.45 / 1.62) is taken where it was chosen: its
+// inner products use weights of 18 mantissa bits, entry 0's FP32 ones.
 const PCfg& cfg_of(const KParams& P, const DevBuffers& B, Launch L)
 {
     pocc_init();
-    if (P.pcfg < 0) {
-        const PCfg& r = g_pcfg[kResidentConfig];
-        if (small32_shape(P, L).u > 0) return r;
-        const double per_row = 4.18879 * P.rc2 * sqrt(P.rc2) * P.n / (P.L[0] * P.L[1] * P.L[2]);
-        const double rows = (double)P.n / (double)std::max<long long>(grid_of(r, P, L), 1);
-        return resident_fits(r, P, B, L) && rows * (16.0 + 4.0 * 1.5 * per_row) <= kResSmemBytes ? r : g_pcfg[0];
-    }
+    if (P.pcfg < 0) return g_pcfg[small32_shape(P, L).u > 0 ? kResidentConfig : 0];
     const int k = P.pcfg < kPersistentConfigs ? P.pcfg : 0;
     if (g_pcfg[k].resident && small32_shape(P, L).u == 0 && !resident_fits(g_pcfg[k], P, B, L)) return g_pcfg[0];
     return g_pcfg[k];
