@@ -159,6 +159,8 @@ def profiled_traffic(workload_name: str, tune, burn_in: int = 0) -> float | None
 
 def solver_kernel_name(tune) -> str:
     """Name of the persistent solver kernel a tile configuration launches."""
+    if tune and tune.get("automatic"):   # no configuration chosen: the pipelined form was the fastest
+        return "k32_cg_pipelined"
     if tune and tune.get("resident"):
         bt = tune["block_threads"]
         return f"k32_cg_resident<{bt},{2048 // bt}>"
@@ -476,7 +478,7 @@ def main():
         plan = plan_algorithmic_bytes(prof["n"], prof["cg_iterations"], "mixed")
         pach = plan / (prof["persistent_ms"] * 1e-3) / 1e9
         kname = solver_kernel_name(tune)
-        resident = bool(tune and tune.get("resident"))
+        resident = bool(tune and (tune.get("resident") or tune.get("automatic")))
         traffic = profiled_traffic(workload.name, tune, args.burn_in)
         persistent = {"kernel": kname, "bound": "latency" if resident else "hbm", "achieved": pach, "peak": peak,
                       "unit": "GB/s", "frac": pach / peak, "traffic": traffic,

@@ -322,10 +322,11 @@ int sp_profile_step(sp_sim* sim, sp_kernel_profile* out);
  * whole solve: their solver vectors in registers, their z = D^-1 r and the
  * matrix entries between two of them in shared memory, so that only entries
  * to other blocks' rows are gathered from global memory; it serves systems of
- * at most 2048 rows per SM and is not timed (ms 0) for larger ones; up to 768
- * rows per SM it runs as pipelined CG with one grid reduction per iteration.
- * A simulation for which no configuration was chosen takes that pipelined form
- * up to 768 rows per SM and configuration 0 beyond.
+ * at most 2048 rows per SM and is not timed (ms 0) for larger ones.
+ * A simulation for which no configuration was chosen runs pipelined CG on chip,
+ * one grid reduction per iteration, up to 768 rows per SM (it goes on with the
+ * other configurations' recurrence where the pipelined one drifts from the true
+ * residual), and configuration 0 beyond.
  * Two configurations (matrix_free = 1) stream only the columns in the
  * iteration and recompute each pair weight w_ij = exp(-|R_ij|^2 / 2 lambda^2)
  * (arXiv 1808.06381, §Method) in FP32 from the positions in 32-bit fixed
@@ -334,13 +335,15 @@ int sp_profile_step(sp_sim* sim, sp_kernel_profile* out);
  * sp_autotune builds the pair list
  * and the system for the current positions, times `trials` solves from a
  * zero start with every configuration on the simulation's stream, keeps the
- * fastest for this simulation, and leaves positions, step counter and the
+ * fastest for this simulation (automatic = 1: the pipelined form was faster than
+ * configuration `config`, the fastest of the table, and the simulation stays
+ * without one), and leaves positions, step counter and the
  * previous velocities (the warm start) unchanged.  With the environment
  * variable SHEARSIM_TUNE_CACHE naming a file, choices are looked up there
  * first, keyed by device name, SM count, n and the mean row length, and new
- * choices are appended (one line per key).  For SP_PREC_FP64, or with
+ * choices are appended.  For SP_PREC_FP64, or with
  * trials < 1, nothing is timed and the present choice is kept (reported as
- * configuration 0 where none was made).  Errors:
+ * configuration 0 with automatic = 1 where none was made).  Errors:
  * SP_ERR_INVALID_ARG (NULL sim), SP_ERR_CUDA, and those of the solve. */
 #define SP_TUNE_MAX_CONFIGS 12
 typedef struct sp_tune_info {
@@ -349,6 +352,8 @@ typedef struct sp_tune_info {
     int32_t blocks_per_sm;       /* its resident blocks per SM */
     int32_t from_cache;          /* 1: taken from the tuning cache, nothing timed */
     int32_t num_configs;         /* configurations available */
+    int32_t automatic;           /* 1: no configuration is chosen; `config` and the fields below describe the
+                                    fastest of the table (this field lies where the struct was padded) */
     double ms[SP_TUNE_MAX_CONFIGS]; /* best time of one solve per configuration (0: not timed) */
     int32_t pipelined;           /* 1: the next batch of columns is requested during the current gathers */
     int32_t block_threads;       /* threads per block (256 per window processed at once) */

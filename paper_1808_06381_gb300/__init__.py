@@ -83,7 +83,8 @@ class sp_vcorr_info(ctypes.Structure):
 
 class sp_tune_info(ctypes.Structure):
     _fields_ = [("config", ctypes.c_int32), ("gathers_in_flight", ctypes.c_int32), ("blocks_per_sm", ctypes.c_int32),
-                ("from_cache", ctypes.c_int32), ("num_configs", ctypes.c_int32), ("ms", ctypes.c_double * 12),
+                ("from_cache", ctypes.c_int32), ("num_configs", ctypes.c_int32), ("automatic", ctypes.c_int32),
+                ("ms", ctypes.c_double * 12),
                 ("pipelined", ctypes.c_int32), ("block_threads", ctypes.c_int32), ("resident", ctypes.c_int32),
                 ("matrix_free", ctypes.c_int32)]
 
@@ -393,7 +394,7 @@ class Simulation:
                 "blocks_per_sm": info.blocks_per_sm, "pipelined": bool(info.pipelined),
                 "block_threads": info.block_threads, "resident": bool(info.resident),
                 "matrix_free": bool(info.matrix_free),
-                "from_cache": bool(info.from_cache),
+                "from_cache": bool(info.from_cache), "automatic": bool(info.automatic),
                 "ms": [info.ms[k] for k in range(info.num_configs)]}
 
     # learned warm start

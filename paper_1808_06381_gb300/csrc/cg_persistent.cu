@@ -2780,10 +2780,9 @@ PCfg g_pcfg[kPersistentConfigs] = {   // entry 0: the default without autotuning
     {4, 1, 0, 512, (const void*)k32_cg_persistent<4, 1, false, 512, true>, 0, 0, 1},
     {4, 3, 0, 256, (const void*)k32_cg_persistent<4, 3, false, 256, true>, 0, 0, 1},
 };
-constexpr int kResidentConfig = 9;    // the on-chip solve that a small system without a chosen configuration takes
 constexpr int kSmall32ChunkSmem = 7 * 1024;   // shared memory planned per chunk (28 entries a row)
 constexpr int kSmall32SpareSmem = 48 * 1024;
-constexpr int kSmall32MaxChunks = 24; // chunks of 32 rows per SM up to which the on-chip configurations run pipelined
+constexpr int kSmall32MaxChunks = 24; // chunks of 32 rows per SM up to which a system without a chosen configuration runs pipelined
 struct BCfg {
     int kb, minb, bs;
     const void* fn;
@@ -2834,10 +2833,12 @@ bool resident_fits(const PCfg& c, const KParams& P, const DevBuffers& B, Launch 
     return g >= 1 && g <= L.num_sms && (P.nslots / 256 + g - 1) / g <= kResWindows;
 }
 
-// The on-chip form of small systems (k32_cg_pipelined): blocks, threads and
-// chunks a thread; u = 0 where the system is larger.
+// The pipelined form (k32_cg_pipelined), which small systems without a chosen
+// configuration take: blocks, threads and chunks a thread; u = 0 where a
+// configuration was chosen or the system is larger.
 p64::Shape small32_shape(const KParams& P, Launch L)
 {
+    if (P.pcfg >= 0) return p64::Shape{};
     const int nch = std::max(P.nchunks, 1), c = (nch + L.num_sms - 1) / L.num_sms;
     p64::Shape s{};
     if (c > kSmall32MaxChunks) return s;
@@ -2851,15 +2852,14 @@ p64::Shape small32_shape(const KParams& P, Launch L)
 // The configuration a launch uses: the chosen one, or entry 0 where the
 // chosen one is the on-chip solve and the system does not fit it.  Without a
 // choice (pcfg < 0): the pipelined on-chip form where it serves the system
-// (figures there), else the streaming entry 0.  k32_cg_resident (n = 145,000: 0.92
+// (small32_shape, asked first; figures there), else entry 0.  k32_cg_resident (n = 145,000: 0.92
 // ms, entry 0 1.20; n = 311,000 1.45 / 1.62) is taken where it was chosen: its
 // inner products use weights of 18 mantissa bits, entry 0's FP32 ones.
 const PCfg& cfg_of(const KParams& P, const DevBuffers& B, Launch L)
 {
     pocc_init();
-    if (P.pcfg < 0) return g_pcfg[small32_shape(P, L).u > 0 ? kResidentConfig : 0];
-    const int k = P.pcfg < kPersistentConfigs ? P.pcfg : 0;
-    if (g_pcfg[k].resident && small32_shape(P, L).u == 0 && !resident_fits(g_pcfg[k], P, B, L)) return g_pcfg[0];
+    const int k = P.pcfg >= 0 && P.pcfg < kPersistentConfigs ? P.pcfg : 0;
+    if (g_pcfg[k].resident && !resident_fits(g_pcfg[k], P, B, L)) return g_pcfg[0];
     return g_pcfg[k];
 }
 }  // namespace
@@ -2921,22 +2921,20 @@ bool cg_persistent_usable(int k, const KParams& P, const DevBuffers& B, Launch L
 {
     pocc_init();
     if (k < 0 || k >= kPersistentConfigs || g_pcfg[k].occ < 1) return false;
-    return !g_pcfg[k].resident || small32_shape(P, L).u > 0 || resident_fits(g_pcfg[k], P, B, L);
+    return !g_pcfg[k].resident || resident_fits(g_pcfg[k], P, B, L);
 }
+
+bool cg_persistent_pipelined(const KParams& P, Launch L) { return small32_shape(P, L).u > 0; }
 
 bool cg_persistent_on_chip(const KParams& P, const DevBuffers& B, Launch L)
 {
-    return cfg_of(P, B, L).resident != 0;
+    return small32_shape(P, L).u > 0 || cfg_of(P, B, L).resident != 0;
 }
 
 int cg_persistent_grid(const KParams& P, const DevBuffers& B, Launch L)
 {
-    const PCfg& c = cfg_of(P, B, L);
-    if (c.resident) {
-        const p64::Shape s = small32_shape(P, L);
-        if (s.u > 0) return s.blocks;
-    }
-    return (int)grid_of(c, P, L);
+    const p64::Shape s = small32_shape(P, L);
+    return s.u > 0 ? s.blocks : (int)grid_of(cfg_of(P, B, L), P, L);
 }
 
 // FP64 solve in one launch.  Systems of up to 16 chunks of 32 rows per SM
@@ -2985,7 +2983,7 @@ int cg64_persistent_grid(const KParams& P, Launch L) { return cg64_shape(P, L).b
 cudaError_t launch_cg32_persistent(const KParams& P, DevBuffers& B, Launch L)
 {
     const PCfg& c = cfg_of(P, B, L);
-    const p64::Shape small = c.resident ? small32_shape(P, L) : p64::Shape{};
+    const p64::Shape small = small32_shape(P, L);
     const int g = (int)grid_of(c, P, L);
     if (g < 1) return cudaErrorCooperativeLaunchTooLarge;
     if (c.mf) {

@@ -810,6 +810,8 @@ int cg_persistent_prelaunches(const KParams& P, const DevBuffers& B, Launch L);
 // The FP64 solver as one cooperative launch (r = b - A x0 with from_x, else x = 0).
 cudaError_t launch_cg64_persistent(const KParams& P, DevBuffers& B, int from_x, Launch L);
 int cg64_persistent_grid(const KParams& P, Launch L);
+// Whether this system, without a chosen configuration, takes the pipelined form of small systems.
+bool cg_persistent_pipelined(const KParams& P, Launch L);
 // Whether the persistent solve of this system runs on chip (and so can form
 // its initial residual itself: launch it with fused_init set and without
 // launch_cg_init, after launch_cg_split_x where it starts from x).

@@ -1,6 +1,7 @@
 // sp_autotune: choice of the persistent solver's tile configuration for one
 // simulation by timing (all configurations run the same iteration; only the
-// grouping of the dot products' partial sums, hence their rounding, differs).
+// grouping of the dot products' partial sums, hence their rounding, differs),
+// against the pipelined form that a small system takes without a choice.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -47,11 +48,13 @@ int cache_lookup(const std::string& path, const std::string& key)
     return found;
 }
 
-void cache_store(const std::string& path, const std::string& key, int cfg)
+// A second line, key|automatic, says whether the system's own form was faster
+// than the configuration (1) or not (0); a file without it holds configurations.
+void cache_store(const std::string& path, const std::string& key, int cfg, bool automatic)
 {
     std::lock_guard<std::mutex> lock(g_cache_mutex);
     std::ofstream f(path, std::ios::app);
-    if (f) f << key << ' ' << cfg << '\n';
+    if (f) f << key << ' ' << cfg << '\n' << key << "|automatic " << (automatic ? 1 : 0) << '\n';
 }
 
 }  // namespace
@@ -79,16 +82,17 @@ extern "C" int sp_autotune(sp_sim* s, int32_t trials, sp_tune_info* info)
     SS_TRY(set_device(s));
     sp_tune_info out{};
     out.num_configs = std::min(kPersistentConfigs, SP_TUNE_MAX_CONFIGS);
-    auto finish = [&](int cfg) {
-        s->kp.pcfg = cfg;
+    auto finish = [&](int cfg, bool automatic) {
+        s->kp.pcfg = automatic ? -1 : cfg;
         free_graphs(s);   // captured graphs hold the previous configuration's kernel
-        out.config = std::max(cfg, 0);   // no choice made (an FP64 simulation): entry 0
+        out.config = cfg;
+        out.automatic = automatic ? 1 : 0;
         cg_persistent_config(cfg, &out.gathers_in_flight, &out.blocks_per_sm, &out.pipelined, &out.block_threads,
                              &out.resident, &out.matrix_free);
         if (info) *info = out;
         return SP_OK;
     };
-    if (!mixed(s) || !s->persistent || trials < 1) return finish(s->kp.pcfg);
+    if (!mixed(s) || !s->persistent || trials < 1) return finish(std::max(s->kp.pcfg, 0), s->kp.pcfg < 0);
 
     // the system of the current positions (noise of the current step counter)
     SS_TRY(do_build(s));
@@ -104,7 +108,7 @@ extern "C" int sp_autotune(sp_sim* s, int32_t trials, sp_tune_info* info)
         const int cfg = cache_lookup(path, key);
         if (cfg >= 0) {
             out.from_cache = 1;
-            return finish(cfg);
+            return finish(cfg, cache_lookup(path, key + "|automatic") == 1);
         }
     }
 
@@ -118,11 +122,8 @@ extern "C" int sp_autotune(sp_sim* s, int32_t trials, sp_tune_info* info)
         cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
         rc = SP_ERR_CUDA;
     const int prev = s->kp.pcfg;
-    int best = prev;
-    double best_ms = 0.0;
-    for (int c = 0; rc == SP_OK && c < out.num_configs; ++c) {
-        if (!cg_persistent_usable(c, s->kp, s->B, launch_of(s, s->stream))) continue;   // ms[c] stays 0
-        s->kp.pcfg = c;
+    auto time_solves = [&](int pcfg) {   // the best of `trials` solves (ms), 0 where one failed
+        s->kp.pcfg = pcfg;
         double cmin = 0.0;
         for (int t = 0; rc == SP_OK && t <= trials; ++t) {   // the first solve warms up
             long long launches = 0;
@@ -136,11 +137,24 @@ extern "C" int sp_autotune(sp_sim* s, int32_t trials, sp_tune_info* info)
             cudaEventElapsedTime(&ms, e0, e1);
             if (rc == SP_OK && t > 0 && (cmin == 0.0 || ms < cmin)) cmin = ms;
         }
-        out.ms[c] = cmin;
-        if (rc == SP_OK && (best_ms == 0.0 || cmin < best_ms)) {
-            best_ms = cmin;
+        return rc == SP_OK ? cmin : 0.0;
+    };
+    int best = std::max(prev, 0);
+    double best_ms = 0.0;
+    for (int c = 0; rc == SP_OK && c < out.num_configs; ++c) {
+        if (!cg_persistent_usable(c, s->kp, s->B, launch_of(s, s->stream))) continue;   // ms[c] stays 0
+        const double ms = time_solves(c);
+        out.ms[c] = ms;
+        if (ms > 0.0 && (best_ms == 0.0 || ms < best_ms)) {
+            best_ms = ms;
             best = c;
         }
+    }
+    s->kp.pcfg = -1;
+    bool automatic = false;
+    if (rc == SP_OK && cg_persistent_pipelined(s->kp, launch_of(s, s->stream))) {
+        const double ms = time_solves(-1);
+        automatic = ms > 0.0 && (best_ms == 0.0 || ms < best_ms);
     }
     if (cudaMemcpyAsync(s->B.v_s, v_save, vbytes, cudaMemcpyDeviceToDevice, s->stream) != cudaSuccess ||
         cudaStreamSynchronize(s->stream) != cudaSuccess)
@@ -154,6 +168,6 @@ extern "C" int sp_autotune(sp_sim* s, int32_t trials, sp_tune_info* info)
         if (s->err.empty()) s->err = "autotuning solve failed";
         return rc;
     }
-    if (path && *path) cache_store(path, key, best);
-    return finish(best);
+    if (path && *path) cache_store(path, key, best, automatic);
+    return finish(best, automatic);
 }

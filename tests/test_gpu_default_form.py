@@ -26,3 +26,51 @@ def test_beyond_the_pipelined_form_the_default_streams(n, monkeypatch):
     info = sim.solve_velocities()
     assert info["status"] == 0 and info["offchip_blocks"] > 0, info
     sim.close()
+
+
+def _sim(n, seed=5):
+    L = synth.box_length(n)
+    pos = synth.uniform_positions(n, (L,) * 3, seed)
+    sim = ss.Simulation(n, (L,) * 3, ss.kappa_from_kappa_tau(0.5), seed=seed, precision="mixed", warm_start="none",
+                        cg_tol=1e-8, positions=pos)
+    sim.set_positions(pos, 0.3 * L)
+    return sim
+
+
+@pytest.mark.parametrize("n", [777, 20011, 100000])
+@pytest.mark.parametrize("config,threads", [(8, 1024), (9, 512)])
+def test_a_chosen_on_chip_configuration_runs_at_every_size(n, config, threads):
+    """Configurations 8 and 9 are k32_cg_resident for small systems too: its blocks are one per 256-row
+    window and 256 threads (at most one per SM), the pipelined form's one per 32 n / SMs rows."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    sim = _sim(n)
+    info = sim.set_solver_config(config)
+    assert info["resident"] and info["block_threads"] == threads
+    windows, groups = (n + 255) // 256, threads // 256
+    blocks = min(sms, (windows + groups - 1) // groups)
+    chunks = -(-n // 32)
+    assert blocks != -(-chunks // -(-chunks // sms))   # what the pipelined form would take
+    assert sim.profile_step()["persistent_blocks"] == blocks
+    sim.close()
+
+
+def test_autotune_reports_the_form_that_runs(tmp_path, monkeypatch):
+    """Where the pipelined form is the fastest the simulation stays without a configuration: one block
+    per 160 rows at n = 20,011, where the configurations run one per 256 rows or more.  A cached choice
+    takes the same form, and one that was made without the second line keeps its configuration."""
+    n = 20011
+    cache = tmp_path / "tune.txt"
+    monkeypatch.setenv("SHEARSIM_TUNE_CACHE", str(cache))
+    for cached in (False, True):
+        sim = _sim(n)
+        info = sim.autotune(trials=2)
+        assert info["from_cache"] == cached
+        assert info["automatic"] == (sim.profile_step()["persistent_blocks"] > n // 256 + 1)
+        sim.close()
+    cache.write_text("".join(line for line in cache.read_text().splitlines(True) if "|automatic" not in line))
+    sim = _sim(n)
+    again = sim.autotune(trials=1)
+    assert again["from_cache"] and not again["automatic"] and again["config"] == info["config"]
+    assert sim.profile_step()["persistent_blocks"] <= n // 256 + 1
+    sim.close()
