@@ -2993,7 +2993,7 @@ cudaError_t launch_cg32_persistent(const KParams& P, DevBuffers& B, Launch L)
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)g);
     cfg.blockDim = dim3((unsigned)c.bs);
-    int smem = std::min(std::max(P.res_smem, 0), kResSmemBytes);
+    int smem = std::min(std::max(P.res_smem, kResMinSmem), kResSmemBytes);
     cfg.dynamicSmemBytes = c.resident ? smem : 0;
     const void* fn = c.fn;
     if (small.u > 0) {

@@ -57,7 +57,7 @@ struct KParams {
     float hly_hi, hly_lo;       // L_y / 2
     float akl_hi, akl_lo;       // alpha kappa L_y
     int pcfg;           // tile configuration of the persistent solver (index, autotuned; -1: chosen by the system)
-    int res_smem;       // shared memory the on-chip solve uses (<= kResSmemBytes; less only to test its fallback)
+    int res_smem;       // shared memory the on-chip solve uses (kResMinSmem .. kResSmemBytes; less only to test its fallback)
     int fused_init;     // on-chip solve: 0 after the initial-residual kernel; 1 forms r = b itself (x0 = 0), 2 r = b - A x0
     long long hcopy;    // on-chip solve: where hcol / hval / hlo hold a second copy region (the lists of blocks
                         // whose entries all stay off chip, at their sliced positions + hcopy); 0: none, and the
@@ -72,6 +72,7 @@ struct KParams {
 
 constexpr int kPersistentConfigs = 12;
 constexpr int kResSmemBytes = 190 * 1024;   // on-chip solve: dynamic shared memory per block
+constexpr int kResMinSmem = 2048 * 16;       // what it needs in any case: a 16-byte record of each of a block's rows
 constexpr int kResLoStride = 49152;          // >= kResSmemBytes / 4: local entries of one block
 
 // Scalars that live on the device so that a whole step runs without the host.

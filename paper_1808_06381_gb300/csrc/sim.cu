@@ -737,7 +737,7 @@ int sp_sim_create(const sp_params* p, const double* pos_host, sp_sim** out)
     // a smaller shared-memory budget for the on-chip solve (its entries then
     // fit on fewer SMs): only to exercise the fallback of blocks that do not fit
     if (const char* rsm = std::getenv("SHEARSIM_RESIDENT_SMEM"))
-        s->kp.res_smem = std::min(std::max(std::atoi(rsm), 0), kResSmemBytes);
+        s->kp.res_smem = std::min(std::max(std::atoi(rsm), kResMinSmem), kResSmemBytes);
     DevBuffers& B = s->B;
     const size_t v3 = 3 * (size_t)npad;
     int a = SP_OK;

@@ -74,3 +74,18 @@ def test_autotune_reports_the_form_that_runs(tmp_path, monkeypatch):
     assert again["from_cache"] and not again["automatic"] and again["config"] == info["config"]
     assert sim.profile_step()["persistent_blocks"] <= n // 256 + 1
     sim.close()
+
+
+@pytest.mark.parametrize("budget", ["0", "12288", "-1"])
+@pytest.mark.parametrize("config", [8, 9])
+def test_the_smallest_shared_memory_budget_holds_the_rows_records(config, budget, monkeypatch):
+    """A budget below the rows' records (16 bytes each of up to 2048 rows) is raised to them: entries
+    are gathered from memory, and the solve meets its tolerance."""
+    monkeypatch.setenv("SHEARSIM_RESIDENT_SMEM", budget)
+    sim = _sim(150000)
+    sim.set_solver_config(config)
+    sim.build_neighbors()
+    sim.assemble()
+    info = sim.solve_velocities()
+    assert info["status"] == 0 and info["residual"] <= 1e-8 and info["offchip_blocks"] > 0, info
+    sim.close()
