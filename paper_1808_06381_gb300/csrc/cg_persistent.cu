@@ -2961,7 +2961,7 @@ cudaError_t launch_cg64_persistent(const KParams& P, DevBuffers& B, int from_x, 
 {
     Shape64 s = cg64_shape(P, L);
     if (s.smem > 32 * 1024) {   // with the static arrays, near the 48 KB a kernel has by default
-        const cudaError_t e = cudaFuncSetAttribute(s.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, s.smem);
+        const cudaError_t e = allow_shared_memory(s.fn, p64::kMaxSmem);
         if (e != cudaSuccess) return e;
     }
     cudaLaunchConfig_t cfg = {};
@@ -3003,7 +3003,7 @@ cudaError_t launch_cg32_persistent(const KParams& P, DevBuffers& B, Launch L)
         cfg.blockDim = dim3((unsigned)small.threads);
         cfg.dynamicSmemBytes = (size_t)smem;
         if (smem > 32 * 1024) {
-            const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            const cudaError_t e = allow_shared_memory(fn, p64::kMaxSmem);
             if (e != cudaSuccess) return e;
         }
     }

@@ -324,7 +324,7 @@ cudaError_t cheb_coeffs(const unsigned long long* bound, int degree, double* cs,
 {
     const int N = degree + 1, smem = (int)sizeof(double) * (2 * N + 1);   // 64 KB at the largest degree
     if (smem > 40 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k_cheb_coeffs, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        const cudaError_t e = allow_shared_memory(k_cheb_coeffs, (int)sizeof(double) * (2 * 4097 + 1));   // degree <= 4096
         if (e != cudaSuccess) return e;
     }
     k_cheb_coeffs<<<(N + 127) / 128, 128, smem, s>>>(bound, degree, cs, csf);

@@ -878,6 +878,16 @@ void launch_reset_step_stats(DevState* st, cudaStream_t s);
 // Architecture of the device code the current device runs (cudaFuncGetAttributes
 // of one of this library's kernels): 10 major + minor, e.g. 103 for sm_103.
 cudaError_t device_code_version(int* binary_version, int* ptx_version);
+
+// Allows a kernel dynamic shared memory beyond the default.  The limit belongs to
+// the kernel, not to the launch, and every simulation and host thread shares it:
+// `bytes` is the kernel's ceiling over all systems, never a launch's own size (a
+// smaller system would lower the limit under another thread's launch).
+template <class F>
+inline cudaError_t allow_shared_memory(F* kernel, int bytes)
+{
+    return cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
 // sfactor.cu: S(q) at q_z = 0 for kx in [-nkx, nkx], ky in [-nky, nky] (kx slowest);
 // G = 0: direct sum over particles; G > 0: CIC grid of G x G in the sheared frame.
 // A_dev: (nkx + 1) G complex values, then max(nkx, nky) + 1 doubles.

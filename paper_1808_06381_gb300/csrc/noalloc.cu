@@ -375,7 +375,7 @@ extern "C" int sp_solve_csr_noalloc(int32_t device, void* stream, int64_t n, con
     // the state (and the grid barriers' counters) must start at zero on every call
     if (cudaMemsetAsync(st, 0, sizeof(NaState), s) != cudaSuccess) return finish(SP_ERR_CUDA, "cudaMemsetAsync");
     if (sp.smem > 32 * 1024 &&   // with the static arrays, near the 48 KB a kernel has by default
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, sp.smem) != cudaSuccess)
+        allow_shared_memory(fn, p64::kMaxSmem) != cudaSuccess)
         return finish(SP_ERR_CUDA, "cudaFuncSetAttribute");
     unsigned long long limit_ns = kDefaultWaitLimitNs;
     cudaLaunchConfig_t cfg = {};

@@ -227,9 +227,9 @@ cudaError_t run_structure_factor(const KParams& P, const DevBuffers& B, double d
     const size_t sx = tab + hf;                                    // at most 192 KB (G = 8,192)
     const int tw_shared = tab + 2 * hf <= 200 * 1024 ? 1 : 0;      // G above ~6,400: the table through L1
     const size_t sy = 2 * hf + (tw_shared ? tab : 0);
-    if (tab + 2 * hf > 32 * 1024 &&
-        (cudaFuncSetAttribute(k_sq_dft_x, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sx) != cudaSuccess ||
-         cudaFuncSetAttribute(k_sq_dft_y, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sy) != cudaSuccess))
+    constexpr int kMaxSmem = 200 * 1024;   // sx and sy at every G
+    if (tab + 2 * hf > 32 * 1024 && (allow_shared_memory(k_sq_dft_x, kMaxSmem) != cudaSuccess ||
+                                     allow_shared_memory(k_sq_dft_y, kMaxSmem) != cudaSuccess))
         return cudaGetLastError();
     k_sq_dft_x<<<G + extra, 256, sx, s>>>(grid_dev, G, nkx, kmax, tw, A_dev, win);
     k_sq_dft_y<<<dim3(nkx + 1, nky / kSqKy + 1), kSqKy * kSqSplit, sy, s>>>(A_dev, G, nkx, nky, tw, win, P, delta, S_dev,
