@@ -337,7 +337,8 @@ int sp_profile_step(sp_sim* sim, sp_kernel_profile* out);
  * zero start with every configuration on the simulation's stream, keeps the
  * fastest for this simulation (automatic = 1: the pipelined form was faster than
  * configuration `config`, the fastest of the table, and the simulation stays
- * without one), and leaves positions, step counter and the
+ * without one; a configuration whose solve fails is not a candidate, and the
+ * error is returned where all fail), and leaves positions, step counter and the
  * previous velocities (the warm start) unchanged.  With the environment
  * variable SHEARSIM_TUNE_CACHE naming a file, choices are looked up there
  * first, keyed by device name, SM count, n and the mean row length, and new

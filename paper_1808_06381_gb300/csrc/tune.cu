@@ -122,6 +122,7 @@ extern "C" int sp_autotune(sp_sim* s, int32_t trials, sp_tune_info* info)
         cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
         rc = SP_ERR_CUDA;
     const int prev = s->kp.pcfg;
+    int failed = SP_OK;   // the status of the last solve that failed: its configuration is no candidate
     auto time_solves = [&](int pcfg) {   // the best of `trials` solves (ms), 0 where one failed
         s->kp.pcfg = pcfg;
         double cmin = 0.0;
@@ -132,7 +133,11 @@ extern "C" int sp_autotune(sp_sim* s, int32_t trials, sp_tune_info* info)
             cudaEventRecord(e1, s->stream);
             if (rc == SP_OK && cudaEventSynchronize(e1) != cudaSuccess) rc = SP_ERR_CUDA;
             if (rc == SP_OK) rc = read_state(s);
-            if (rc == SP_OK && s->st_host->error) rc = s->st_host->error;
+            if (rc == SP_OK && s->st_host->error) {
+                failed = s->st_host->error;
+                rc = clear_flags(s);
+                return 0.0;
+            }
             float ms = 0.f;
             cudaEventElapsedTime(&ms, e0, e1);
             if (rc == SP_OK && t > 0 && (cmin == 0.0 || ms < cmin)) cmin = ms;
@@ -156,6 +161,7 @@ extern "C" int sp_autotune(sp_sim* s, int32_t trials, sp_tune_info* info)
         const double ms = time_solves(-1);
         automatic = ms > 0.0 && (best_ms == 0.0 || ms < best_ms);
     }
+    if (rc == SP_OK && best_ms == 0.0 && !automatic) rc = failed;   // no configuration solved the system
     if (cudaMemcpyAsync(s->B.v_s, v_save, vbytes, cudaMemcpyDeviceToDevice, s->stream) != cudaSuccess ||
         cudaStreamSynchronize(s->stream) != cudaSuccess)
         rc = rc == SP_OK ? SP_ERR_CUDA : rc;

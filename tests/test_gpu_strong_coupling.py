@@ -68,3 +68,38 @@ def test_solve_converges_at_strong_coupling(precision, alpha, n):
     slack = (1e-12 if precision == "mixed" else 1e-15) * 2 * np.linalg.norm(sys.diag[:, None] * v) / np.linalg.norm(sys.b)
     res = np.linalg.norm(sys.b - sys.matvec(v)) / np.linalg.norm(sys.b)
     assert res <= 1e-8 + slack, (res, slack)
+
+
+def test_autotune_leaves_out_configurations_that_do_not_converge():
+    """At alpha = 1,000 the pipelined form and the streaming one need different numbers of iterations: with
+    a limit between the two, tuning keeps the one that converges; with one below both it returns
+    their error and leaves the simulation as it was."""
+    n, alpha = 20011, 1000.0
+    L, pos, _ = _system(n, alpha)
+
+    def sim_of(limit):
+        sim = ss.Simulation(n, (L,) * 3, ss.kappa_from_kappa_tau(0.5), alpha=alpha, seed=3, precision="mixed",
+                            warm_start="none", cg_tol=1e-8, cg_max_iter=limit, positions=pos)
+        sim.set_positions(pos, 0.3 * L)
+        sim.build_neighbors()
+        sim.assemble()
+        return sim
+
+    sim = sim_of(1000)
+    own = sim.solve_velocities()["iterations"]
+    sim.set_solver_config(0)
+    streaming = sim.solve_velocities()["iterations"]
+    sim.close()
+    assert abs(own - streaming) > 10   # else the limit below separates nothing
+    sim = sim_of((own + streaming) // 2)
+    info = sim.autotune(trials=1)
+    assert (info["ms"][0] > 0) == (streaming < own) and (own > streaming or info["automatic"]), info
+    assert sim.solve_velocities()["status"] == 0
+    sim.close()
+    sim = sim_of(20)
+    with pytest.raises(ss.ShearsimError) as e:
+        sim.autotune(trials=1)
+    assert e.value.code == ss.SP_ERR_NOT_CONVERGED
+    sim.set_positions(pos, 0.3 * L)   # the simulation stays usable
+    assert sim.num_pairs() > 0
+    sim.close()
