@@ -36,7 +36,7 @@ struct PShared {
     float2 df[32];
     double d[32];
     float2 dfk[2][32];   // per-warp sums of the grid reductions
-    double dk[4][32];
+    double dk[3][32];
     double bcast[4];
     float bcastf[2];     // the same totals rounded to FP32 (the on-chip iteration's scalars)
     int flag;
@@ -46,7 +46,6 @@ struct PShared {
     int action;   // 0 continue, 1 replace the residual, 2 stop
     // thread 0's CG state, kept here rather than in every thread's registers
     double rho, rr_restart, bnorm2, last_res;
-    double alpha_d, beta_d;   // the pipelined FP64 solve's scalars (its reductions overwrite bcast)
     float rho_f, target_f;   // on-chip iteration: rho and its stopping target in FP32
     int iter, restarts, status;
 };
