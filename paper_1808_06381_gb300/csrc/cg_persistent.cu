@@ -262,7 +262,7 @@ __device__ __forceinline__ bool grid_allreduce(DevState* st, unsigned int& gen, 
                                                const double (&v)[K], double* partials, double (&out)[K],
                                                int bid, int nb)
 {
-    static_assert(K <= 4, "four values at most");
+    static_assert(K <= 3, "three values at most");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double w[K];
 #pragma unroll
