@@ -125,7 +125,9 @@ double sp_kappa_from_kappa_tau(double kappa_tau, double rc, double zeta, double 
 /* Create a simulation on p->device.  pos_host: [n][3] initial positions in
  * [0, L) (copied), or NULL for positions uniform in the box drawn from the
  * counter-based generator keyed by p->seed.  The Lees-Edwards offset starts at
- * 0 and the step counter at 0.  On success *out owns all device memory. */
+ * 0 and the step counter at 0.  On success *out owns all device memory: about
+ * 1.7 KB per particle (mixed) or 1.3 KB (FP64) at the paper's density with its
+ * pair lists, 480 bytes of it the pair candidates (96 partners a row). */
 int sp_sim_create(const sp_params* p, const double* pos_host, sp_sim** out);
 
 /* Free everything; NULL is allowed. */
@@ -220,7 +222,10 @@ int sp_stress_xy(sp_sim* sim, double* sigma_xy);
  * (host).  lambda_max (may be NULL) receives the interval's upper end; when it
  * is 1 (no coupling) xi = g.  One sliced-layout SpMV per degree (FP64 for the
  * FP64 path, double-float on the FP32 pipes for the mixed path); steps_ms (may be NULL)
- * receives their time (CUDA events on the simulation's stream).  Errors:
+ * receives their time (CUDA events on the simulation's stream).  The first call
+ * allocates five vectors (160 bytes per particle mixed, 120 FP64), which the
+ * simulation keeps for the next call and for sp_set_fdt_noise until it is
+ * destroyed or sp_set_fdt_noise(sim, 0) gives them back.  Errors:
  * SP_ERR_INVALID_ARG (NULL pointer, degree outside [1, 4096], no assembled
  * system), SP_ERR_OOM, SP_ERR_CUDA. */
 int sp_sqrt_apply(sp_sim* sim, int32_t degree, const double* g_host, double* xi_host, double* lambda_max,
@@ -230,7 +235,8 @@ int sp_sqrt_apply(sp_sim* sim, int32_t degree, const double* g_host, double* xi_
  * sp_step_host replaces the independent normals g in its right-hand side by
  * xi = p(A) g as sp_sqrt_apply forms it (on the device, inside the step's
  * graph): b += (noise amplitude / zeta) (xi - g) after the assembly.  degree =
- * 0 restores the paper's independent noise (the default).  Costs one SpMV
+ * 0 restores the paper's independent noise (the default) and gives the vectors
+ * back.  Costs one SpMV
  * per degree per step.  Batched steps (sp_batch_step) keep the independent
  * noise.  Errors: SP_ERR_INVALID_ARG (degree outside [0, 4096]),
  * SP_ERR_OOM. */

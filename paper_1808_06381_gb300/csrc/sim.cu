@@ -1636,6 +1636,7 @@ int sp_set_fdt_noise(sp_sim* s, int32_t degree)
     }
     s->fdt_degree = degree;
     free_graphs(s);   // the step graph is captured again with (or without) the noise pass
+    if (degree == 0) fdt_free(s->fdt);   // no step uses it; sp_sqrt_apply allocates it again
     return SP_OK;
 }
 
