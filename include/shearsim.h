@@ -200,7 +200,8 @@ int64_t sp_state_record_bytes(void);
  * x' = x - (delta/L_y) y by cloud-in-cell (z summed), transformed, and the CIC
  * window divided out; |kx|, |ky| must stay below grid / 4 (aliasing grows
  * towards the mesh's Nyquist limit).  grid = 0: exact direct sum over the
- * particles for every mode (cost n x modes). */
+ * particles for every mode (cost n x modes).  Work arrays of up to 64 MB (grid
+ * 2048) stay with the simulation for the next call; larger ones are freed. */
 int sp_structure_factor(sp_sim* sim, int32_t nkx, int32_t nky, int32_t grid, double* S_host,
                         double* qx_host, double* qy_host);
 

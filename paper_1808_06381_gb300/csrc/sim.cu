@@ -81,6 +81,8 @@ void fdt_free(FdtBuffers& V)
     V = FdtBuffers{};
 }
 
+constexpr size_t kSqKeepBytes = 64ull << 20;   // the structure factor's arrays that a simulation keeps (G = 2,048: 34 MB)
+
 void sq_free(SqBuffers& Q)
 {
     void* ptrs[] = {Q.out, Q.tw, Q.grid, Q.A};
@@ -1720,10 +1722,15 @@ int sp_structure_factor(sp_sim* s, int32_t nkx, int32_t nky, int32_t grid, doubl
     const double delta = s->st_host->delta;
     const size_t m = (size_t)(2 * nkx + 1) * (2 * nky + 1);
     SqBuffers& Q = s->sq;
-    SS_TRY(sq_grow(s, &Q.out, &Q.out_cap, 3 * m));
+    int grown = sq_grow(s, &Q.out, &Q.out_cap, 3 * m);
+    if (grown == SP_OK && grid > 0) grown = sq_grow(s, &Q.grid, &Q.grid_cap, (size_t)grid * grid);
+    if (grown == SP_OK && grid > 0)   // A, and the windows behind it
+        grown = sq_grow(s, &Q.A, &Q.A_cap, (size_t)(nkx + 1) * grid + std::max(nkx, nky) / 2 + 1);
+    if (grown != SP_OK) {
+        sq_free(Q);
+        return grown;
+    }
     if (grid > 0) {
-        SS_TRY(sq_grow(s, &Q.grid, &Q.grid_cap, (size_t)grid * grid));
-        SS_TRY(sq_grow(s, &Q.A, &Q.A_cap, (size_t)(nkx + 1) * grid + std::max(nkx, nky) / 2 + 1));   // and the windows
         if (Q.G != grid) {
             // twiddle table (cos, sin)(2 pi m / G), m = 0..G-1
             cudaFree(Q.tw);
@@ -1753,6 +1760,8 @@ int sp_structure_factor(sp_sim* s, int32_t nkx, int32_t nky, int32_t grid, doubl
             rc = SP_ERR_CUDA;
     }
     if (rc == SP_ERR_CUDA && s->err.empty()) s->err = std::string("structure factor: ") + cudaGetErrorString(cudaGetLastError());
+    // large work arrays are not held for a later call (their allocation is a small part of such a call)
+    if (sizeof(double) * (Q.out_cap + Q.grid_cap + 2 * Q.A_cap) > kSqKeepBytes) sq_free(Q);
     return rc;
 }
 
