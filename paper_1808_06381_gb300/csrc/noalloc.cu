@@ -33,6 +33,7 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <cstdlib>
 #include <cstring>
 #include <mutex>
 #include <string>
@@ -364,7 +365,11 @@ extern "C" int sp_solve_csr_noalloc(int32_t device, void* stream, int64_t n, con
     int num_sms = 1;
     if (cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
         return finish(SP_ERR_CUDA, "cudaDeviceGetAttribute");
+    // fewer SMs than the device has: only to exercise the forms that a device of few SMs (a part of a
+    // GB300 given out as an instance of its own) takes, four and sixteen chunks a thread
+    if (const char* few = std::getenv("SHEARSIM_NOALLOC_SMS")) num_sms = std::max(1, std::min(num_sms, std::atoi(few)));
     p64::Shape sp = p64::shape_of((int)((n + 31) / 32), std::min(num_sms, kNaMaxBlocks), 16);
+    // sixteen chunks a thread keep part of their vectors in local memory
     const void* fn = sp.u == 1 ? (const void*)k_na_solve<1, 12>
                                : (sp.u == 2 ? (const void*)k_na_solve<2, 8>
                                             : (sp.u == 4 ? (const void*)k_na_solve<4, 6> : (const void*)k_na_solve<16, 4>));
