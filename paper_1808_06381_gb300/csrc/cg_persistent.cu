@@ -2339,8 +2339,8 @@ __global__ void __launch_bounds__(p64::max_threads(U), 1) k64_cg_pipelined(KPara
 // step at n = 20,011).
 // Measured (whole solve of a clustered
 // system to 1e-8; streaming form / k32_cg_resident / this one): n = 500 0.52 /
-// 0.33 / 0.19 ms, n = 20,011 1.02 / 0.75 / 0.38, n = 48,000 1.03 / 0.69 / 0.43,
-// n = 72,960 1.12 / 0.80 / 0.54, n = 100,000 1.13 / 0.84 / 0.79, n = 145,000
+// 0.33 / 0.23 ms, n = 20,011 1.02 / 0.75 / 0.39, n = 48,000 1.03 / 0.69 / 0.44,
+// n = 72,960 1.12 / 0.80 / 0.56, n = 100,000 1.13 / 0.84 / 0.79, n = 145,000
 // 1.20 / 0.92 / 1.04 (there its gathers, which k32_cg_resident serves from
 // shared memory).
 template <int KB, class Sys>
